@@ -129,6 +129,43 @@ __device__ __forceinline__ bool all_opaque(const float* T)
     return bits == 0u;
 }
 
+// Exact early termination.  With B >= |S| of every record of the batch and B >=
+// |i_bc|, whatever a ray still adds to a wavelength is at most T B (1 + 2^-21) per
+// segment.  Where T B 2^26 <= I that is below a quarter of the spacing of floats
+// at I, so every later update, and the boundary term, rounds back to I: the rest
+// of the ray cannot change a bit of it.  A ray is done when this holds for all of
+// its wavelengths, near tau = 18 where exact underflow of T takes 87 to 104.
+// stop = B 2^26, or negative where no bound is known (then T = 0 everywhere).
+__device__ __forceinline__ float stop_factor(float bound, float i_bc)
+{
+    const float f = fmaxf(bound, fabsf(i_bc)) * 67108864.0f;  // 2^26
+    return bound >= 0.0f && f <= 3.402823466e38f ? f : -1.0f;
+}
+
+// The larger of two bounds, or -1 (none known) if either is.
+__device__ __forceinline__ float join_bounds(float a, float b) { return fminf(a, b) < 0.0f ? -1.0f : fmaxf(a, b); }
+
+// Bound of one wavelength's record, or -1 unless S is finite and chi finite and not negative.
+__device__ __forceinline__ float bound_of(float S, float chi)
+{
+    const float a = fabsf(S);
+    return a <= 3.402823466e38f && chi >= 0.0f && chi <= 3.402823466e38f ? a : -1.0f;
+}
+
+template <int W>
+__device__ __forceinline__ bool ray_done(const float* I, const float* T, float stop)
+{
+    if (stop < 0.0f) return all_opaque<W>(T);
+    float m = 0.0f;
+#pragma unroll
+    for (int w = 0; w + 1 < W; w += 2) {
+        const float2 d = __ffma2_rn(make_float2(T[w], T[w + 1]), make_float2(stop, stop), make_float2(-I[w], -I[w + 1]));
+        m = fmaxf(m, fmaxf(d.x, d.y));
+    }
+    if constexpr (W % 2 == 1) m = fmaxf(m, fmaf(T[W - 1], stop, -I[W - 1]));
+    return !(m > 0.0f);
+}
+
 // All W wavelengths of a record: pairs on the packed pipe, an odd one alone.
 template <int W>
 __device__ __forceinline__ void segments(const float* S, const float* chi, float nl2, float* I, float* T)

@@ -12,6 +12,7 @@ namespace dex {
 struct DenseParams {
     int nx, nz, n_lambda, W, n_batch;
     int exclude_own;        // leave out each probe's own-cell emission (the first segment)
+    int scanned;            // J holds the bound of the exact early termination (launch_solve_dense)
     long long n_cells;
     const float* planes;
     int n_probe;

@@ -1,0 +1,76 @@
+"""Exact early termination and split directions: the bits of the full walk.
+
+A counting solve walks every ray until its transmissions are exactly zero (the
+plain solver: to the grid's edge) and one warp takes all directions of a probe.
+The solves that users time stop rays as soon as the rest cannot change a bit of
+I, and share a probe's directions between warps on small grids.  Both must give
+the same J and I, bit for bit, so every comparison here is for equality.
+"""
+
+import numpy as np
+import pytest
+import torch
+
+import synth
+
+pytestmark = pytest.mark.gpu
+
+
+def ctx_():
+    from paper_2511_08498_gb300 import api
+    return api.Context(0)
+
+
+def thick_medium(nx, nz, L, seed, emitters=False, log_chi=(-3.0, 2.5)):
+    """Random medium whose rays die after 1 to 100 cells, with empty cells (and blocks)."""
+    m = synth.random_medium(nx, nz, L, seed=synth.SEED_BASE + seed, log_chi_range=log_chi,
+                            emitter_frac=0.02 if emitters else 0.0)
+    e, c = m["eta"].copy(), m["chi"].copy()
+    e[:, -(nz // 4):], c[:, -(nz // 4):] = 0.0, 0.0
+    return torch.from_numpy(e.reshape(L, -1)).cuda(), torch.from_numpy(c.reshape(L, -1)).cuda()
+
+
+def same(a, b):
+    assert (a is None) == (b is None)
+    assert a is None or torch.equal(a, b)
+
+
+@pytest.mark.parametrize("nx,nz,L,W", [(33, 17, 1, 1), (64, 64, 3, 2), (31, 70, 9, 4), (97, 65, 20, 8)])
+@pytest.mark.parametrize("i_bc,emitters", [(0.0, False), (0.7, True)])
+def test_plain(nx, nz, L, W, i_bc, emitters):
+    from paper_2511_08498_gb300 import api
+    ctx = ctx_()
+    eta, chi = thick_medium(nx, nz, L, 800 + W, emitters)
+    planes = api.pack_planes(ctx, eta, chi, W)
+    dirs, w = synth.directions(12, offset=0.0)  # axis-parallel and corner rays among them
+    for own in (True, False):
+        ctx.set_own_cell(own)
+        full = api.formal_solve_dense(ctx, nx, nz, L, W, planes, dirs, w, i_bc=i_bc, want_intensity=True,
+                                      count_segments=True)
+        fast = api.formal_solve_dense(ctx, nx, nz, L, W, planes, dirs, w, i_bc=i_bc, want_intensity=True)
+        same(full[0], fast[0])
+        same(full[1], fast[1])
+    ctx.set_own_cell(True)
+    # enough probes for one warp per 32 of them and all directions (unsplit)
+    probes = torch.arange(nx * nz, dtype=torch.int32, device="cuda").repeat(-(-312000 // (nx * nz)))
+    J, _, _ = api.formal_solve_dense(ctx, nx, nz, L, W, planes, dirs, w, probes=probes, i_bc=i_bc)
+    ref, _, _ = api.formal_solve_dense(ctx, nx, nz, L, W, planes, dirs, w, i_bc=i_bc)
+    same(J, ref[:, probes.long()])
+    ctx.check()
+
+
+@pytest.mark.parametrize("bad", [float("inf"), float("nan"), -1.0])
+def test_plain_records_without_a_bound(bad):
+    """Hand-made records with a non-finite source function or a negative opacity: no early end.
+    Opacities near 1 per cell keep every transmission above zero, as in the counting walk."""
+    from paper_2511_08498_gb300 import api
+    ctx = ctx_()
+    nx, nz, L, W = 40, 24, 8, 8
+    eta, chi = thick_medium(nx, nz, L, 811, log_chi=(-0.2, 0.1))
+    planes = api.pack_planes(ctx, eta, chi, W)
+    planes[0, 500, 3 if bad != -1.0 else 8 + 3] = bad * (1e-3 if bad == -1.0 else 1.0)
+    dirs, w = synth.directions(8)
+    full = api.formal_solve_dense(ctx, nx, nz, L, W, planes, dirs, w, want_intensity=True, count_segments=True)
+    fast = api.formal_solve_dense(ctx, nx, nz, L, W, planes, dirs, w, want_intensity=True)
+    for a, b in zip(full[:2], fast[:2]):
+        assert np.array_equal(a.cpu().numpy(), b.cpu().numpy(), equal_nan=True)
