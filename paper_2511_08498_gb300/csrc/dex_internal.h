@@ -46,6 +46,14 @@ constexpr int kInfoMaxBlocks = 8192;
 // hold 160 KB).
 constexpr int kPairInfoMaxBlocks = 16384;
 
+// Static solves whose one CTA per (block, batch) would be less than two full loads
+// of the chip (152 SMs x 4) split the directions over the warps of eight CTAs per
+// block instead: the slowest CTA's directions in series set the time there.  256 x
+// 192, 20 wavelengths, 32 directions, bfloat16 (576 CTAs): 2.97 -> 1.97 ms; 144 x
+// 160, 21 wavelengths, paired (270): 0.85 -> 0.33 ms; but 784 x 288, 29 wavelengths
+// (3528): 5.07 -> 5.52 ms, and the 1024^2 paired solve 101 -> 115 ms.
+constexpr long long kSplitCtas = 1216;
+
 // Distance thresholds of levels 1..4 padded to four, as the traversal compares
 // them (the number of thresholds band[m-1] <= t is the highest level allowed):
 // +inf for the levels beyond the n_band given (never reached), 0 for all four
@@ -114,6 +122,8 @@ struct HddaParams {
                      // (band padded to four by pad_bands)
     int traversal;   // DEX_TRAVERSAL_PER_BATCH, _SHARED or _PAIRED (static model, W = 8)
     int exclude_own; // leave out each probe's own-voxel emission (static model, W = 8, float32)
+    int scanned;     // J holds the bounds of the exact early termination (scan.cuh)
+    int split_at;    // float offset of the split kernels' intensities in dynamic shared memory
     float band[4];
     long long n_cells;
     const float* bricks;
@@ -128,6 +138,11 @@ struct HddaParams {
     unsigned int* status;
     Quadrature quad;
 };
+
+inline bool split_directions(const HddaParams& P)
+{
+    return !P.seg_count && (long long)P.cap_active * P.n_batch < kSplitCtas && P.split_at <= 24576;  // table <= 96 KB
+}
 
 struct AtomParams {
     dex_atom atom;

@@ -15,6 +15,7 @@ struct Geo {
     int x_lo, x_hi, z_lo, z_hi;  // cell faces bounding the non-empty blocks
     const float* batch_base;     // bricks of the wavelength batch being solved
     float band[4];               // distance thresholds, padded (pad_bands)
+    float stop;                  // stop_factor of the early termination
 };
 
 // Rays end where they leave this box: beyond it every block is empty and adds
@@ -138,18 +139,43 @@ struct PairRecModel {
         return v;
     }
     __device__ __forceinline__ static void integrate(const Params&, const Voxel& v, int, float, float, float nl2,
-                                                     float* I, float* T)
+                                                     float* I, float* T, float)
     {
         segments<8>(v.a.S, v.a.chi, nl2, I, T);
         segments<8>(v.b.S, v.b.chi, nl2, I + 8, T + 8);
     }
 };
 
+// Steps the traversal loop is unrolled: models with few instructions per step
+// four (twice and eight times measured slower on the 1024^2 benchmark solve, for
+// the single- and the two-batch model); models that declare kUnroll that many.
+template <class M, class = void>
+struct UnrollOf {
+    static constexpr int value = 4;
+};
+template <class M>
+struct UnrollOf<M, decltype((void)M::kUnroll)> {
+    static constexpr int value = M::kUnroll;
+};
+
+// Model::stage(M): shared-memory tables of a model, filled by the CTA before its
+// first barrier (models that declare it).
+template <class Model>
+__device__ __forceinline__ auto model_stage(const typename Model::Params& M, int) -> decltype(Model::stage(M))
+{
+    Model::stage(M);
+}
+template <class Model>
+__device__ __forceinline__ void model_stage(const typename Model::Params&, long)
+{
+}
+
 // Voxel models: Model::kStride floats per voxel record, Model::kPerBatch whether
 // records differ per wavelength batch, Model::kEarlyLoad whether the record is
 // loaded at the top of each step, Model::kZeroNoop whether a record of zeros
 // integrates to no change, Model::Voxel / load / integrate the per-segment
-// update of the W wavelengths of batch b along propagation (wx, wz).
+// update of the W wavelengths of batch b along propagation (wx, wz); its last
+// argument is the early termination's factor, for models that skip wavelengths.
 //
 // One ray from the centre of cell (i, j) (in active block a0 = (bx0, bz0), whose
 // level is mip0) along d = (dx, dz): accumulates I and T (initialised by the
@@ -194,10 +220,9 @@ __device__ __forceinline__ void trace_ray(const Geo& G, const typename Model::Pa
     // the step left the block: look up the next one and re-initialise the tracer
     // there (false: the ray ends)
     auto enter = [&](bool on_x, float th) -> bool {
-        // early termination: once every transmission has underflowed to exactly
-        // zero the rest of the ray adds exact zeros, so stopping leaves I and T
-        // bit-identical
-        if (all_opaque<W>(T)) return false;
+        // early termination: the rest of the ray changes no bit of I (1024^2 paired
+        // benchmark solve: 165 -> 105 ms, J bit-identical)
+        if (ray_done<W>(I, T, G.stop)) return false;
         if (on_x) bxc += sx;
         else bzc += sz;
         if ((unsigned)bxc >= (unsigned)G.nbx || (unsigned)bzc >= (unsigned)G.nbz) {
@@ -243,9 +268,8 @@ __device__ __forceinline__ void trace_ray(const Geo& G, const typename Model::Pa
     };
     typename Model::Voxel cur;
 
-    // unrolled four times (twice and eight times measured slower on the 1024^2
-    // benchmark solve, for the single- and the two-batch model)
-#pragma unroll 4
+    constexpr int kUnroll = UnrollOf<Model>::value;
+#pragma unroll kUnroll
     for (int it = 0;; ++it) {
         // models with kEarlyLoad issue the current voxel's record before the
         // stepping and crossing bookkeeping, which then hides its latency
@@ -284,7 +308,7 @@ __device__ __forceinline__ void trace_ray(const Geo& G, const typename Model::Pa
         // integrate the voxel left (in empty blocks: the zero record, or nothing)
         if (kZero || cur_mip >= 0) {
             if constexpr (!Model::kEarlyLoad) cur = model_load<Model>(M, cur_rp);
-            Model::integrate(M, cur, b, -dx, -dz, len * kNegLog2e, I, T);
+            Model::integrate(M, cur, b, -dx, -dz, len * kNegLog2e, I, T, G.stop);
             if constexpr (EXT) {
                 if (it == 0) {
 #pragma unroll
@@ -294,6 +318,9 @@ __device__ __forceinline__ void trace_ray(const Geo& G, const typename Model::Pa
             if (COUNT) nseg += (cur_mip >= 0) & (th > th_prev);
         }
         if (last) break;
+        // within blocks the termination test runs every fourth step: in thick cells
+        // rays end long before the next block face
+        if ((it & 3) == 3 && ray_done<W>(I, T, G.stop)) break;
         th_prev = th;
         tl_prev = tl;
         if constexpr (kZero) {
@@ -302,15 +329,60 @@ __device__ __forceinline__ void trace_ray(const Geo& G, const typename Model::Pa
     }
 }
 
+// Directions shared by the warps of a CTA (SPLIT kernels): the warps take the
+// directions of one 8 x 4 tile from a counter, kSplitChunk at a time, and leave
+// their intensities in shared memory; then the CTA adds them to J in the order
+// of the directions, the bits of the unsplit sum.  s_I [kSplitChunk][W][32],
+// after the block table in dynamic shared memory.
+template <int W>
+constexpr int split_chunk() { return W > 8 ? 16 : 32; }
+template <int W>
+constexpr size_t split_bytes() { return sizeof(float) * split_chunk<W>() * W * 32; }
+
+template <int W, int NW, class Ray, class Store>
+__device__ __forceinline__ void split_solve(const Quadrature& quad, float* s_I, int* s_next, int warp, int lane,
+                                            Ray ray, Store store)
+{
+    constexpr int KD = split_chunk<W>(), kPer = (W + NW - 1) / NW;
+    float J[kPer];  // wavelengths warp, warp + NW, ... of the lane's probe
+#pragma unroll
+    for (int q = 0; q < kPer; ++q) J[q] = 0.0f;
+    for (int k0 = 0; k0 < quad.n_dir; k0 += KD) {
+        if (threadIdx.x == 0) *s_next = 0;
+        __syncthreads();
+        for (;;) {
+            int g = 0;
+            if (lane == 0) g = atomicAdd(s_next, 1);
+            g = __shfl_sync(0xffffffffu, g, 0);
+            if (g >= KD || k0 + g >= quad.n_dir) break;
+            ray(k0 + g, s_I + g * (W * 32) + lane);
+        }
+        __syncthreads();
+#pragma unroll
+        for (int q = 0; q < kPer; ++q) {
+            const int w = warp + q * NW;
+            if (w < W)
+                for (int g = 0; g < KD && k0 + g < quad.n_dir; ++g)
+                    J[q] = fmaf(quad.w[k0 + g], s_I[(g * W + w) * 32 + lane], J[q]);
+        }
+    }
+#pragma unroll
+    for (int q = 0; q < kPer; ++q)
+        if (warp + q * NW < W) store(warp + q * NW, J[q]);
+}
+
 // kInfo: the CTA stages one word per block (offset * 8 + state, InfoLookup;
 // dynamic shared memory 4 * nbx * nbz bytes, grids of at most kInfoMaxBlocks
 // blocks); otherwise the packed state words (WordLookup; 8 * n_words bytes).
-template <int W, bool COUNT, class Model, bool kInfo = false, bool EXT = false>
+// SPLIT: eight CTAs per block, one per 8 x 4 tile, whose warps share the tile's
+// directions (split_solve; s_I at P.split_at floats of the dynamic shared
+// memory); otherwise one CTA per block, one warp per tile.
+template <int W, bool COUNT, class Model, bool kInfo = false, bool EXT = false, bool SPLIT = false>
 __global__ void __launch_bounds__(256, Model::kMinBlocks) k_solve_hdda_t(const HddaParams P, const typename Model::Params M)
 {
     extern __shared__ unsigned long long s_dyn[];
-    __shared__ float s_J[W][256];
-    const int a0 = blockIdx.x;
+    __shared__ float s_J[SPLIT ? 1 : W][256];
+    const int a0 = SPLIT ? blockIdx.x >> 3 : blockIdx.x;
     if (a0 >= *P.n_active) return;
     const int b = blockIdx.y;
     const int tid = threadIdx.x;
@@ -322,8 +394,11 @@ __global__ void __launch_bounds__(256, Model::kMinBlocks) k_solve_hdda_t(const H
     } else {
         for (int q = tid; q < P.n_words; q += blockDim.x) s_dyn[q] = words_b[q];
     }
+    if constexpr (!SPLIT) {
 #pragma unroll
-    for (int w = 0; w < W; ++w) s_J[w][tid] = 0.0f;
+        for (int w = 0; w < W; ++w) s_J[w][tid] = 0.0f;
+    }
+    model_stage<Model>(M, 0);
     // box around the non-empty (active) blocks, in block units
     __shared__ int s_box[4];
     if (tid < 4) s_box[tid] = (tid & 1) ? -1 : 0x7fffffff;
@@ -357,9 +432,9 @@ __global__ void __launch_bounds__(256, Model::kMinBlocks) k_solve_hdda_t(const H
     // warp w covers an 8 x 4 tile of the block (lanes along x, then z): a warp's rays
     // meet x faces in at most 8 different iterations (16 with whole 16-cell rows),
     // while its record loads stay within the block's brick
-    const int wrp = tid >> 5;
-    const int i = bx0 * DEX_BLOCK + (wrp & 1) * 8 + (tid & 7);
-    const int j = bz0 * DEX_BLOCK + (wrp >> 1) * 4 + ((tid & 31) >> 3);
+    const int wrp = tid >> 5, lane = tid & 31, tile = SPLIT ? (int)(blockIdx.x & 7) : wrp;
+    const int i = bx0 * DEX_BLOCK + (tile & 1) * 8 + (lane & 7);
+    const int j = bz0 * DEX_BLOCK + (tile >> 1) * 4 + (lane >> 3);
     const int state0 = (kInfo ? (s_info[blk0] & 7) : block_state(s_dyn, blk0)) - 1;
     if (state0 < 0) {  // state words do not describe this active block
         raise_status(P.status, DEX_ERR_TRAVERSAL_CAP);
@@ -379,35 +454,58 @@ __global__ void __launch_bounds__(256, Model::kMinBlocks) k_solve_hdda_t(const H
     G.z_hi = (s_box[3] + 1) * DEX_BLOCK;
 #pragma unroll
     for (int q = 0; q < 4; ++q) G.band[q] = P.band[q];
+    G.stop = !COUNT && P.scanned ? stop_factor(P.J[(size_t)(b * W) * P.n_cells + (size_t)j * P.nx + i], P.i_bc) : -1.0f;
     const int mip0 = min(state0, distance_cap(G, 0.0f));
     unsigned int nseg = 0;
     bool capped = false;
 
-    for (int k = 0; k < P.quad.n_dir; ++k) {
-        const float dx = P.quad.dx[k], dz = P.quad.dz[k];
-        float I[W], T[W];
+    auto ray = [&](int k, float* I, float* T) {
 #pragma unroll
         for (int w = 0; w < W; ++w) { I[w] = 0.0f; T[w] = 1.0f; }
         if constexpr (kInfo)
-            trace_ray<W, COUNT, Model, InfoLookup, EXT>(G, M, b, i, j, bx0, bz0, a0, mip0, dx, dz,
+            trace_ray<W, COUNT, Model, InfoLookup, EXT>(G, M, b, i, j, bx0, bz0, a0, mip0, P.quad.dx[k], P.quad.dz[k],
                                                         InfoLookup{s_info}, I, T, nseg, capped);
         else
-            trace_ray<W, COUNT, Model, WordLookup, EXT>(G, M, b, i, j, bx0, bz0, a0, mip0, dx, dz,
+            trace_ray<W, COUNT, Model, WordLookup, EXT>(G, M, b, i, j, bx0, bz0, a0, mip0, P.quad.dx[k], P.quad.dz[k],
                                                         WordLookup{s_dyn, P.block_offset}, I, T, nseg, capped);
-        const float wk = P.quad.w[k];
+    };
+    const size_t cell = (size_t)j * P.nx + i;
+    if constexpr (SPLIT) {
+        __shared__ int s_next;
+        split_solve<W, 8>(
+            P.quad, reinterpret_cast<float*>(s_dyn) + P.split_at, &s_next, wrp, lane,
+            [&](int k, float* out) {
+                float I[W], T[W];
+                ray(k, I, T);
+#pragma unroll
+                for (int w = 0; w < W; ++w) {
+                    const float Iw = fmaf(T[w], P.i_bc, I[w]);
+                    out[w * 32] = Iw;
+                    const int l = b * W + w;
+                    if (P.I != nullptr && l < P.n_lambda) P.I[((size_t)l * P.quad.n_dir + k) * P.n_cells + cell] = Iw;
+                }
+            },
+            [&](int w, float J) {
+                if (b * W + w < P.n_lambda) P.J[(size_t)(b * W + w) * P.n_cells + cell] = J;
+            });
+    } else {
+        for (int k = 0; k < P.quad.n_dir; ++k) {
+            float I[W], T[W];
+            ray(k, I, T);
+            const float wk = P.quad.w[k];
+#pragma unroll
+            for (int w = 0; w < W; ++w) {
+                const float Iw = fmaf(T[w], P.i_bc, I[w]);
+                s_J[w][tid] = fmaf(wk, Iw, s_J[w][tid]);
+                const int l = b * W + w;
+                if (P.I != nullptr && l < P.n_lambda) P.I[((size_t)l * P.quad.n_dir + k) * P.n_cells + cell] = Iw;
+            }
+        }
 #pragma unroll
         for (int w = 0; w < W; ++w) {
-            const float Iw = fmaf(T[w], P.i_bc, I[w]);
-            s_J[w][tid] = fmaf(wk, Iw, s_J[w][tid]);
             const int l = b * W + w;
-            if (P.I != nullptr && l < P.n_lambda)
-                P.I[((size_t)l * P.quad.n_dir + k) * P.n_cells + (size_t)j * P.nx + i] = Iw;
+            if (l < P.n_lambda) P.J[(size_t)l * P.n_cells + cell] = s_J[w][tid];
         }
-    }
-#pragma unroll
-    for (int w = 0; w < W; ++w) {
-        const int l = b * W + w;
-        if (l < P.n_lambda) P.J[(size_t)l * P.n_cells + (size_t)j * P.nx + i] = s_J[w][tid];
     }
     if (capped) raise_status(P.status, DEX_ERR_TRAVERSAL_CAP);
     if (COUNT && P.seg_count != nullptr) atomicAdd(P.seg_count, (unsigned long long)nseg);

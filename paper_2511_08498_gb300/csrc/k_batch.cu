@@ -9,7 +9,7 @@
 // one atmosphere batch wide.  Per-atmosphere completion times (globaltimer, ns)
 // are recorded when requested.
 
-#include "hdda.cuh"
+#include "scan.cuh"
 
 namespace dex {
 
@@ -44,7 +44,7 @@ struct StaticRec {
         return BrickFmt<W, kStoreF32>::load(p, coff);
     }
     __device__ __forceinline__ static void integrate(const Params&, const Voxel& v, int, float, float, float nl2,
-                                                     float* I, float* T)
+                                                     float* I, float* T, float)
     {
         segments<W>(v.S, v.chi, nl2, I, T);
     }
@@ -152,6 +152,12 @@ __global__ void __launch_bounds__(NT, kMinCtas) k_batch_solve(const BatchParams 
             set_box_full(G);
 #pragma unroll
             for (int q = 0; q < 4; ++q) G.band[q] = A.band[q];
+            // the batch's bound (k_scan_batch) waits where this thread's first J will go
+            const size_t cell = (size_t)j * A.nx + i;
+            const size_t plane = (size_t)W * A.nx * A.nz;
+            float bound = A.J[b1 * plane + cell];
+            if (kPair && b2 >= 0) bound = join_bounds(bound, A.J[b2 * plane + cell]);
+            G.stop = stop_factor(bound, A.i_bc);
             const int mip0 = min(state0, distance_cap(G, 0.0f));
             typename StaticRec<W>::Params M{};
             for (int k = 0; k < A.n_dir; ++k) {
@@ -197,6 +203,57 @@ __global__ void __launch_bounds__(NT, kMinCtas) k_batch_solve(const BatchParams 
     if (capped) raise_status(P.status, DEX_ERR_TRAVERSAL_CAP);
 }
 
+// Bounds of the early termination, as k_scan_bricks and k_spread_bounds for every
+// atmosphere (blockIdx.z) and wavelength batch (blockIdx.y).
+template <int W>
+__global__ void __launch_bounds__(128) k_scan_batch(const BatchParams P)
+{
+    const AtmDesc& A = P.atm[blockIdx.z];
+    const int b = blockIdx.y;
+    if (b * W >= A.n_lambda || blockIdx.x >= A.cap_active) return;
+    const int na = *A.n_active;
+    float* J = A.J + (size_t)(b * W) * A.nx * A.nz;
+    for (int a = blockIdx.x; a < na; a += gridDim.x) {
+        const float m = join_cta(chain_bound<W, kStoreF32>(A.bricks + ((size_t)b * A.cap_active + a) * A.chain * (2 * W), A.chain));
+        const int blk = A.active[a];
+        if (threadIdx.x == 0) J[(size_t)(blk / A.nbx * DEX_BLOCK) * A.nx + blk % A.nbx * DEX_BLOCK] = m;
+    }
+}
+
+template <int W>
+__global__ void __launch_bounds__(256) k_spread_batch(const BatchParams P)
+{
+    const AtmDesc& A = P.atm[blockIdx.z];
+    const int b = blockIdx.y;
+    if (b * W >= A.n_lambda || blockIdx.x >= A.cap_active) return;
+    const int na = *A.n_active;
+    float* J = A.J + (size_t)(b * W) * A.nx * A.nz;
+    float m = 0.0f;
+    for (int a = threadIdx.x; a < na; a += blockDim.x) {
+        const int blk = A.active[a];
+        m = join_bounds(m, __ldcg(J + (size_t)(blk / A.nbx * DEX_BLOCK) * A.nx + blk % A.nbx * DEX_BLOCK));
+    }
+    m = join_cta(m);
+    for (int a = blockIdx.x; a < na; a += gridDim.x) {
+        const int blk = A.active[a];
+        J[(size_t)(blk / A.nbx * DEX_BLOCK + (threadIdx.x >> 4)) * A.nx + blk % A.nbx * DEX_BLOCK + (threadIdx.x & 15)] = m;
+    }
+}
+
+template <int W>
+void scan_batch(cudaStream_t s, const BatchParams& P)
+{
+    int cap = 1, n_batch = 1;
+    for (int a = 0; a < P.n_atm; ++a) {
+        cap = max(cap, P.atm[a].cap_active);
+        n_batch = max(n_batch, (P.atm[a].n_lambda + W - 1) / W);
+    }
+    const dim3 scan((unsigned)min(cap, 608), (unsigned)n_batch, (unsigned)P.n_atm);
+    const dim3 spread((unsigned)min(cap, 76), (unsigned)n_batch, (unsigned)P.n_atm);
+    k_scan_batch<W><<<scan, 128, 0, s>>>(P);
+    k_spread_batch<W><<<spread, 256, 0, s>>>(P);
+}
+
 template <int W, int NT, bool kInfo, int kMinCtas, bool kPair = false>
 cudaError_t launch_batch_t(cudaStream_t s, const BatchParams& P, int ctas, size_t smem)
 {
@@ -213,12 +270,12 @@ template <int W, bool kOcc>
 cudaError_t launch_batch_w(cudaStream_t s, const BatchParams& P, int ctas, int packet, bool info, size_t smem)
 {
     switch (packet * 2 + (info ? 1 : 0)) {
-        case 256 * 2: return launch_batch_t<W, 256, false, kOcc ? 4 : 1>(s, P, ctas, smem);
-        case 256 * 2 + 1: return launch_batch_t<W, 256, true, kOcc ? 4 : 1>(s, P, ctas, smem);
-        case 128 * 2: return launch_batch_t<W, 128, false, kOcc ? 8 : 1>(s, P, ctas, smem);
-        case 128 * 2 + 1: return launch_batch_t<W, 128, true, kOcc ? 8 : 1>(s, P, ctas, smem);
-        case 64 * 2: return launch_batch_t<W, 64, false, kOcc ? 16 : 1>(s, P, ctas, smem);
-        case 64 * 2 + 1: return launch_batch_t<W, 64, true, kOcc ? 16 : 1>(s, P, ctas, smem);
+        case 256 * 2: return launch_batch_t<W, 256, false, kOcc ? 4 : 3>(s, P, ctas, smem);
+        case 256 * 2 + 1: return launch_batch_t<W, 256, true, kOcc ? 4 : 3>(s, P, ctas, smem);
+        case 128 * 2: return launch_batch_t<W, 128, false, kOcc ? 8 : 6>(s, P, ctas, smem);
+        case 128 * 2 + 1: return launch_batch_t<W, 128, true, kOcc ? 8 : 6>(s, P, ctas, smem);
+        case 64 * 2: return launch_batch_t<W, 64, false, kOcc ? 16 : 12>(s, P, ctas, smem);
+        case 64 * 2 + 1: return launch_batch_t<W, 64, true, kOcc ? 16 : 12>(s, P, ctas, smem);
         default: return cudaErrorInvalidValue;
     }
 }
@@ -245,6 +302,13 @@ cudaError_t launch_batch_solve(cudaStream_t s, const BatchParams& P, int ctas, i
     cudaError_t e = cudaMemsetAsync(P.queue, 0, sizeof(unsigned int), s);
     if (e != cudaSuccess || P.n_items == 0) return e;
     if (occupancy && W != 8) return cudaErrorInvalidValue;
+    switch (W) {
+        case 1: scan_batch<1>(s, P); break;
+        case 2: scan_batch<2>(s, P); break;
+        case 4: scan_batch<4>(s, P); break;
+        case 8: scan_batch<8>(s, P); break;
+        default: return cudaErrorInvalidValue;
+    }
     if (P.paired) {
         // pairs of batches (W = 8): one word per block staged, the compiler's budget
         // bounded at 128 registers (two 256-thread CTAs per SM)

@@ -75,7 +75,7 @@ struct CavMlpModel {
         return v;
     }
     __device__ __forceinline__ static void integrate(const Params& M, const Voxel& v, int b, float wx, float wz,
-                                                     float nl2, float* I, float* T)
+                                                     float nl2, float* I, float* T, float)
     {
         const float proj = fmaf(v.p[4], wx, v.p[5] * wz);
         const float inv = v.p[3];
@@ -114,7 +114,7 @@ struct CavModel {
         return v;
     }
     __device__ __forceinline__ static void integrate(const Params& M, const Voxel& v, int b, float wx, float wz,
-                                                     float nl2, float* I, float* T)
+                                                     float nl2, float* I, float* T, float)
     {
         const float proj = fmaf(v.p[4], wx, v.p[5] * wz);
         // not unrolled: eight inlined copies of the four-branch Voigt evaluation made

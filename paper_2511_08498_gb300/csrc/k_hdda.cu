@@ -23,7 +23,7 @@
 // ends where it leaves the box around the non-empty blocks (nothing beyond it
 // adds to I or T); a ray that would step out of the grid before that sets
 // DEX_ERR_TRAVERSAL_CAP.
-#include "hdda.cuh"
+#include "scan.cuh"
 
 namespace dex {
 
@@ -52,7 +52,7 @@ struct StaticModel {
         return BrickFmt<W, ST>::load(p, coff);
     }
     __device__ __forceinline__ static void integrate(const Params&, const Voxel& v, int, float, float, float nl2,
-                                                     float* I, float* T)
+                                                     float* I, float* T, float)
     {
         segments<W>(v.S, v.chi, nl2, I, T);
     }
@@ -61,7 +61,7 @@ struct StaticModel {
 template <typename K, typename MP>
 cudaError_t launch_hdda_kernel(K kernel, dim3 grid, size_t smem, cudaStream_t s, const HddaParams& P, const MP& M)
 {
-    if (smem > 32 * 1024) {
+    if (smem > 24 * 1024) {
         cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         if (e != cudaSuccess) return e;
     }
@@ -71,9 +71,34 @@ cudaError_t launch_hdda_kernel(K kernel, dim3 grid, size_t smem, cudaStream_t s,
 
 }  // namespace
 
-cudaError_t launch_solve_hdda(cudaStream_t s, const HddaParams& P)
+// Bounds of the exact early termination for the static solves (not for counting
+// ones, whose segment counts run to exactly zero transmission).
+static void scan_bricks(cudaStream_t s, HddaParams& P)
 {
-    if (P.cap_active == 0 || P.n_batch == 0) return cudaSuccess;
+    const dim3 grid((unsigned)P.cap_active, (unsigned)P.n_batch);
+    switch (P.W * 4 + P.storage) {
+#define DEX_SCAN(WW, ST) \
+    case WW * 4 + ST: k_scan_bricks<WW, ST><<<grid, 128, 0, s>>>(P); break;
+        DEX_SCAN(1, kStoreF32)
+        DEX_SCAN(2, kStoreF32)
+        DEX_SCAN(4, kStoreF32)
+        DEX_SCAN(8, kStoreF32)
+        DEX_SCAN(4, kStoreBF16)
+        DEX_SCAN(8, kStoreBF16)
+        DEX_SCAN(4, kStoreF16)
+        DEX_SCAN(8, kStoreF16)
+#undef DEX_SCAN
+        default: return;
+    }
+    launch_spread(s, P);
+    P.scanned = 1;
+}
+
+cudaError_t launch_solve_hdda(cudaStream_t s, const HddaParams& P0)
+{
+    if (P0.cap_active == 0 || P0.n_batch == 0) return cudaSuccess;
+    HddaParams P = P0;
+    if (!P.scanned && !P.seg_count && !solve_hdda_shared_applies(P)) scan_bricks(s, P);
     if (P.traversal == DEX_TRAVERSAL_PAIRED) {
         if (!solve_hdda_paired_applies(P)) return cudaErrorNotSupported;
         return launch_solve_hdda_paired(s, P);
@@ -99,28 +124,26 @@ cudaError_t launch_solve_hdda(cudaStream_t s, const HddaParams& P)
     // block (InfoLookup); otherwise the packed state words (WordLookup)
     const long long n_blocks = (long long)P.nbx * P.nbz;
     const bool info = P.W == 8 && n_blocks <= kInfoMaxBlocks;
-    const size_t smem = info ? sizeof(int) * (size_t)n_blocks : sizeof(unsigned long long) * (size_t)P.n_words;
-    dim3 grid((unsigned)P.cap_active, (unsigned)P.n_batch);
+    P.split_at = (int)(((info ? n_blocks : 2LL * P.n_words) + 3) & ~3LL);
+    const bool split = split_directions(P);
+    const size_t smem = sizeof(float) * ((size_t)P.split_at + (split ? (size_t)split_chunk<8>() * P.W * 32 : 0));
+    const dim3 grid((unsigned)P.cap_active * (split ? 8u : 1u), (unsigned)P.n_batch);
     cudaError_t e = cudaSuccess;
     switch (P.W * 4 + P.storage) {
-#define MP_(WW, ST) typename StaticModel<WW, ST>::Params{}
-#define DEX_LAUNCH(WW, ST)                                                                                   \
-    case WW * 4 + ST:                                                                                        \
-        if (P.seg_count)                                                                                     \
-            e = launch_hdda_kernel(k_solve_hdda_t<WW, true, StaticModel<WW, ST>>, grid, smem, s, P, MP_(WW, ST));   \
-        else                                                                                                 \
-            e = launch_hdda_kernel(k_solve_hdda_t<WW, false, StaticModel<WW, ST>>, grid, smem, s, P, MP_(WW, ST));  \
-        break;
-#define DEX_LAUNCH_INFO(ST)                                                                                  \
-    case 8 * 4 + ST:                                                                                         \
-        if (info && P.seg_count)                                                                             \
-            e = launch_hdda_kernel(k_solve_hdda_t<8, true, StaticModel<8, ST>, true>, grid, smem, s, P, MP_(8, ST));  \
-        else if (info)                                                                                       \
-            e = launch_hdda_kernel(k_solve_hdda_t<8, false, StaticModel<8, ST>, true>, grid, smem, s, P, MP_(8, ST)); \
-        else if (P.seg_count)                                                                                \
-            e = launch_hdda_kernel(k_solve_hdda_t<8, true, StaticModel<8, ST>>, grid, smem, s, P, MP_(8, ST));     \
-        else                                                                                                 \
-            e = launch_hdda_kernel(k_solve_hdda_t<8, false, StaticModel<8, ST>>, grid, smem, s, P, MP_(8, ST));    \
+#define DEX_LAUNCH_(WW, ST, INFO)                                                                                     \
+    {                                                                                                                 \
+        using M_ = StaticModel<WW, ST>;                                                                               \
+        if (P.seg_count) e = launch_hdda_kernel(k_solve_hdda_t<WW, true, M_, INFO>, grid, smem, s, P, M_::Params{});  \
+        else if (split)                                                                                               \
+            e = launch_hdda_kernel(k_solve_hdda_t<WW, false, M_, INFO, false, true>, grid, smem, s, P, M_::Params{}); \
+        else e = launch_hdda_kernel(k_solve_hdda_t<WW, false, M_, INFO>, grid, smem, s, P, M_::Params{});             \
+    }
+#define DEX_LAUNCH(WW, ST) \
+    case WW * 4 + ST: DEX_LAUNCH_(WW, ST, false) break;
+#define DEX_LAUNCH_INFO(ST)                  \
+    case 8 * 4 + ST:                         \
+        if (info) DEX_LAUNCH_(8, ST, true)   \
+        else DEX_LAUNCH_(8, ST, false)       \
         break;
         DEX_LAUNCH(1, kStoreF32)
         DEX_LAUNCH(2, kStoreF32)
@@ -132,7 +155,7 @@ cudaError_t launch_solve_hdda(cudaStream_t s, const HddaParams& P)
         DEX_LAUNCH_INFO(kStoreF16)
 #undef DEX_LAUNCH_INFO
 #undef DEX_LAUNCH
-#undef MP_
+#undef DEX_LAUNCH_
         default: return cudaErrorInvalidValue;
     }
     if (e != cudaSuccess) return e;

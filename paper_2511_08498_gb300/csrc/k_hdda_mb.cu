@@ -293,6 +293,7 @@ __global__ void __launch_bounds__(256, 2) k_solve_hdda_mb(const HddaParams P)
     }
     constexpr int REC = RecFmt<8, ST>::kStride;
     Geo G;
+    G.stop = -1.0f;
     G.nx = P.nx;
     G.nz = P.nz;
     G.nbx = P.nbx;

@@ -59,13 +59,14 @@ using PairModel = PairRecModel<ST, pair_min_blocks<ST>()>;
 
 // EXT: each probe's own-voxel emission is left out (the first segment of every
 // ray, as k_solve_hdda_t with EXT).
-template <int ST, bool COUNT, bool EXT>
+// SPLIT: a CTA's warps share the directions of one 8 x 4 tile (split_solve).
+template <int ST, bool COUNT, bool EXT, bool SPLIT>
 __global__ void __launch_bounds__(pair_threads<ST>(), pair_min_blocks<ST>()) k_solve_hdda_pair(const HddaParams P)
 {
     using Model = PairModel<ST>;
-    constexpr int kParts = pair_parts<ST>();
+    constexpr int kParts = SPLIT ? 8 : pair_parts<ST>(), NW = pair_threads<ST>() / 32;
     extern __shared__ int s_info[];
-    __shared__ float s_J[16][pair_threads<ST>()];
+    __shared__ float s_J[SPLIT ? 1 : 16][pair_threads<ST>()];
     __shared__ int s_box[4];
     const int a0 = blockIdx.x / kParts, part = blockIdx.x - a0 * kParts;
     if (a0 >= *P.n_active) return;
@@ -77,8 +78,10 @@ __global__ void __launch_bounds__(pair_threads<ST>(), pair_min_blocks<ST>()) k_s
     const int n_blocks = P.nbx * P.nbz;
     for (int q = tid; q < n_blocks; q += blockDim.x)
         s_info[q] = pack_block_info(P.block_offset[q], min(block_state(w1, q), block_state(w2, q)));
+    if constexpr (!SPLIT) {
 #pragma unroll
-    for (int w = 0; w < 16; ++w) s_J[w][tid] = 0.0f;
+        for (int w = 0; w < 16; ++w) s_J[w][tid] = 0.0f;
+    }
     if (tid < 4) s_box[tid] = (tid & 1) ? -1 : 0x7fffffff;
     __syncthreads();
     {
@@ -110,9 +113,10 @@ __global__ void __launch_bounds__(pair_threads<ST>(), pair_min_blocks<ST>()) k_s
     const int bx0 = blk0 % P.nbx, bz0 = blk0 / P.nbx;
     // the CTA's probes: rows part * (16 / kParts) .. of the block; warp w covers an
     // 8 x 4 tile of them (as in k_solve_hdda_t)
-    const int wrp = tid >> 5;
-    const int i = bx0 * DEX_BLOCK + (wrp & 1) * 8 + (tid & 7);
-    const int j = bz0 * DEX_BLOCK + part * (DEX_BLOCK / kParts) + (wrp >> 1) * 4 + ((tid & 31) >> 3);
+    const int wrp = tid >> 5, lane = tid & 31, tile = SPLIT ? part : part * NW + wrp;
+    const int i = bx0 * DEX_BLOCK + (tile & 1) * 8 + (lane & 7);
+    const int j = bz0 * DEX_BLOCK + (tile >> 1) * 4 + (lane >> 3);
+    const size_t cell = (size_t)j * P.nx + i;
     const int state0 = (s_info[blk0] & 7) - 1;
     if (state0 < 0) {  // state words do not describe this active block
         raise_status(P.status, DEX_ERR_TRAVERSAL_CAP);
@@ -133,35 +137,61 @@ __global__ void __launch_bounds__(pair_threads<ST>(), pair_min_blocks<ST>()) k_s
     G.z_hi = (s_box[3] + 1) * DEX_BLOCK;
 #pragma unroll
     for (int q = 0; q < 4; ++q) G.band[q] = P.band[q];
+    G.stop = -1.0f;
+    if (!COUNT && P.scanned) {
+        G.stop = stop_factor(join_bounds(P.J[(size_t)(b1 * 8) * P.n_cells + cell], P.J[(size_t)(b2 * 8) * P.n_cells + cell]), P.i_bc);
+    }
     const typename Model::Params M{(long long)(b2 - b1) * (long long)batch_floats};
     const int mip0 = min(state0, distance_cap(G, 0.0f));
     unsigned int nseg = 0;
     bool capped = false;
 
-    for (int k = 0; k < P.quad.n_dir; ++k) {
-        const float dx = P.quad.dx[k], dz = P.quad.dz[k];
-        float I[16], T[16];
+    auto ray = [&](int k, float* I, float* T) {
 #pragma unroll
         for (int w = 0; w < 16; ++w) {
             I[w] = 0.0f;
             T[w] = 1.0f;
         }
-        trace_ray<16, COUNT, Model, InfoLookup, EXT>(G, M, b1, i, j, bx0, bz0, a0, mip0, dx, dz, InfoLookup{s_info},
-                                                     I, T, nseg, capped);
-        const float wk = P.quad.w[k];
+        trace_ray<16, COUNT, Model, InfoLookup, EXT>(G, M, b1, i, j, bx0, bz0, a0, mip0, P.quad.dx[k], P.quad.dz[k],
+                                                     InfoLookup{s_info}, I, T, nseg, capped);
+    };
+    auto lambda = [&](int w) { return w < 8 ? b1 * 8 + w : b2 * 8 + (w - 8); };
+    auto store_I = [&](int w, int k, float Iw) {
+        if (P.I != nullptr && lambda(w) < P.n_lambda)
+            P.I[((size_t)lambda(w) * P.quad.n_dir + k) * P.n_cells + cell] = Iw;
+    };
+    if constexpr (SPLIT) {
+        __shared__ int s_next;
+        split_solve<16, NW>(
+            P.quad, reinterpret_cast<float*>(s_info) + P.split_at, &s_next, wrp, lane,
+            [&](int k, float* out) {
+                float I[16], T[16];
+                ray(k, I, T);
 #pragma unroll
-        for (int w = 0; w < 16; ++w) {
-            const float Iw = fmaf(T[w], P.i_bc, I[w]);
-            s_J[w][tid] = fmaf(wk, Iw, s_J[w][tid]);
-            const int l = w < 8 ? b1 * 8 + w : b2 * 8 + (w - 8);
-            if (P.I != nullptr && l < P.n_lambda)
-                P.I[((size_t)l * P.quad.n_dir + k) * P.n_cells + (size_t)j * P.nx + i] = Iw;
+                for (int w = 0; w < 16; ++w) {
+                    const float Iw = fmaf(T[w], P.i_bc, I[w]);
+                    out[w * 32] = Iw;
+                    store_I(w, k, Iw);
+                }
+            },
+            [&](int w, float J) {
+                if (lambda(w) < P.n_lambda) P.J[(size_t)lambda(w) * P.n_cells + cell] = J;
+            });
+    } else {
+        for (int k = 0; k < P.quad.n_dir; ++k) {
+            float I[16], T[16];
+            ray(k, I, T);
+            const float wk = P.quad.w[k];
+#pragma unroll
+            for (int w = 0; w < 16; ++w) {
+                const float Iw = fmaf(T[w], P.i_bc, I[w]);
+                s_J[w][tid] = fmaf(wk, Iw, s_J[w][tid]);
+                store_I(w, k, Iw);
+            }
         }
-    }
 #pragma unroll
-    for (int w = 0; w < 16; ++w) {
-        const int l = w < 8 ? b1 * 8 + w : b2 * 8 + (w - 8);
-        if (l < P.n_lambda) P.J[(size_t)l * P.n_cells + (size_t)j * P.nx + i] = s_J[w][tid];
+        for (int w = 0; w < 16; ++w)
+            if (lambda(w) < P.n_lambda) P.J[(size_t)lambda(w) * P.n_cells + cell] = s_J[w][tid];
     }
     if (capped) raise_status(P.status, DEX_ERR_TRAVERSAL_CAP);
     // segments of the two batches
@@ -169,12 +199,20 @@ __global__ void __launch_bounds__(pair_threads<ST>(), pair_min_blocks<ST>()) k_s
 }
 
 template <int ST>
-cudaError_t launch_pair(cudaStream_t s, const HddaParams& P)
+cudaError_t launch_pair(cudaStream_t s, const HddaParams& P0)
 {
-    const size_t smem = sizeof(int) * (size_t)P.nbx * P.nbz;
-    dim3 grid((unsigned)(P.cap_active * pair_parts<ST>()), (unsigned)pair_count(P.n_batch, P.pair_group));
-    auto kernel = P.exclude_own ? (P.seg_count ? k_solve_hdda_pair<ST, true, true> : k_solve_hdda_pair<ST, false, true>)
-                                : (P.seg_count ? k_solve_hdda_pair<ST, true, false> : k_solve_hdda_pair<ST, false, false>);
+    HddaParams P = P0;
+    const unsigned pairs = (unsigned)pair_count(P.n_batch, P.pair_group);
+    P.split_at = (P.nbx * P.nbz + 3) & ~3;
+    const bool split = split_directions(P);
+    const size_t smem = sizeof(int) * (size_t)P.split_at + (split ? split_bytes<16>() : 0);
+    const dim3 grid((unsigned)P.cap_active * (split ? 8u : (unsigned)pair_parts<ST>()), pairs);
+    auto kernel = P.seg_count ? (P.exclude_own ? k_solve_hdda_pair<ST, true, true, false>
+                                               : k_solve_hdda_pair<ST, true, false, false>)
+                  : split     ? (P.exclude_own ? k_solve_hdda_pair<ST, false, true, true>
+                                               : k_solve_hdda_pair<ST, false, false, true>)
+                              : (P.exclude_own ? k_solve_hdda_pair<ST, false, true, false>
+                                               : k_solve_hdda_pair<ST, false, false, false>);
     if (smem > 24 * 1024) {
         cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         if (e != cudaSuccess) return e;

@@ -42,7 +42,7 @@ struct VelModel {
         return Voxel{h.x, h.y, h.z, q + 4};
     }
     __device__ __forceinline__ static void integrate(const Params&, const Voxel& v, int, float wx, float wz,
-                                                     float nl2, float* I, float* T)
+                                                     float nl2, float* I, float* T, float)
     {
         const float proj = fminf(fmaxf(fmaf(v.vx, wx, v.vz * wz), -v.V), v.V);
         const float f = v.V > 0.0f ? __fdividef(proj + v.V, 2.0f * v.V) * (float)(kNV - 1) : 0.0f;

@@ -15,6 +15,8 @@ import synth
 
 pytestmark = pytest.mark.gpu
 
+BAND = [6.0, 24.0, 96.0]
+
 
 def ctx_():
     from paper_2511_08498_gb300 import api
@@ -74,3 +76,30 @@ def test_plain_records_without_a_bound(bad):
     fast = api.formal_solve_dense(ctx, nx, nz, L, W, planes, dirs, w, want_intensity=True)
     for a, b in zip(full[:2], fast[:2]):
         assert np.array_equal(a.cpu().numpy(), b.cpu().numpy(), equal_nan=True)
+
+
+@pytest.mark.parametrize("walk", ["per_batch", "paired"])
+@pytest.mark.parametrize("nx,nz,L,W,storage", [(64, 48, 20, 8, 0), (64, 48, 24, 8, 1), (48, 64, 17, 8, 2),
+                                               (48, 48, 6, 4, 0), (512, 512, 24, 8, 0), (32, 32, 3, 1, 0)])
+def test_sparse(walk, nx, nz, L, W, storage):
+    from paper_2511_08498_gb300 import api
+    if walk == "paired" and W != 8:
+        pytest.skip("the paired walk needs W = 8")
+    ctx = ctx_()
+    eta, chi = thick_medium(nx, nz, L, 820 + L, emitters=storage == 0)
+    grid = api.grid_build(ctx, nx, nz, eta, chi)
+    dirs, w = synth.directions(10, offset=0.0)
+    ctx.set_traversal(api.TRAVERSAL_PAIRED if walk == "paired" else api.TRAVERSAL_PER_BATCH)
+    for iod, band, i_bc in ((1e-2, BAND, 0.0), (1e30, None, 0.4)):
+        mips = api.mips_build(ctx, grid, eta, chi, W, 3, iod, iod, storage=storage)
+        for own in (True, False):
+            if not own and (W != 8 or storage != 0):
+                continue
+            ctx.set_own_cell(own)
+            full = api.formal_solve_hdda(ctx, grid, mips, dirs, w, band=band, i_bc=i_bc, want_intensity=True,
+                                         count_segments=True)
+            fast = api.formal_solve_hdda(ctx, grid, mips, dirs, w, band=band, i_bc=i_bc, want_intensity=True)
+            same(full[0], fast[0])
+            same(full[1], fast[1])
+        ctx.set_own_cell(True)
+    ctx.check()
