@@ -3,6 +3,8 @@
 // See k_hdda.cu for the description of the traversal.
 #pragma once
 
+#include <type_traits>
+
 #include "dex_internal.h"
 
 namespace dex {
@@ -90,6 +92,18 @@ struct SplitOf<M, decltype((void)M::kSplit)> {
     static constexpr int stride = M::kSplitStride;
 };
 
+// Models whose grids are bounded so that a batch's bricks span less than 4 GB declare
+// kOffset32 = true: the walk then keeps the current record as a 32-bit byte offset
+// from the batch's base, one register and one add per step instead of two.
+template <class M, class = void>
+struct Offset32Of {
+    static constexpr bool value = false;
+};
+template <class M>
+struct Offset32Of<M, decltype((void)M::kOffset32)> {
+    static constexpr bool value = M::kOffset32;
+};
+
 // Record load of a voxel model: Model::load(M, p) where the model declares it
 // (its records need the launch parameters, e.g. a second batch's offset),
 // Model::load(p) otherwise.
@@ -118,6 +132,9 @@ struct PairRecModel {
     static constexpr int kMinBlocks = MINB;
     static constexpr bool kEarlyLoad = ST == kStoreF32;
     static constexpr bool kZeroNoop = false;
+    // grids of at most kPairInfoMaxBlocks blocks: 341 voxels of 64 bytes each
+    static constexpr bool kOffset32 = true;
+    static_assert(64LL * 341 * kPairInfoMaxBlocks < (1LL << 32), "offsets of the paired walk");
     struct Params {
         long long off;
     };
@@ -184,9 +201,9 @@ __device__ __forceinline__ void model_stage(const typename Model::Params&, long)
 //
 // Each step integrates the voxel it leaves and steps to the next voxel of the
 // same level; only a step that leaves the block (one divergent branch) looks up
-// the next block: after the integration for models with kZeroNoop (the
-// transmission test then sees the block's last segment), before it otherwise.  A ray's block indices change monotonically and it takes at
-// most 2 * 16 steps in a block, so the grid bounds check also bounds the loop.
+// the next block: after the integration for models with kZeroNoop, before it
+// otherwise.  A ray's block indices change monotonically and it takes at most 2 * 16
+// steps in a block, so the grid bounds check also bounds the loop.
 template <int W, bool COUNT, class Model, class Lookup, bool EXT = false>
 __device__ __forceinline__ void trace_ray(const Geo& G, const typename Model::Params& M, int b, int i, int j,
                                           int bx0, int bz0, int a0, int mip0, float dx, float dz,
@@ -198,6 +215,20 @@ __device__ __forceinline__ void trace_ray(const Geo& G, const typename Model::Pa
     constexpr int XS = kSplit ? SplitOf<Model>::stride : REC;  // floats between x neighbours of a row
     static_assert(!kSplit || Model::kEarlyLoad, "float32 brick rows are read at the top of the step");
     const float* __restrict__ batch_base = G.batch_base;
+    // position of a record: a pointer, or a byte offset from the batch's base
+    constexpr bool k32 = Offset32Of<Model>::value;
+    using Pos = std::conditional_t<k32, unsigned int, const float*>;
+    constexpr int UNIT = k32 ? 4 : 1;
+    auto pos_of = [&](int block, int m, int z, int x, int sd) -> Pos {
+        if constexpr (k32)
+            return ((unsigned)(block * G.chain + level_offset(m) + z * sd) * REC + (unsigned)(x * XS)) * 4u;
+        else
+            return batch_base + ((size_t)block * G.chain + level_offset(m) + z * sd) * REC + x * XS;
+    };
+    auto record = [&](Pos r) -> const float* {
+        if constexpr (k32) return reinterpret_cast<const float*>(reinterpret_cast<const char*>(batch_base) + r);
+        else return r;
+    };
     const float ox = (float)i + 0.5f, oz = (float)j + 0.5f;
     const bool negx = dx < 0.0f, negz = dz < 0.0f;
     const int sx = negx ? -1 : 1, sz = negz ? -1 : 1;
@@ -215,14 +246,15 @@ __device__ __forceinline__ void trace_ray(const Geo& G, const typename Model::Pa
     float Px = (float)(bx0 * DEX_BLOCK + (lx + (negx ? 0 : 1)) * vox - i) - 0.5f;
     float Pz = (float)(bz0 * DEX_BLOCK + (lz + (negz ? 0 : 1)) * vox - j) - 0.5f;
     // record (S) of the current voxel: rows of side voxels, x neighbours XS floats apart
-    const float* rp = batch_base + ((size_t)a0 * G.chain + level_offset(mip) + lz * side) * REC + lx * XS;
+    Pos rp = pos_of(a0, mip, lz, lx, side);
+    // signed steps of the plane offsets and the record position: kept where the
+    // 32-bit position has freed the registers for them, formed in each step otherwise
+    float fvx = negx ? -fvox : fvox, fvz = negz ? -fvox : fvox;
+    int rz = (negz ? -side : side) * (REC * UNIT);
     float th_prev = 0.0f, tl_prev = 0.0f;
     // the step left the block: look up the next one and re-initialise the tracer
     // there (false: the ray ends)
     auto enter = [&](bool on_x, float th) -> bool {
-        // early termination: the rest of the ray changes no bit of I (1024^2 paired
-        // benchmark solve: 165 -> 105 ms, J bit-identical)
-        if (ray_done<W>(I, T, G.stop)) return false;
         if (on_x) bxc += sx;
         else bzc += sz;
         if ((unsigned)bxc >= (unsigned)G.nbx || (unsigned)bzc >= (unsigned)G.nbz) {
@@ -255,28 +287,29 @@ __device__ __forceinline__ void trace_ray(const Geo& G, const typename Model::Pa
             vox = 1 << shift;
             fvox = (float)vox;
             side = DEX_BLOCK >> shift;
+            fvx = negx ? -fvox : fvox;
+            fvz = negz ? -fvox : fvox;
+            rz = (negz ? -side : side) * (REC * UNIT);
             lx = (m0x - bxc * DEX_BLOCK) >> shift;
             lz = (m0z - bzc * DEX_BLOCK) >> shift;
             Px = (float)(bxc * DEX_BLOCK + (lx + (negx ? 0 : 1)) * vox - i) - 0.5f;
             Pz = (float)(bzc * DEX_BLOCK + (lz + (negz ? 0 : 1)) * vox - j) - 0.5f;
         }
-        if (mip >= 0)
-            rp = batch_base + ((size_t)L.offset_of(key) * G.chain + level_offset(mip) + lz * side) * REC + lx * XS;
-        else if (kZero)
-            rp = g_zero_record;
+        if (mip >= 0) rp = pos_of(L.offset_of(key), mip, lz, lx, side);
+        else if constexpr (kZero) rp = g_zero_record;
         return true;
     };
     typename Model::Voxel cur;
 
-    constexpr int kUnroll = UnrollOf<Model>::value;
+    constexpr int kUnroll = UnrollOf<Model>::value, kStopEvery = kUnroll == 1 ? 1 : 4;
 #pragma unroll kUnroll
     for (int it = 0;; ++it) {
         // models with kEarlyLoad issue the current voxel's record before the
         // stepping and crossing bookkeeping, which then hides its latency
         if constexpr (Model::kEarlyLoad) {
             if (kZero || mip >= 0) {
-                if constexpr (kSplit) cur = Model::load_split(M, rp, side * XS);
-                else cur = model_load<Model>(M, rp);
+                if constexpr (kSplit) cur = Model::load_split(M, record(rp), side * XS);
+                else cur = model_load<Model>(M, record(rp));
             }
         }
         const float tnx = Px * ax.ih, tnz = Pz * az.ih;
@@ -286,18 +319,18 @@ __device__ __forceinline__ void trace_ray(const Geo& G, const typename Model::Pa
         const float len = fmaxf((th - th_prev) + (tl - tl_prev), 0.0f);
         const bool last = th >= t2;
         const int cur_mip = mip;
-        const float* cur_rp = rp;
+        const Pos cur_rp = rp;
         // step to the next voxel of this level (not used once last)
         bool cross;
         if (on_x) {
             lx += sx;
-            Px += negx ? -fvox : fvox;
-            rp += negx ? -XS : XS;
+            Px += k32 ? fvx : (negx ? -fvox : fvox);
+            rp += (negx ? -XS : XS) * UNIT;
             cross = (unsigned)lx >= (unsigned)side;
         } else {
             lz += sz;
-            Pz += negz ? -fvox : fvox;
-            rp += negz ? -side * REC : side * REC;
+            Pz += k32 ? fvz : (negz ? -fvox : fvox);
+            rp += k32 ? rz : (negz ? -side * REC : side * REC);
             cross = (unsigned)lz >= (unsigned)side;
         }
         if constexpr (!kZero) {
@@ -307,7 +340,7 @@ __device__ __forceinline__ void trace_ray(const Geo& G, const typename Model::Pa
         }
         // integrate the voxel left (in empty blocks: the zero record, or nothing)
         if (kZero || cur_mip >= 0) {
-            if constexpr (!Model::kEarlyLoad) cur = model_load<Model>(M, cur_rp);
+            if constexpr (!Model::kEarlyLoad) cur = model_load<Model>(M, record(cur_rp));
             Model::integrate(M, cur, b, -dx, -dz, len * kNegLog2e, I, T, G.stop);
             if constexpr (EXT) {
                 if (it == 0) {
@@ -317,10 +350,9 @@ __device__ __forceinline__ void trace_ray(const Geo& G, const typename Model::Pa
             }
             if (COUNT) nseg += (cur_mip >= 0) & (th > th_prev);
         }
-        if (last) break;
-        // within blocks the termination test runs every fourth step: in thick cells
-        // rays end long before the next block face
-        if ((it & 3) == 3 && ray_done<W>(I, T, G.stop)) break;
+        // early termination, tested by all lanes together every few steps: the rest of
+        // the ray changes no bit of I (1024^2 paired benchmark solve: 163 -> 95 ms)
+        if (last || ((it & (kStopEvery - 1)) == kStopEvery - 1 && ray_done<W>(I, T, G.stop))) break;
         th_prev = th;
         tl_prev = tl;
         if constexpr (kZero) {
