@@ -20,8 +20,8 @@
 // evaluated as a ray along each w_k samples them, u = dv + v_child . w_k: the
 // closest-to-core values of children moving in different directions can agree
 // while the profiles a ray sees are shifted apart.
-#include "hdda.cuh"
 #include "mlp.cuh"
+#include "scan.cuh"
 #include "vlm.cuh"
 #include "voigt.cuh"
 
@@ -63,6 +63,7 @@ struct CavMlpModel {
     static constexpr bool kEarlyLoad = false;
     static constexpr bool kZeroNoop = false;  // profile parameters of zero are not a no-op
     using Params = CavMlpParams;
+    __device__ __forceinline__ static void stage(const Params& M) { stage_dawson(M.cav.coef); }
     struct Voxel {
         float p[kCavStride];
     };
@@ -98,10 +99,14 @@ template <int W>
 struct CavModel {
     static constexpr int kStride = kCavStride;
     static constexpr bool kPerBatch = false;
-    static constexpr int kMinBlocks = 4;
+    static constexpr int kMinBlocks = 3;  // 4 CTAs per SM (64 registers): 101 against 95 ms
     static constexpr bool kEarlyLoad = false;
     static constexpr bool kZeroNoop = false;  // profile parameters of zero are not a no-op
+    // one copy of the step: four copies of eight profiles overflowed the instruction
+    // cache (5.6 of 13 stall cycles per instruction waited for instructions)
+    static constexpr int kUnroll = 1;
     using Params = CavParams;
+    __device__ __forceinline__ static void stage(const Params& M) { stage_dawson(M.coef); }
     struct Voxel {
         float p[kCavStride];
     };
@@ -114,14 +119,16 @@ struct CavModel {
         return v;
     }
     __device__ __forceinline__ static void integrate(const Params& M, const Voxel& v, int b, float wx, float wz,
-                                                     float nl2, float* I, float* T, float)
+                                                     float nl2, float* I, float* T, float stop)
     {
         const float proj = fmaf(v.p[4], wx, v.p[5] * wz);
-        // not unrolled: eight inlined copies of the four-branch Voigt evaluation made
-        // the solve instruction-fetch bound (1024 x 512, 64 wavelengths: 9.4 s against
-        // 2.3 s with one copy; bit-identical)
-#pragma unroll 1
+        // unrolled: the wavelengths' I and T stay in registers (one copy of the body:
+        // 110 against 101 ms at 512 x 256, 64 wavelengths)
+#pragma unroll
         for (int w = 0; w < W; ++w) {
+            // a wavelength whose intensity can no longer change (ray_done's test) needs
+            // no profile: line cores end long before the batch's other wavelengths
+            if (stop >= 0.0f && T[w] * stop <= I[w]) continue;
             const int l = b * W + w;
             float eta, chi;
             cav_eta_chi(M, v.p, l, M.dv[l] + proj, eta, chi);
@@ -130,6 +137,33 @@ struct CavModel {
         }
     }
 };
+
+// Bound of the early termination: a mixture of line and continuum emits at most
+// the larger of their source functions.
+__device__ __forceinline__ float cav_bound(float e, float c)
+{
+    return c > 0.0f ? bound_of(__fdividef(e, c), c) : (e == 0.0f && c == 0.0f ? 0.0f : -1.0f);
+}
+
+// CTA a: the bound of active block a, to its first cell in every batch (the
+// records are shared by the batches).
+__global__ void __launch_bounds__(128) k_scan_cav(const HddaParams P)
+{
+    const int a = blockIdx.x;
+    if (a >= *P.n_active) return;
+    const float* brick = P.bricks + (size_t)a * P.chain * kCavStride;
+    float m = 0.0f;
+    for (int q = threadIdx.x; q < P.chain; q += blockDim.x) {
+        const float* p = brick + (size_t)q * kCavStride;
+        m = join_bounds(m, join_bounds(cav_bound(p[0], p[1]), cav_bound(p[6], p[7])));
+    }
+    // the ratios' rounding, and the profile's where it should vanish
+    m = join_cta(m) * 16.0f;
+    const int blk = P.active[a];
+    if (threadIdx.x < P.n_batch)
+        for (int b = threadIdx.x; b < P.n_batch; b += blockDim.x)
+            P.J[(size_t)(b * P.W) * P.n_cells + (size_t)(blk / P.nbx * DEX_BLOCK) * P.nx + blk % P.nbx * DEX_BLOCK] = m;
+}
 
 // flag[blk] = 1 if any parameter that makes emission or opacity is non-zero in the block
 __global__ void __launch_bounds__(256) k_cav_block_flags(int nx, int nbx, CavFields F, int* __restrict__ flag)
@@ -146,6 +180,7 @@ template <int W>
 __global__ void __launch_bounds__(256) k_cav_mips_build(const CavMipParams P, const CavParams M)
 {
     __shared__ float sp[level_offset(5)][kCavStride];
+    stage_dawson(M.coef);
     const int a = blockIdx.x;
     if (a >= *P.n_active) return;
     const int b = blockIdx.y;
@@ -325,9 +360,15 @@ cudaError_t launch_solve_cav_mlp(cudaStream_t s, const HddaParams& P, const CavM
     return cudaGetLastError();
 }
 
-cudaError_t launch_solve_cav(cudaStream_t s, const HddaParams& P, const CavParams& M)
+cudaError_t launch_solve_cav(cudaStream_t s, const HddaParams& P0, const CavParams& M)
 {
-    if (P.cap_active == 0 || P.n_batch == 0) return cudaSuccess;
+    if (P0.cap_active == 0 || P0.n_batch == 0) return cudaSuccess;
+    HddaParams P = P0;
+    if (!P.seg_count) {
+        k_scan_cav<<<(unsigned)P.cap_active, 128, 0, s>>>(P);
+        launch_spread(s, P);
+        P.scanned = 1;
+    }
     const size_t smem = sizeof(unsigned long long) * (size_t)P.n_words;
     dim3 grid((unsigned)P.cap_active, (unsigned)P.n_batch);
     cudaError_t e = cudaSuccess;

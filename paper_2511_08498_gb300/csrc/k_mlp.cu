@@ -439,6 +439,8 @@ __global__ void k_mlp_adam(float* __restrict__ p, const float* __restrict__ g, f
 // ------------------------------------------------------ training targets --
 __global__ void k_mlp_targets(long long n, const float* __restrict__ xau, float* __restrict__ out, VoigtCoef C)
 {
+    stage_dawson(C);
+    __syncthreads();
     const long long s = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     if (s >= n) return;
     out[s] = logf(voigt_h(C, xau[3 * s + 1], xau[3 * s] - xau[3 * s + 2]));

@@ -81,6 +81,8 @@ __global__ void __launch_bounds__(256) k_vel_mips_build(const CavMipParams P, co
     __shared__ float s_e[level_offset(5)][W];             // rest-frame eta chain
     __shared__ float s_c[level_offset(5)][W];             // rest-frame chi chain
     __shared__ float s_v[level_offset(5)][3];             // mean vx, mean vz, max speed
+    stage_dawson(M.coef);
+    __syncthreads();
     const int a = blockIdx.x;
     if (a >= *P.n_active) return;
     const int b = blockIdx.y;

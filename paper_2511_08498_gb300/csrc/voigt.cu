@@ -1,4 +1,4 @@
-// Voigt function: host-side Weideman coefficients, constant-memory upload, and
+// Voigt function: host-side coefficients (Weideman's sum, Dawson's integral) and
 // an elementwise kernel behind dex_voigt.
 #include <cmath>
 #include <mutex>
@@ -25,9 +25,30 @@ void weideman_coefficients(double* a, int n)
     }
 }
 
+// D^(n)(x) / n!, n = 1 .. kDawsonTerms
+void dawson_coefficients(double x, float* c)
+{
+    // D(x) = e^{-x^2} sum_k x^(2k+1) / (k! (2k+1))
+    double term = x, sum = x;
+    for (int k = 1; k < 200; ++k) {
+        term *= x * x / k;
+        sum += term / (2 * k + 1);
+    }
+    double prev = std::exp(-x * x) * sum, cur = 1.0 - 2.0 * x * prev, fact = 1.0;
+    for (int n = 1; n <= kDawsonTerms; ++n) {
+        fact *= n;
+        c[n - 1] = (float)(cur / fact);
+        const double next = -2.0 * x * cur - 2.0 * n * prev;
+        prev = cur;
+        cur = next;
+    }
+}
+
 __global__ void k_voigt(const VoigtCoef C, long long n, const float* __restrict__ a, const float* __restrict__ x,
                         float* __restrict__ h)
 {
+    stage_dawson(C);
+    __syncthreads();
     for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x)
         h[i] = voigt_h(C, a[i], x[i]);
 }
@@ -42,6 +63,7 @@ const VoigtCoef& voigt_coefficients()
         double a[kWeidemanN];
         weideman_coefficients(a, kWeidemanN);
         for (int i = 0; i < kWeidemanN; ++i) coef.a[i] = (float)a[i];
+        for (int i = 0; i < kDawsonNodes; ++i) dawson_coefficients(i / 8.0, coef.dawson + i * kDawsonTerms);
     });
     return coef;
 }
