@@ -11,20 +11,20 @@
 // Tensor cores (tcgen05, kind::f16, accumulators in tensor memory) do every
 // contraction over the hidden width or over the samples of a tile; CUDA cores
 // do the 3-input first layer, the activations and the output dot product.
-// One CTA of 128 threads owns tiles of 128 samples, thread t = sample t = TMEM
-// lane t.  Per tile:
+// Tiles hold 128 samples, sample = TMEM lane: inference one thread per sample (128
+// threads), training two (256; each has half of the hidden units).  Per tile:
 //   forward   D2 = H1 W2^T                      (M 128, N 64, K 64)
 //   backward  D3 = Delta2 W2                    (M 128, N 64, K 64)   -> dL/dh1
-//             D4 += [Delta2^T; (dy h2)^T] [H1^T; 1]^T
-//                                               (M 128, N 80, K 128)  -> dW2, db2, dw3
-//             D5 += Delta1^T [F^T; 1]^T         (M 128, N 16, K 128)  -> dW1, db1
-// (tensor-memory columns: D2 0-63, D3 64-127, D4 128-207, D5 224-239 of 256)
+//             D4 += [Delta2, dy h2]^T [H1, 1]   (M 128, N 80, K 128)  -> dW2, db2, dw3
+//             D5 += [Delta1, .]^T [F, 1]        (M 128, N 16, K 128)  -> dW1, db1
+// (tensor-memory columns: D2 0-63, D3 64-127, D4 128-207, D5 224-239 of 256).  The
+// sums over samples read the row-per-sample tiles as MN-major operands, so nothing
+// is stored twice; W2 likewise serves D2 and D3.
 // D4 and D5 accumulate over all tiles of the CTA and are added to the global
 // gradient once at the end.  Every mbarrier wait is bounded; on expiry the CTA
 // records DEX_ERR_TIMEOUT, waits (bounded) once more, frees its tensor memory
 // and returns.
 #include <cmath>
-#include <cstddef>
 
 #include "dex_internal.h"
 #include "mlp.cuh"
@@ -36,8 +36,6 @@ namespace dex {
 namespace {
 
 using namespace umma;
-using mlp::Act;
-using mlp::gelu;
 using mlp::kB1;
 using mlp::kB2;
 using mlp::kB3;
@@ -49,47 +47,48 @@ using mlp::kW3;
 constexpr int kTile = 128;  // samples per tile (MMA M)
 constexpr int kWaitPolls = 1 << 20;
 
-// tile geometry (rows R of each K-major operand)
-constexpr int kRowsH1T = 80;  // 64 hidden units, the ones row 64, zero rows 65..79
-constexpr int kRowsFT = 16;   // 3 features, the ones row 3, zero rows 4..15
+constexpr int kColsH1 = 80;  // 64 hidden units, the ones column 64, zero columns 65..79
+constexpr int kColsF = 16;   // 3 features, the ones column 3, zero columns 4..15
 
 // TMEM columns
 constexpr uint32_t kColD2 = 0, kColD3 = 64, kColD4 = 128, kColD5 = 224;
 constexpr uint32_t kColsTrain = 256, kColsInfer = 64;
 
+// layer-1 weights by input feature: neighbouring units side by side
+struct SmemNet {
+    alignas(16) float w1t[3][kH];
+    alignas(16) float b1[kH];
+    float b2[kH], w3[kH], b3;
+};
+
 struct SmemInfer {
-    unsigned char W2[kH * kH * 2];        // B of D2: rows out j, K in i
-    unsigned char H1[kTile * kH * 2];     // A of D2: rows sample, K in i
-    float w1[kH * 3], b1[kH], b2[kH], w3[kH], b3;
-    alignas(16) float w1t[3][kH];         // w1 by input feature: neighbouring units side by side
+    alignas(16) unsigned char W2[kH * kH * 2];     // B of D2: rows out j, K in i
+    alignas(16) unsigned char H1[kTile * kH * 2];  // A of D2: rows sample, K in i
+    SmemNet net;
     unsigned long long mbar;
     unsigned int tmem;
 };
 
 struct SmemTrain {
-    unsigned char W2[kH * kH * 2];              // B of D2
-    unsigned char W2T[kH * kH * 2];             // B of D3: rows in i, K out j
-    unsigned char H1[kTile * kH * 2];           // A of D2
-    unsigned char D2[kTile * kH * 2];           // A of D3: rows sample, K out j
-    unsigned char D2T[kTile * kTile * 2];       // A of D4 (rows j: delta2, rows 64 + j: dy h2), then A of D5
-    unsigned char H1T[kRowsH1T * kTile * 2];    // B of D4: rows i (+ ones row), K sample
-    unsigned char FT[kRowsFT * kTile * 2];      // B of D5: rows feature (+ ones row), K sample
-    float w1[kH * 3], b1[kH], b2[kH], w3[kH], b3;
+    alignas(16) unsigned char W2[kH * kH * 2];          // [out j][in i]: B of D2, transposed B of D3
+    alignas(16) unsigned char H1[kTile * kColsH1 * 2];  // [sample][in i, 1]: A of D2, transposed B of D4
+    alignas(16) unsigned char D[kTile * 2 * kH * 2];    // [sample][delta2 | dy h2]: A of D3, transposed A of D4;
+                                                        // then delta1 in its first half: transposed A of D5
+    alignas(16) unsigned char F[kTile * kColsF * 2];    // [sample][feature, 1]: transposed B of D5
+    SmemNet net;
+    float y[2][kTile];
     float red_loss[4], red_gb3[4];
     unsigned long long mbar;
     unsigned int tmem;
 };
 
-// dynamic shared memory requested per CTA: at most 4 inference / 2 training
-// CTAs fit on an SM, so their tensor-memory allocations always fit (512 columns)
-constexpr size_t kSmemInfer = 48 * 1024;
-constexpr size_t kSmemTrain = 110 * 1024;
-static_assert(sizeof(SmemInfer) <= kSmemInfer, "inference shared memory");
-// the packed inference loads read float2 pairs of these arrays at even indices
-static_assert(offsetof(SmemInfer, b1) % 8 == 0 && offsetof(SmemInfer, b2) % 8 == 0 &&
-                  offsetof(SmemInfer, w3) % 8 == 0 && offsetof(SmemInfer, w1t) % 8 == 0,
-              "inference weight alignment");
-static_assert(sizeof(SmemTrain) <= kSmemTrain, "training shared memory");
+// Dynamic shared memory requested per CTA bounds the CTAs per SM so that their
+// tensor-memory allocations always fit its 512 columns: 8 x 64 inference, 2 x 256
+// training.
+constexpr size_t kSmemInfer = 27 * 1024;
+constexpr size_t kSmemTrain = 80 * 1024;
+static_assert(sizeof(SmemInfer) <= kSmemInfer && 9 * (kSmemInfer + 1024) > 228 * 1024, "inference shared memory");
+static_assert(sizeof(SmemTrain) <= kSmemTrain && 3 * kSmemTrain > 228 * 1024, "training shared memory");
 
 __device__ __forceinline__ float bf16_round(float x) { return __bfloat162float(__float2bfloat16_rn(x)); }
 
@@ -111,46 +110,50 @@ __device__ __forceinline__ bool features(const float* xau, long long s, float* f
     return true;
 }
 
-template <class S>
-__device__ void stage_weights(S& sm, const float* __restrict__ p, bool transposed_copy, unsigned char* W2T)
+__device__ void stage_weights(SmemNet& net, unsigned char* W2, const float* __restrict__ p)
 {
     const int t = threadIdx.x;
-    for (int q = t; q < kH * kH; q += blockDim.x) {
-        const int j = q / kH, i = q - j * kH;
-        const float w = p[kW2 + q];
-        put_bf16(sm.W2, tile_offset(j, i, kH), w);
-        if (transposed_copy) put_bf16(W2T, tile_offset(i, j, kH), w);
-    }
-    for (int q = t; q < kH * 3; q += blockDim.x) sm.w1[q] = bf16_round(p[kW1 + q]);
+    for (int q = t; q < kH * kH; q += blockDim.x) put_bf16(W2, tile_offset(q / kH, q % kH, kH), p[kW2 + q]);
+    for (int q = t; q < kH * 3; q += blockDim.x) net.w1t[q % 3][q / 3] = bf16_round(p[kW1 + q]);
     if (t < kH) {
-        sm.b1[t] = p[kB1 + t];
-        sm.b2[t] = p[kB2 + t];
-        sm.w3[t] = bf16_round(p[kW3 + t]);
+        net.b1[t] = p[kB1 + t];
+        net.b2[t] = p[kB2 + t];
+        net.w3[t] = bf16_round(p[kW3 + t]);
     }
-    if (t == 0) sm.b3 = p[kB3];
+    if (t == 0) net.b3 = p[kB3];
 }
 
-// layer 1 + GELU for sample row t: writes h1 (BF16) to H1 (row t), and when
-// H1T is given to H1T (column t); returns nothing else (z1 is recomputed).
-template <class S>
-__device__ __forceinline__ void layer1(S& sm, const float* f, int t, unsigned char* H1T)
-{
-#pragma unroll 1
-    for (int i0 = 0; i0 < kH; i0 += 8) {
-        __align__(16) __nv_bfloat16 hb[8];
-#pragma unroll
-        for (int q = 0; q < 8; ++q) {
-            const int i = i0 + q;
-            const float z = fmaf(sm.w1[3 * i + 2], f[2], fmaf(sm.w1[3 * i + 1], f[1], fmaf(sm.w1[3 * i], f[0], sm.b1[i])));
-            hb[q] = __float2bfloat16_rn(gelu(z).g);
-            if (H1T) *reinterpret_cast<__nv_bfloat16*>(H1T + tile_offset(i, t, kRowsH1T)) = hb[q];
-        }
-        *reinterpret_cast<uint4*>(sm.H1 + tile_offset(t, i0, kTile)) = *reinterpret_cast<const uint4*>(hb);
+// GELU of two hidden units on the packed FP32 pipe.  The special-function units
+// bound these kernels (2^x and a reciprocal per activation: 16 per SM and clock),
+// so the two logistic functions share one reciprocal, 1/a = b / (a b): three
+// special-function operations for two activations.  2^x is bounded at 2^60, below
+// which the product cannot overflow and above which the activation is 0 to 1e-17.
+struct Gelu2 {
+    float2 z, z2, s;
+    __device__ __forceinline__ explicit Gelu2(float2 zz) : z(zz)
+    {
+        // -2 log2(e) c (z + k z^3), c = sqrt(2 / pi), k = 0.044715
+        constexpr float c1 = -2.3022081986f, c2 = -0.1029432397f;
+        z2 = __fmul2_rn(z, z);
+        const float2 a = __fmul2_rn(z, __ffma2_rn(make_float2(c2, c2), z2, make_float2(c1, c1)));
+        const float2 e = make_float2(mlp::mlp_ex2(fminf(a.x, 60.0f)), mlp::mlp_ex2(fminf(a.y, 60.0f)));
+        const float2 d = __fadd2_rn(make_float2(1.0f, 1.0f), e);
+        const float r = mlp::mlp_rcp(d.x * d.y);
+        s = __fmul2_rn(make_float2(r, r), make_float2(d.y, d.x));
     }
-}
+    __device__ __forceinline__ float2 g() const { return __fmul2_rn(z, s); }
+    // s + z s (1 - s) 2 c (1 + 3 k z^2), from g = z s
+    __device__ __forceinline__ float2 dg(float2 g) const
+    {
+        constexpr float k0 = 1.5957691216f, k1 = 0.2140644488f;  // 2 c, 6 c k
+        const float2 q = __ffma2_rn(make_float2(-g.x, -g.y), s, g);
+        return __ffma2_rn(q, __ffma2_rn(make_float2(k1, k1), z2, make_float2(k0, k0)), s);
+    }
+};
 
-// GELU of two hidden units at once on the packed FP32 pipe (FMUL2/FFMA2/FADD2):
-// every lane rounded exactly as mlp::gelu(z).g
+// GELU of two hidden units, every lane rounded as mlp::gelu(z).g: for activations
+// that are rounded to bfloat16 next, where another float32 rounding now and then
+// lands on the other side of a bfloat16 boundary.
 __device__ __forceinline__ float2 gelu2(float2 z)
 {
     const float c = 0.79788456080286536f, k = 0.044715f;
@@ -162,36 +165,44 @@ __device__ __forceinline__ float2 gelu2(float2 z)
     return __fmul2_rn(z, make_float2(mlp::mlp_rcp(d.x), mlp::mlp_rcp(d.y)));
 }
 
-// layer 1 + GELU for sample row t (inference): units in pairs on the packed pipe,
-// every value rounded as in layer1()
-__device__ __forceinline__ void layer1_infer(SmemInfer& sm, const float* f, int t)
+// GELU of four hidden units with one reciprocal: 1/(p q) gives q/(p q) and p/(p q) for
+// the two pairs' products, as in Gelu2.  2^x is bounded at 2^30 (the product below
+// 2^121): activations at z < -5.6 come out as z 2^-30, off by less than 6e-9.
+__device__ __forceinline__ void gelu4(float2 za, float2 zb, float2& ga, float2& gb)
 {
-    const float2 f0 = make_float2(f[0], f[0]), f1 = make_float2(f[1], f[1]), f2 = make_float2(f[2], f[2]);
-#pragma unroll 1
-    for (int i0 = 0; i0 < kH; i0 += 8) {
-        __align__(16) __nv_bfloat162 hb[4];
-#pragma unroll
-        for (int q = 0; q < 4; ++q) {
-            const int i = i0 + 2 * q;
-            const float2 b = *reinterpret_cast<const float2*>(&sm.b1[i]);
-            const float2 w0 = *reinterpret_cast<const float2*>(&sm.w1t[0][i]);
-            const float2 w1 = *reinterpret_cast<const float2*>(&sm.w1t[1][i]);
-            const float2 w2 = *reinterpret_cast<const float2*>(&sm.w1t[2][i]);
-            const float2 z = __ffma2_rn(w2, f2, __ffma2_rn(w1, f1, __ffma2_rn(w0, f0, b)));
-            hb[q] = __float22bfloat162_rn(gelu2(z));
-        }
-        *reinterpret_cast<uint4*>(sm.H1 + tile_offset(t, i0, kTile)) = *reinterpret_cast<const uint4*>(hb);
-    }
+    auto den = [](float2 z) {
+        constexpr float c1 = -2.3022081986f, c2 = -0.1029432397f;
+        const float2 a = __fmul2_rn(z, __ffma2_rn(make_float2(c2, c2), __fmul2_rn(z, z), make_float2(c1, c1)));
+        return __fadd2_rn(make_float2(1.0f, 1.0f),
+                          make_float2(mlp::mlp_ex2(fminf(a.x, 30.0f)), mlp::mlp_ex2(fminf(a.y, 30.0f))));
+    };
+    const float2 da = den(za), db = den(zb);
+    const float pa = da.x * da.y, pb = db.x * db.y, r = mlp::mlp_rcp(pa * pb), ra = r * pb, rb = r * pa;
+    ga = __fmul2_rn(za, __fmul2_rn(make_float2(ra, ra), make_float2(da.y, da.x)));
+    gb = __fmul2_rn(zb, __fmul2_rn(make_float2(rb, rb), make_float2(db.y, db.x)));
+}
+
+__device__ __forceinline__ unsigned int pack_bf16(float2 v)
+{
+    const __nv_bfloat162 b = __float22bfloat162_rn(v);
+    return *reinterpret_cast<const unsigned int*>(&b);
+}
+
+// z1 of units i, i + 1
+__device__ __forceinline__ float2 layer1_z(const SmemNet& net, const float* f, int i)
+{
+    const float2 b = *reinterpret_cast<const float2*>(&net.b1[i]);
+    const float2 w0 = *reinterpret_cast<const float2*>(&net.w1t[0][i]);
+    const float2 w1 = *reinterpret_cast<const float2*>(&net.w1t[1][i]);
+    const float2 w2 = *reinterpret_cast<const float2*>(&net.w1t[2][i]);
+    return __ffma2_rn(w2, make_float2(f[2], f[2]),
+                      __ffma2_rn(w1, make_float2(f[1], f[1]), __ffma2_rn(w0, make_float2(f[0], f[0]), b)));
 }
 
 // one MMA chain: D (+)= A B^T over K/16 K-steps, issued by the calling thread
-__device__ __forceinline__ void mma_chain(uint32_t d, const unsigned char* A, int rowsA, const unsigned char* B,
-                                          int rowsB, int K, uint32_t idesc, bool accumulate)
+__device__ __forceinline__ void mma_chain(uint32_t d, Operand A, Operand B, int K, uint32_t idesc, bool accumulate)
 {
-    const uint32_t a0 = smem_u32(A), b0 = smem_u32(B);
-    for (int k = 0; k < K / 16; ++k)
-        mma_bf16(d, smem_desc(a0 + k * kstep_bytes(rowsA)), smem_desc(b0 + k * kstep_bytes(rowsB)), idesc,
-                 accumulate || k > 0);
+    for (int k = 0; k < K / 16; ++k) mma_bf16(d, A.step(k), B.step(k), idesc, accumulate || k > 0);
 }
 
 // make every thread's shared-memory writes and TMEM reads ordered before the
@@ -215,13 +226,15 @@ __device__ __forceinline__ bool wait_all(unsigned long long* mbar, uint32_t& pha
 }
 
 // ------------------------------------------------------------ inference --
-__global__ void __launch_bounds__(128, 1) k_mlp_forward(const MlpParams P)
+// Bound by the special-function units (208 operations per sample, of 16 per SM and
+// clock: 174 us for 2^22 samples); eight CTAs per
+// SM, whose phases interleave, hide the barriers and the MMA's latency.
+__global__ void __launch_bounds__(128, 8) k_mlp_forward(const MlpParams P)
 {
     extern __shared__ __align__(1024) unsigned char smem_raw[];
     SmemInfer& sm = *reinterpret_cast<SmemInfer*>(smem_raw);
     const int t = threadIdx.x, warp = t >> 5;
-    stage_weights(sm, P.params, false, nullptr);
-    for (int q = t; q < kH * 3; q += blockDim.x) sm.w1t[q % 3][q / 3] = bf16_round(P.params[kW1 + q]);
+    stage_weights(sm.net, sm.W2, P.params);
     if (t == 0) mbar_init(&sm.mbar, 1);
     if (warp == 0) tmem_alloc(&sm.tmem, kColsInfer);
     sync_for_mma();
@@ -237,24 +250,35 @@ __global__ void __launch_bounds__(128, 1) k_mlp_forward(const MlpParams P)
             raise_status(P.status, DEX_ERR_NUMERIC);
             valid = false;
         }
-        layer1_infer(sm, f, t);
+#pragma unroll 2
+        for (int i0 = 0; i0 < kH; i0 += 8) {
+            uint4 h;
+            unsigned int* hw = reinterpret_cast<unsigned int*>(&h);
+#pragma unroll
+            for (int q = 0; q < 4; ++q) hw[q] = pack_bf16(gelu2(layer1_z(sm.net, f, i0 + 2 * q)));
+            *reinterpret_cast<uint4*>(sm.H1 + tile_offset(t, i0, kTile)) = h;
+        }
         sync_for_mma();
         if (t == 0) {
-            mma_chain(tm + kColD2, sm.H1, kTile, sm.W2, kH, kH, idesc_bf16_f32(kTile, kH), false);
+            mma_chain(tm + kColD2, {smem_u32(sm.H1), kTile, false}, {smem_u32(sm.W2), kH, false}, kH,
+                      idesc_bf16_f32(kTile, kH), false);
             mma_commit(&sm.mbar);
         }
         if (!(ok = wait_all(&sm.mbar, phase))) break;
         // output unit: two partial sums (even and odd hidden units) on the packed pipe
-        float2 y2 = make_float2(sm.b3, 0.0f);
+        float2 y2 = make_float2(sm.net.b3, 0.0f);
 #pragma unroll 1
         for (int c = 0; c < kH; c += 16) {
             float z[16];
             tmem_ld16(tmem_at(tm, warp * 32, kColD2 + c), z);
 #pragma unroll
-            for (int q = 0; q < 16; q += 2) {
-                const float2 b = *reinterpret_cast<const float2*>(&sm.b2[c + q]);
-                const float2 w = *reinterpret_cast<const float2*>(&sm.w3[c + q]);
-                y2 = __ffma2_rn(w, gelu2(__fadd2_rn(make_float2(z[q], z[q + 1]), b)), y2);
+            for (int q = 0; q < 16; q += 4) {
+                const float4 b = *reinterpret_cast<const float4*>(&sm.net.b2[c + q]);
+                const float4 w = *reinterpret_cast<const float4*>(&sm.net.w3[c + q]);
+                float2 ga, gb;
+                gelu4(__fadd2_rn(make_float2(z[q], z[q + 1]), make_float2(b.x, b.y)),
+                      __fadd2_rn(make_float2(z[q + 2], z[q + 3]), make_float2(b.z, b.w)), ga, gb);
+                y2 = __ffma2_rn(make_float2(w.z, w.w), gb, __ffma2_rn(make_float2(w.x, w.y), ga, y2));
             }
         }
         const float y = y2.x + y2.y;
@@ -270,25 +294,46 @@ __global__ void __launch_bounds__(128, 1) k_mlp_forward(const MlpParams P)
 }
 
 // ------------------------------------------------------------- training --
-__global__ void __launch_bounds__(128, 1) k_mlp_grad(const MlpParams P)
+// Four consecutive gradient entries; one 16-byte reduction where aligned.
+__device__ __forceinline__ void add4(float* p, float4 v, bool wide)
+{
+    if (wide) {
+        atomicAdd(reinterpret_cast<float4*>(p), v);
+    } else {
+        atomicAdd(p, v.x);
+        atomicAdd(p + 1, v.y);
+        atomicAdd(p + 2, v.z);
+        atomicAdd(p + 3, v.w);
+    }
+}
+
+// A minibatch is about one tile per CTA, so a step's time is one tile's chain of
+// phases: two threads per sample halve it, each keeping its 32 units' activations
+// and derivatives in registers from the pass that first needs them.
+__global__ void __launch_bounds__(256, 2) k_mlp_grad(const MlpParams P)
 {
     extern __shared__ __align__(1024) unsigned char smem_raw[];
     SmemTrain& sm = *reinterpret_cast<SmemTrain*>(smem_raw);
-    const int t = threadIdx.x, warp = t >> 5, lane = t & 31;
-    stage_weights(sm, P.params, true, sm.W2T);
-    // constant rows: H1T row 64 = 1, rows 65..79 = 0; FT row 3 = 1, rows 4..15 = 0
-    for (int q = t; q < (kRowsH1T - kH) * kTile; q += blockDim.x) {
-        const int r = kH + q / kTile, k = q % kTile;
-        put_bf16(sm.H1T, tile_offset(r, k, kRowsH1T), r == kH ? 1.0f : 0.0f);
+    constexpr int kHalf = kH / 2;
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int quarter = warp & 3, t = quarter * 32 + lane;  // sample of the tile, TMEM lane
+    const int h0 = (warp >> 2) * kHalf;                     // first hidden unit of this thread
+    const bool first = h0 == 0;
+    stage_weights(sm.net, sm.W2, P.params);
+    // constant columns: H1 column 64 = 1, 65..79 = 0; F column 3 = 1, 4..15 = 0
+    if (first) {
+        const uint4 one = make_uint4(0x3f80u, 0u, 0u, 0u), zero = make_uint4(0u, 0u, 0u, 0u);
+        *reinterpret_cast<uint4*>(sm.H1 + tile_offset(t, kH, kTile)) = one;
+        *reinterpret_cast<uint4*>(sm.H1 + tile_offset(t, kH + 8, kTile)) = zero;
+        *reinterpret_cast<uint4*>(sm.F + tile_offset(t, 8, kTile)) = zero;
     }
-    for (int q = t; q < (kRowsFT - 3) * kTile; q += blockDim.x) {
-        const int r = 3 + q / kTile, k = q % kTile;
-        put_bf16(sm.FT, tile_offset(r, k, kRowsFT), r == 3 ? 1.0f : 0.0f);
-    }
-    if (t == 0) mbar_init(&sm.mbar, 1);
+    if (threadIdx.x == 0) mbar_init(&sm.mbar, 1);
     if (warp == 0) tmem_alloc(&sm.tmem, kColsTrain);
     sync_for_mma();
     const uint32_t tm = sm.tmem;
+    const Operand W2{smem_u32(sm.W2), kH, false}, W2t{smem_u32(sm.W2), kH, true};
+    const Operand H1{smem_u32(sm.H1), kTile, false}, H1t{smem_u32(sm.H1), kTile, true};
+    const Operand D{smem_u32(sm.D), kTile, false}, Dt{smem_u32(sm.D), kTile, true}, Ft{smem_u32(sm.F), kTile, true};
     uint32_t phase = 0;
     const long long n_tiles = (P.n + kTile - 1) / kTile;
     bool ok = true, any = false;
@@ -305,71 +350,97 @@ __global__ void __launch_bounds__(128, 1) k_mlp_grad(const MlpParams P)
                 f[0] = f[1] = f[2] = 0.0f;
             }
         }
-        layer1(sm, f, t, sm.H1T);
+        // layer 1
+        float2 dg1[kHalf / 2];
 #pragma unroll
-        for (int k = 0; k < 3; ++k) put_bf16(sm.FT, tile_offset(k, t, kRowsFT), f[k]);
+        for (int i0 = 0; i0 < kHalf; i0 += 8) {
+            uint4 h;
+            unsigned int* hw = reinterpret_cast<unsigned int*>(&h);
+#pragma unroll
+            for (int q = 0; q < 4; ++q) {
+                const Gelu2 a(layer1_z(sm.net, f, h0 + i0 + 2 * q));
+                const float2 g = a.g();
+                hw[q] = pack_bf16(g);
+                dg1[i0 / 2 + q] = a.dg(g);
+            }
+            *reinterpret_cast<uint4*>(sm.H1 + tile_offset(t, h0 + i0, kTile)) = h;
+        }
+        if (first)
+            *reinterpret_cast<uint4*>(sm.F + tile_offset(t, 0, kTile)) =
+                make_uint4(pack_bf16(make_float2(f[0], f[1])), pack_bf16(make_float2(f[2], 1.0f)), 0u, 0u);
         sync_for_mma();
-        if (t == 0) {
-            mma_chain(tm + kColD2, sm.H1, kTile, sm.W2, kH, kH, idesc_bf16_f32(kTile, kH), false);
+        if (threadIdx.x == 0) {
+            mma_chain(tm + kColD2, H1, W2, kH, idesc_bf16_f32(kTile, kH), false);
             mma_commit(&sm.mbar);
         }
         if (!(ok = wait_all(&sm.mbar, phase))) break;
 
-        // forward output (first pass over z2 in tensor memory), then dy
-        float y = sm.b3;
-#pragma unroll 1
-        for (int c = 0; c < kH; c += 16) {
-            float z[16];
-            tmem_ld16(tmem_at(tm, warp * 32, kColD2 + c), z);
+        // forward output, then dy
+        float2 g2[kHalf / 2], dg2[kHalf / 2], y2 = make_float2(0.0f, 0.0f);
 #pragma unroll
-            for (int q = 0; q < 16; ++q) y = fmaf(sm.w3[c + q], gelu(z[q] + sm.b2[c + q]).g, y);
+        for (int c = 0; c < kHalf; c += 16) {
+            float z[16];
+            tmem_ld16(tmem_at(tm, quarter * 32, kColD2 + h0 + c), z);
+#pragma unroll
+            for (int q = 0; q < 16; q += 2) {
+                const float2 b = *reinterpret_cast<const float2*>(&sm.net.b2[h0 + c + q]);
+                const float2 w = *reinterpret_cast<const float2*>(&sm.net.w3[h0 + c + q]);
+                const Gelu2 a(__fadd2_rn(make_float2(z[q], z[q + 1]), b));
+                const float2 g = a.g();
+                y2 = __ffma2_rn(w, g, y2);
+                g2[(c + q) / 2] = g;
+                dg2[(c + q) / 2] = __fmul2_rn(w, a.dg(g));
+            }
         }
+        sm.y[warp >> 2][t] = y2.x + y2.y;
+        __syncthreads();
+        const float y = sm.net.b3 + (sm.y[0][t] + sm.y[1][t]);
         const float r = valid ? y - target : 0.0f;
         const float dy = 2.0f * r;
-        loss = fmaf(r, r, loss);
-        gb3 += dy;
-        // second pass: delta2 = dy w3 g'(z2) into the rows of D2 (K-major by j) and
-        // the columns of D2T, dy h2 into the columns of D2T's rows 64 + j
-#pragma unroll 1
-        for (int c = 0; c < kH; c += 16) {
-            float z[16];
-            tmem_ld16(tmem_at(tm, warp * 32, kColD2 + c), z);
-            __align__(16) __nv_bfloat16 db[16];
+        if (first) {
+            loss = fmaf(r, r, loss);
+            gb3 += dy;
+        }
+        // delta2 = dy w3 g'(z2) and dy h2, row by sample
+        const float2 dy2 = make_float2(dy, dy);
 #pragma unroll
-            for (int q = 0; q < 16; ++q) {
-                const int j = c + q;
-                const Act a = gelu(z[q] + sm.b2[j]);
-                db[q] = __float2bfloat16_rn(dy * sm.w3[j] * a.dg);
-                *reinterpret_cast<__nv_bfloat16*>(sm.D2T + tile_offset(j, t, kTile)) = db[q];
-                put_bf16(sm.D2T, tile_offset(kH + j, t, kTile), dy * a.g);
+        for (int c = 0; c < kHalf; c += 8) {
+            uint4 d, e;
+            unsigned int *dw = reinterpret_cast<unsigned int*>(&d), *ew = reinterpret_cast<unsigned int*>(&e);
+#pragma unroll
+            for (int q = 0; q < 4; ++q) {
+                dw[q] = pack_bf16(__fmul2_rn(dy2, dg2[c / 2 + q]));
+                ew[q] = pack_bf16(__fmul2_rn(dy2, g2[c / 2 + q]));
             }
-            *reinterpret_cast<uint4*>(sm.D2 + tile_offset(t, c, kTile)) = *reinterpret_cast<const uint4*>(db);
-            *reinterpret_cast<uint4*>(sm.D2 + tile_offset(t, c + 8, kTile)) = *reinterpret_cast<const uint4*>(db + 8);
+            *reinterpret_cast<uint4*>(sm.D + tile_offset(t, h0 + c, kTile)) = d;
+            *reinterpret_cast<uint4*>(sm.D + tile_offset(t, kH + h0 + c, kTile)) = e;
         }
         sync_for_mma();
-        if (t == 0) {
-            mma_chain(tm + kColD3, sm.D2, kTile, sm.W2T, kH, kH, idesc_bf16_f32(kTile, kH), false);
-            mma_chain(tm + kColD4, sm.D2T, kTile, sm.H1T, kRowsH1T, kTile, idesc_bf16_f32(kTile, kRowsH1T), any);
+        if (threadIdx.x == 0) {
+            mma_chain(tm + kColD3, D, W2t, kH, idesc_bf16_f32(kTile, kH, false, true), false);
+            mma_chain(tm + kColD4, Dt, H1t, kTile, idesc_bf16_f32(kTile, kColsH1, true, true), any);
             mma_commit(&sm.mbar);
         }
         if (!(ok = wait_all(&sm.mbar, phase))) break;
 
-        // delta1 = (dL/dh1) g'(z1) into the columns of the D2T buffer (rows 0..63)
-#pragma unroll 1
-        for (int c = 0; c < kH; c += 16) {
-            float dh[16];
-            tmem_ld16(tmem_at(tm, warp * 32, kColD3 + c), dh);
+        // delta1 = (dL/dh1) g'(z1) over delta2
 #pragma unroll
-            for (int q = 0; q < 16; ++q) {
-                const int i = c + q;
-                const float z1 =
-                    fmaf(sm.w1[3 * i + 2], f[2], fmaf(sm.w1[3 * i + 1], f[1], fmaf(sm.w1[3 * i], f[0], sm.b1[i])));
-                put_bf16(sm.D2T, tile_offset(i, t, kTile), dh[q] * gelu(z1).dg);
+        for (int c = 0; c < kHalf; c += 16) {
+            float dh[16];
+            tmem_ld16(tmem_at(tm, quarter * 32, kColD3 + h0 + c), dh);
+#pragma unroll
+            for (int q0 = 0; q0 < 16; q0 += 8) {
+                uint4 d;
+                unsigned int* dw = reinterpret_cast<unsigned int*>(&d);
+#pragma unroll
+                for (int q = 0; q < 4; ++q)
+                    dw[q] = pack_bf16(__fmul2_rn(make_float2(dh[q0 + 2 * q], dh[q0 + 2 * q + 1]), dg1[(c + q0) / 2 + q]));
+                *reinterpret_cast<uint4*>(sm.D + tile_offset(t, h0 + c + q0, kTile)) = d;
             }
         }
         sync_for_mma();
-        if (t == 0) {
-            mma_chain(tm + kColD5, sm.D2T, kTile, sm.FT, kRowsFT, kTile, idesc_bf16_f32(kTile, kRowsFT), any);
+        if (threadIdx.x == 0) {
+            mma_chain(tm + kColD5, Dt, Ft, kTile, idesc_bf16_f32(kTile, kColsF, true, true), any);
             mma_commit(&sm.mbar);
         }
         if (!(ok = wait_all(&sm.mbar, phase))) break;
@@ -386,40 +457,54 @@ __global__ void __launch_bounds__(128, 1) k_mlp_grad(const MlpParams P)
             loss += __shfl_xor_sync(0xffffffffu, loss, o);
             gb3 += __shfl_xor_sync(0xffffffffu, gb3, o);
         }
-        if (lane == 0) {
+        if (first && lane == 0) {
             sm.red_loss[warp] = loss;
             sm.red_gb3[warp] = gb3;
         }
         __syncthreads();
-        if (t == 0 && any) {
+        if (threadIdx.x == 0 && any) {
             atomicAdd(P.loss, (sm.red_loss[0] + sm.red_loss[1] + sm.red_loss[2] + sm.red_loss[3]) * inv_n);
             atomicAdd(P.grad + kB3, (sm.red_gb3[0] + sm.red_gb3[1] + sm.red_gb3[2] + sm.red_gb3[3]) * inv_n);
         }
         if (any) {
             // D4 row r < 64: dW2[r][0..63], db2[r] (column 64); row 64 + j: dw3[j] (column 64)
+            const bool wide = (reinterpret_cast<uintptr_t>(P.grad) & 15) == 0;
             float v[16];
 #pragma unroll 1
-            for (int c = 0; c < kH; c += 16) {
-                tmem_ld16(tmem_at(tm, warp * 32, kColD4 + c), v);
+            for (int c = h0; c < h0 + kHalf; c += 16) {
+                tmem_ld16(tmem_at(tm, quarter * 32, kColD4 + c), v);
                 if (t < kH)
 #pragma unroll
-                    for (int q = 0; q < 16; ++q) atomicAdd(P.grad + kW2 + t * kH + c + q, v[q] * inv_n);
+                    for (int q = 0; q < 16; q += 4)
+                        add4(P.grad + kW2 + t * kH + c + q,
+                             make_float4(v[q] * inv_n, v[q + 1] * inv_n, v[q + 2] * inv_n, v[q + 3] * inv_n), wide);
             }
-            tmem_ld16(tmem_at(tm, warp * 32, kColD4 + kH), v);
-            if (t < kH) atomicAdd(P.grad + kB2 + t, v[0] * inv_n);
-            else atomicAdd(P.grad + kW3 + (t - kH), v[0] * inv_n);
-            // D5 row r < 64: dW1[r][0..2], db1[r] (column 3)
-            tmem_ld16(tmem_at(tm, warp * 32, kColD5), v);
-            if (t < kH) {
+            if (first) {
+                tmem_ld16(tmem_at(tm, quarter * 32, kColD4 + kH), v);
+                if (t < kH) atomicAdd(P.grad + kB2 + t, v[0] * inv_n);
+                else atomicAdd(P.grad + kW3 + (t - kH), v[0] * inv_n);
+            } else {
+                // D5 row r < 64: dW1[r][0..2], db1[r] (column 3)
+                tmem_ld16(tmem_at(tm, quarter * 32, kColD5), v);
+                if (t < kH) {
 #pragma unroll
-                for (int k = 0; k < 3; ++k) atomicAdd(P.grad + kW1 + 3 * t + k, v[k] * inv_n);
-                atomicAdd(P.grad + kB1 + t, v[3] * inv_n);
+                    for (int k = 0; k < 3; ++k) atomicAdd(P.grad + kW1 + 3 * t + k, v[k] * inv_n);
+                    atomicAdd(P.grad + kB1 + t, v[3] * inv_n);
+                }
             }
         }
     }
     fence_before_sync();
     __syncthreads();
     if (warp == 0) tmem_dealloc(tm, kColsTrain);
+}
+
+// the sums' start: one launch in place of two memsets
+__global__ void k_mlp_zero(float* __restrict__ grad, int n, float* __restrict__ loss)
+{
+    const int q = blockIdx.x * blockDim.x + threadIdx.x;
+    if (q < n) grad[q] = 0.0f;
+    if (q == 0) *loss = 0.0f;
 }
 
 // ----------------------------------------------------------------- Adam --
@@ -464,17 +549,20 @@ cudaError_t launch_mlp_forward(cudaStream_t s, const MlpParams& P)
     const int sms = sm_count();
     if (sms == 0) return cudaErrorInvalidDevice;
     cudaError_t e = cudaFuncSetAttribute(k_mlp_forward, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemInfer);
+    if (e == cudaSuccess)  // room for all eight CTAs
+        e = cudaFuncSetAttribute(k_mlp_forward, cudaFuncAttributePreferredSharedMemoryCarveout,
+                                 cudaSharedmemCarveoutMaxShared);
     if (e != cudaSuccess) return e;
     const long long tiles = (P.n + kTile - 1) / kTile;
-    const long long grid = tiles < 4LL * sms ? tiles : 4LL * sms;
+    const long long grid = tiles < 8LL * sms ? tiles : 8LL * sms;
     k_mlp_forward<<<(unsigned)grid, 128, kSmemInfer, s>>>(P);
     return cudaGetLastError();
 }
 
 cudaError_t launch_mlp_grad(cudaStream_t s, const MlpParams& P)
 {
-    cudaError_t e = cudaMemsetAsync(P.grad, 0, sizeof(float) * mlp_param_count(), s);
-    if (e == cudaSuccess) e = cudaMemsetAsync(P.loss, 0, sizeof(float), s);
+    k_mlp_zero<<<(mlp_param_count() + 255) / 256, 256, 0, s>>>(P.grad, mlp_param_count(), P.loss);
+    cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess || P.n == 0) return e;
     const int sms = sm_count();
     if (sms == 0) return cudaErrorInvalidDevice;
@@ -482,7 +570,7 @@ cudaError_t launch_mlp_grad(cudaStream_t s, const MlpParams& P)
     if (e != cudaSuccess) return e;
     const long long tiles = (P.n + kTile - 1) / kTile;
     const long long grid = tiles < 2LL * sms ? tiles : 2LL * sms;
-    k_mlp_grad<<<(unsigned)grid, 128, kSmemTrain, s>>>(P);
+    k_mlp_grad<<<(unsigned)grid, 256, kSmemTrain, s>>>(P);
     return cudaGetLastError();
 }
 

@@ -2,13 +2,17 @@
 // allocation, single-thread MMA issue, commit to an mbarrier, bounded mbarrier
 // waits and tensor-memory loads, as inline PTX.
 //
-// Operand layout used by every MMA here: BF16, K-major, no swizzle.  An R x K
-// tile (R a multiple of 8, K a multiple of 16) is stored as K/16 blocks of one
-// MMA K-step each; inside a block the 8-row groups are 256 B apart, the two
-// 8-element K halves of a group are 128 B apart (two 8 x 16 B core matrices),
-// and a core matrix row is 16 B.  So the shared-memory descriptor of a K-step
-// has leading (K-direction) byte offset 128 and stride (row-direction) byte
-// offset 256, and block s starts s * R/8 * 256 bytes after the tile.
+// Operand layout used by every MMA here: BF16, no swizzle.  An R x K tile (R and K
+// multiples of 8) is stored by column groups of 8: group k / 8 starts R * 16 bytes
+// after the one before; inside it row r takes 16 bytes (its 8 columns), so 8 x 8
+// core matrices of 128 bytes follow each other down the rows.  A thread that owns a
+// row writes 16-byte pieces next to its neighbours', free of bank conflicts.
+// The same tile serves the tensor core two ways:
+//  * K-major, rows = M or N, columns = K: K-direction core matrices are R * 16 bytes
+//    apart (leading offset), row-direction ones 128 bytes (stride offset);
+//  * MN-major, columns = M or N, rows = K: M/N-direction core matrices are R * 16
+//    bytes apart (stride offset), K-direction ones 128 bytes (leading offset) --
+//    the transposed operand, with no transposed copy.
 #pragma once
 
 #include <cstdint>
@@ -18,32 +22,42 @@ namespace dex {
 namespace umma {
 
 // byte offset of element (r, k) in an R-row tile
-__host__ __device__ __forceinline__ int tile_offset(int r, int k, int R)
+__host__ __device__ __forceinline__ constexpr int tile_offset(int r, int k, int R)
 {
-    return (k >> 4) * (R >> 3) * 256 + (r >> 3) * 256 + ((k >> 3) & 1) * 128 + (r & 7) * 16 + (k & 7) * 2;
+    return (k >> 3) * R * 16 + r * 16 + (k & 7) * 2;
 }
-
-// bytes of one K-step block of an R-row tile
-__host__ __device__ constexpr int kstep_bytes(int R) { return (R >> 3) * 256; }
 
 __device__ __forceinline__ uint32_t smem_u32(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
 
 // shared-memory matrix descriptor: start address, leading / stride byte
 // offsets (all >> 4), the fixed version bit 46, no swizzle, base offset 0
-__device__ __forceinline__ uint64_t smem_desc(uint32_t addr)
+__device__ __forceinline__ uint64_t smem_desc(uint32_t addr, uint32_t leading, uint32_t stride)
 {
     uint64_t d = (uint64_t)((addr & 0x3FFFFu) >> 4);
-    d |= (uint64_t)(128u >> 4) << 16;
-    d |= (uint64_t)(256u >> 4) << 32;
+    d |= (uint64_t)(leading >> 4) << 16;
+    d |= (uint64_t)(stride >> 4) << 32;
     d |= 1ull << 46;
     return d;
 }
 
-// instruction descriptor of kind::f16: F32 accumulator, BF16 A and B, both
-// K-major, dense, M x N
-__host__ __device__ constexpr uint32_t idesc_bf16_f32(int M, int N)
+// One operand: its tile's shared-memory address and rows R, and which way it is read.
+struct Operand {
+    uint32_t addr;
+    uint32_t R;
+    bool mn_major;
+    // K-step s (16 values of K)
+    __device__ __forceinline__ uint64_t step(int s) const
+    {
+        return mn_major ? smem_desc(addr + s * 256u, 128u, R * 16u) : smem_desc(addr + s * 32u * R, R * 16u, 128u);
+    }
+};
+
+// instruction descriptor of kind::f16: F32 accumulator, BF16 A and B, dense, M x N;
+// bits 15 and 16 mark MN-major A and B
+__host__ __device__ constexpr uint32_t idesc_bf16_f32(int M, int N, bool a_mn = false, bool b_mn = false)
 {
-    return (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(N >> 3) << 17) | ((uint32_t)(M >> 4) << 24);
+    return (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)a_mn << 15) | ((uint32_t)b_mn << 16) |
+           ((uint32_t)(N >> 3) << 17) | ((uint32_t)(M >> 4) << 24);
 }
 
 // ---- tensor memory (executed by one full warp) ----
@@ -68,7 +82,7 @@ __device__ __forceinline__ void fence_after_sync() { asm volatile("tcgen05.fence
 __device__ __forceinline__ void fence_async_smem() { asm volatile("fence.proxy.async.shared::cta;" ::: "memory"); }
 
 // ---- MMA issue and completion (one thread) ----
-// D[tmem] (+)= A[smem] * B[smem]^T, both operands K-major
+// D[tmem] (+)= A[smem] * B[smem]^T, operands as their descriptors and idesc say
 __device__ __forceinline__ void mma_bf16(uint32_t d_tmem, uint64_t a_desc, uint64_t b_desc, uint32_t idesc,
                                          bool accumulate)
 {
