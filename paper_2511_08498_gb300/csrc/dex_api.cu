@@ -83,6 +83,7 @@ int fill_quadrature(dex_ctx* ctx, int n_dir, const float* dirs, const float* wei
 
 constexpr double kH_ = 6.62607015e-27;
 constexpr double kC_ = 2.99792458e10;
+constexpr double kKB_ = 1.380649e-16;
 
 // Validate the atom and the wavelength samples; fill the launch parameters
 // (frequencies, per-line trapezoid weights in frequency, Einstein B).
@@ -136,6 +137,19 @@ int fill_atom(dex_ctx* ctx, const dex_atom* atom, int n_lambda, const double* la
             P.wq[idx[a + 1]] += 0.5 * h;
         }
     }
+    short n = 0;
+    for (int l = 0; l <= atom->n_line; ++l) {
+        P.first[l] = n;
+        for (int k = 0; k < n_lambda; ++k)
+            if (line_tag[k] == (l < atom->n_line ? l : -1)) P.order[n++] = (short)k;
+    }
+    for (int k = 0; k < n_lambda; ++k) {
+        P.off[k] = line_tag[k] >= 0 ? P.nu[k] - P.nu0[line_tag[k]] : 0.0;
+        P.bx[k] = kH_ * P.nu[k] / kKB_;
+        P.by[k] = P.bx[k] * (256.0 / M_LN2);
+        P.bc[k] = 2.0 * kH_ * P.nu[k] * P.nu[k] * P.nu[k] / (kC_ * kC_);
+    }
+    for (int j = 0; j < 256; ++j) P.exp_table[j] = std::exp2(j / 256.0);
     return DEX_OK;
 }
 

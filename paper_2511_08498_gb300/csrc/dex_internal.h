@@ -150,6 +150,15 @@ struct AtomParams {
     double nu[DEX_MAX_ATOM_LAMBDA];    // sample frequencies (Hz)
     double wq[DEX_MAX_ATOM_LAMBDA];    // trapezoid weight in frequency within the sample's line
     signed char tag[DEX_MAX_ATOM_LAMBDA];
+    // samples grouped by line (line li: order[first[li]] .. order[first[li + 1] - 1]),
+    // those without a line last, up to n_lambda
+    short order[DEX_MAX_ATOM_LAMBDA];
+    short first[DEX_MAX_LINES + 1];
+    double off[DEX_MAX_ATOM_LAMBDA];   // nu - nu0 of the sample's line
+    double bx[DEX_MAX_ATOM_LAMBDA];    // h nu / k (K)
+    double by[DEX_MAX_ATOM_LAMBDA];    // the same in units of ln2 / 256
+    double bc[DEX_MAX_ATOM_LAMBDA];    // 2 h nu^3 / c^2
+    double exp_table[256];             // 2^(j / 256)
     double nu0[DEX_MAX_LINES];
     double b_ul[DEX_MAX_LINES];
     double b_lu[DEX_MAX_LINES];
