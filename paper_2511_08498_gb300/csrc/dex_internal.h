@@ -330,17 +330,21 @@ struct RcParams {
     int spacing, pnx, pnz, n_dir, level_cap;  // this cascade: probe lattice, directions, MIP cap
     int dir_fastest;                           // thread order: directions (1) or probes (0) fastest
     int paired, pair_group;                    // W = 8: one walk per pair of batches (pair_batches)
+    int siblings;                              // sibling directions in neighbouring lanes: 4, or 1
+    float* J;                                  // cascade 0 of four directions: their mean goes here, else nullptr
+    const float* bounds;                       // the batches' bounds of the early termination, or nullptr
     float t_s, t_e, i_bc;                      // radiance interval, boundary intensity
     const float* bricks;
     const unsigned long long* words;
     const int* block_offset;
     const float* dirs;                         // [n_dir][2] of this cascade
-    const float* upper;                        // merged radiance of the cascade above, or nullptr
-    float* out;                                // [n_batch][n_dir][pnz * pnx][W] merged radiance
+    const float* upper;                        // sums over siblings of the cascade above, or nullptr
+    float* out;                                // [n_batch][n_dir / siblings][pnz * pnx][W] merged radiance
     unsigned long long* seg_count;
     unsigned int* status;
 };
 cudaError_t launch_rc_cascade(cudaStream_t s, const RcParams& P);
+cudaError_t launch_rc_scan(cudaStream_t s, const RcParams& P, float* scratch, const float** bounds);
 cudaError_t launch_rc_mean(cudaStream_t s, const RcParams& P, const float* L0, float* J);
 
 // ------------------------------------------------------------------- 3D --
@@ -387,6 +391,7 @@ struct Hdda3Params {
     int nx, ny, nz, nbx, nby, nbz, n_lambda, W, n_batch, max_mip, chain, n_words, cap_active, storage;
     int traversal;  // DEX_TRAVERSAL_PAIRED: one walk per pair of batches; otherwise one per batch
     int pair_group; // batches paired within groups of this many (0: one group), as HddaParams
+    int scanned;    // J holds the bounds of the exact early termination, as HddaParams
     int n_band;
     float band[4];
     long long n_cells;

@@ -9,19 +9,25 @@
 //   on the top cascade), else the bilinear interpolation at this probe of the
 //   mean over the 4 child directions (4k .. 4k+3) of the cascade above (its 4
 //   nearest probes, indices clamped at the lattice edge).
-// Thread = (direction, probe) of one wavelength batch.  On the lower cascades
-// probes run fastest, so the lanes of a warp trace parallel rays from
+// Thread = (direction, probe) of one wavelength batch, the four siblings 4k .. 4k+3
+// of a direction in neighbouring lanes.  A cascade hands down the sum over the
+// siblings, added in their order by shuffles, so the cascade below reads 4 values
+// per ray and wavelength instead of 16 and a quarter of the radiance is stored (the
+// 16 scalar reads kept the lower cascades at 85% of the L1 data pipe).  Cascade 0
+// likewise adds its directions into J where there are four; otherwise it stores
+// them and a final kernel averages.  On the lower cascades a warp holds eight
 // neighbouring probes; on the upper ones (long intervals from probes 16 or more
-// cells apart) directions run fastest, so a warp's rays fan out from one probe
-// and read neighbouring bricks.  Cascade 0 skips
-// probes in empty blocks (J is not defined there).  A final kernel averages the
-// cascade-0 radiance over its directions into J.
+// cells apart) 32 neighbouring directions of one probe, whose rays fan out and read
+// neighbouring bricks.  CTAs of 64 threads: a warp's rays end together, those of a
+// 256-thread CTA did not, and its finished warps held their registers (10 of 16
+// resident warps active on the long cascades).  Cascade 0 skips probes in empty
+// blocks (J is not defined there).
 //
 // The tracer starts at t_s: the entry cell is floor(p(t_s)) (a rounding that
 // lands in the next cell back only yields a zero-length first step), plane
 // offsets from the probe are exact (probes sit at multiples of 1/2), and the
 // last segment is clipped at min(t_e, grid exit).
-#include "dex_internal.h"
+#include "scan.cuh"
 
 namespace dex {
 
@@ -53,8 +59,8 @@ template <int W, bool COUNT, int ST, int NB = 1>
 __device__ __forceinline__ bool rc_interval(const RcParams& P, const float* __restrict__ base, long long off,
                                             const unsigned long long* __restrict__ words,
                                             const unsigned long long* __restrict__ words2, float ox, float oz,
-                                            float dx, float dz, float* I, float* T, unsigned int& nseg,
-                                            bool& capped)
+                                            float dx, float dz, float stop, float* I, float* T,
+                                            unsigned int& nseg, bool& capped)
 {
     using BF = BrickFmt<W, ST>;
     constexpr int REC = BF::kRec;
@@ -118,7 +124,6 @@ __device__ __forceinline__ bool rc_interval(const RcParams& P, const float* __re
                 rp += negz ? -side * REC : side * REC;
                 cross = (unsigned)lz >= (unsigned)side;
             }
-            if (cross && all_opaque<NB * W>(T)) break;  // the rest adds exact zeros
             if (cross) {
                 const int bxn = bxc + (on_x ? sx : 0), bzn = bzc + (on_x ? 0 : sz);
                 if ((unsigned)bxn >= (unsigned)P.nbx || (unsigned)bzn >= (unsigned)P.nbz) {
@@ -165,97 +170,159 @@ __device__ __forceinline__ bool rc_interval(const RcParams& P, const float* __re
             if constexpr (NB == 2) segments<W>(r2.S, r2.chi, len * kNegLog2e, I + W, T + W);
             if (COUNT) nseg += NB * (th > th_prev);
         }
-        if (last) break;
+        // the rest changes no bit of the radiance
+        if (last || ((it & 3) == 3 && ray_done<NB * W>(I, T, stop))) break;
         th_prev = th;
         tl_prev = tl;
     }
     return left;
 }
 
+constexpr int kRcThreads = 64;
+
+// W consecutive floats, 16-byte aligned for W >= 4
+template <int W>
+__device__ __forceinline__ void load_w(const float* __restrict__ p, float* v)
+{
+    if constexpr (W >= 4) {
+#pragma unroll
+        for (int w = 0; w < W; w += 4) {
+            const float4 a = __ldg(reinterpret_cast<const float4*>(p + w));
+            v[w] = a.x; v[w + 1] = a.y; v[w + 2] = a.z; v[w + 3] = a.w;
+        }
+    } else {
+#pragma unroll
+        for (int w = 0; w < W; ++w) v[w] = __ldg(p + w);
+    }
+}
+
+template <int W>
+__device__ __forceinline__ void store_w(float* __restrict__ p, const float* v)
+{
+    if constexpr (W >= 4) {
+#pragma unroll
+        for (int w = 0; w < W; w += 4)
+            *reinterpret_cast<float4*>(p + w) = make_float4(v[w], v[w + 1], v[w + 2], v[w + 3]);
+    } else {
+#pragma unroll
+        for (int w = 0; w < W; ++w) p[w] = v[w];
+    }
+}
+
+// ((s0 + s1) + s2) + s3 over four neighbouring lanes, in the first of them
+__device__ __forceinline__ float sibling_sum(float v)
+{
+    const float s1 = __shfl_down_sync(0xffffffffu, v, 1), s2 = __shfl_down_sync(0xffffffffu, v, 2),
+                s3 = __shfl_down_sync(0xffffffffu, v, 3);
+    return ((v + s1) + s2) + s3;
+}
+
 // NB = 1: blockIdx.y is the batch (with P.paired: the lone batch
 // pair_lone_batch(blockIdx.y)); NB = 2: the pair pair_batches(blockIdx.y), one
 // walk for both batches on the smaller of their levels.
 template <int W, bool COUNT, int ST, int NB>
-__global__ void __launch_bounds__(256, NB == 1 ? 4 : 2) k_rc_cascade(const RcParams P)
+__global__ void __launch_bounds__(kRcThreads, (NB == 1 ? 1024 : 512) / kRcThreads) k_rc_cascade(const RcParams P)
 {
     int b = blockIdx.y, b2 = blockIdx.y;
     if constexpr (NB == 2) pair_batches(blockIdx.y, P.n_batch, P.pair_group, b, b2);
     else if (P.paired) b = b2 = pair_lone_batch(blockIdx.y, P.n_batch, P.pair_group);
     const long long g = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     const long long n_probe = (long long)P.pnx * P.pnz;
-    if (g >= n_probe * P.n_dir) return;
-    int k, p;
+    // rays come in groups of `sib` sibling lanes (4, or 1 on a cascade 0 of other than
+    // four directions per group of lanes): group q, ray s of it
+    const int sib = P.siblings, s = sib == 4 ? (int)(g & 3) : 0;
+    const long long q = sib == 4 ? g >> 2 : g;
+    const int n_group = P.n_dir / sib;
+    bool live = g < n_probe * P.n_dir;
+    int j, p;
     if (P.dir_fastest) {  // lanes: neighbouring directions of one probe
-        p = (int)(g / P.n_dir);
-        k = (int)(g - (long long)p * P.n_dir);
-    } else {              // lanes: neighbouring probes, one direction
-        k = (int)(g / n_probe);
-        p = (int)(g - (long long)k * n_probe);
+        p = (int)(q / n_group);
+        j = (int)(q - (long long)p * n_group);
+    } else {              // lanes: neighbouring probes
+        j = (int)(q / n_probe);
+        p = (int)(q - (long long)j * n_probe);
     }
+    const int k = j * sib + s;
     const int px = p % P.pnx, pz = p / P.pnx;
     const unsigned long long* words = P.words + (size_t)b * P.n_words;
     const unsigned long long* words2 = P.words + (size_t)b2 * P.n_words;
-    if (P.spacing == 1) {  // cascade 0: probes only in non-empty blocks
-        if (rc_block_state(words, (pz >> 4) * P.nbx + (px >> 4)) == 0) return;
-    }
+    if (live && P.spacing == 1)  // cascade 0: probes only in non-empty blocks
+        live = rc_block_state(words, (pz >> 4) * P.nbx + (px >> 4)) != 0;
     constexpr int REC = RecFmt<W, ST>::kStride;
     const size_t batch_floats = (size_t)P.cap_active * P.chain * REC;
     const float* base = P.bricks + (size_t)b * batch_floats;
     const long long off = (long long)(b2 - b) * (long long)batch_floats;
     const float ox = (float)P.spacing * ((float)px + 0.5f), oz = (float)P.spacing * ((float)pz + 0.5f);
-    const float dx = P.dirs[2 * k], dz = P.dirs[2 * k + 1];
     float I[NB * W], T[NB * W];
 #pragma unroll
     for (int w = 0; w < NB * W; ++w) { I[w] = 0.0f; T[w] = 1.0f; }
     unsigned int nseg = 0;
-    bool capped = false;
-    const bool left = rc_interval<W, COUNT, ST, NB>(P, base, off, words, words2, ox, oz, dx, dz, I, T, nseg, capped);
+    bool capped = false, left = true;
+    if (live) {
+        // the merged radiance above is bounded as the emission and the boundary are
+        float stop = -1.0f;
+        if (!COUNT && P.bounds != nullptr) {
+            float m = __ldg(P.bounds + b);
+            if (NB == 2) m = join_bounds(m, __ldg(P.bounds + b2));
+            stop = stop_factor(m, P.i_bc);
+        }
+        left = rc_interval<W, COUNT, ST, NB>(P, base, off, words, words2, ox, oz, P.dirs[2 * k], P.dirs[2 * k + 1], stop,
+                                             I, T, nseg, capped);
+    }
 
 #pragma unroll
-    for (int q = 0; q < NB; ++q) {
-    const int bq = q == 0 ? b : b2;
-    float R[W];
+    for (int h = 0; h < NB; ++h) {
+        const int bq = h == 0 ? b : b2;
+        float R[W];
 #pragma unroll
-    for (int w = 0; w < W; ++w) R[w] = P.i_bc;
-    if (!left && P.upper != nullptr) {
-        // bilinear stencil on the coarser lattice: this probe sits at (p + 1/2)/2 - 1/2
-        const int qnx = P.pnx >> 1, qnz = P.pnz >> 1;
-        const float ux = 0.5f * ((float)px + 0.5f) - 0.5f, uz = 0.5f * ((float)pz + 0.5f) - 0.5f;
-        const int x0 = (int)floorf(ux), z0 = (int)floorf(uz);
-        const float fx = ux - (float)x0, fz = uz - (float)z0;
-        const int xa = min(max(x0, 0), qnx - 1), xb = min(max(x0 + 1, 0), qnx - 1);
-        const int za = min(max(z0, 0), qnz - 1), zb = min(max(z0 + 1, 0), qnz - 1);
-        const long long q_probe = (long long)qnx * qnz;
-        const float* up = P.upper + (size_t)bq * (size_t)(4 * P.n_dir) * q_probe * W;
-        const int qs[4] = {za * qnx + xa, za * qnx + xb, zb * qnx + xa, zb * qnx + xb};
-        const float ws[4] = {(1.0f - fz) * (1.0f - fx), (1.0f - fz) * fx, fz * (1.0f - fx), fz * fx};
+        for (int w = 0; w < W; ++w) R[w] = P.i_bc;
+        if (!left && P.upper != nullptr) {
+            // bilinear stencil on the coarser lattice: this probe sits at (p + 1/2)/2 - 1/2
+            const int qnx = P.pnx >> 1, qnz = P.pnz >> 1;
+            const float ux = 0.5f * ((float)px + 0.5f) - 0.5f, uz = 0.5f * ((float)pz + 0.5f) - 0.5f;
+            const int x0 = (int)floorf(ux), z0 = (int)floorf(uz);
+            const float fx = ux - (float)x0, fz = uz - (float)z0;
+            const int xa = min(max(x0, 0), qnx - 1), xb = min(max(x0 + 1, 0), qnx - 1);
+            const int za = min(max(z0, 0), qnz - 1), zb = min(max(z0 + 1, 0), qnz - 1);
+            const long long q_probe = (long long)qnx * qnz;
+            // sums over the four child directions 4k .. 4k + 3
+            const float* up = P.upper + ((size_t)bq * P.n_dir + k) * q_probe * W;
+            const int qs[4] = {za * qnx + xa, za * qnx + xb, zb * qnx + xa, zb * qnx + xb};
+            const float ws[4] = {(1.0f - fz) * (1.0f - fx), (1.0f - fz) * fx, fz * (1.0f - fx), fz * fx};
 #pragma unroll
-        for (int w = 0; w < W; ++w) R[w] = 0.0f;
+            for (int w = 0; w < W; ++w) R[w] = 0.0f;
 #pragma unroll
-        for (int c = 0; c < 4; ++c) {
-            float m[W];
+            for (int c = 0; c < 4; ++c) {
+                float m[W];
+                load_w<W>(up + (size_t)qs[c] * W, m);
 #pragma unroll
-            for (int w = 0; w < W; ++w) m[w] = 0.0f;
-#pragma unroll
-            for (int s = 0; s < 4; ++s) {
-                const float* src = up + ((size_t)(4 * k + s) * q_probe + qs[c]) * W;
-#pragma unroll
-                for (int w = 0; w < W; ++w) m[w] += __ldg(src + w);
+                for (int w = 0; w < W; ++w) R[w] = fmaf(ws[c] * 0.25f, m[w], R[w]);
             }
-#pragma unroll
-            for (int w = 0; w < W; ++w) R[w] = fmaf(ws[c] * 0.25f, m[w], R[w]);
         }
-    }
-    float* dst = P.out + ((size_t)bq * (size_t)P.n_dir * n_probe + (size_t)k * n_probe + p) * W;
+        float L[W];
 #pragma unroll
-    for (int w = 0; w < W; ++w) dst[w] = fmaf(T[q * W + w], R[w], I[q * W + w]);
+        for (int w = 0; w < W; ++w) L[w] = fmaf(T[h * W + w], R[w], I[h * W + w]);
+        if (sib == 4) {
+#pragma unroll
+            for (int w = 0; w < W; ++w) L[w] = sibling_sum(L[w]);
+        }
+        if (!live || s != 0) continue;
+        if (P.J != nullptr) {  // cascade 0 of four directions: J is their mean
+#pragma unroll
+            for (int w = 0; w < W; ++w) {
+                const int l = bq * W + w;
+                if (l < P.n_lambda) P.J[(size_t)l * n_probe + p] = L[w] * 0.25f;
+            }
+        } else {
+            store_w<W>(P.out + (((size_t)bq * n_group + j) * n_probe + p) * W, L);
+        }
     }
     if (capped) raise_status(P.status, DEX_ERR_TRAVERSAL_CAP);
     if (COUNT && P.seg_count != nullptr) atomicAdd(P.seg_count, (unsigned long long)nseg);
 }
 
 // J at every cell of every non-empty block: the mean of the cascade-0 radiance
-// over its n0 directions
+// over its n0 directions (n0 other than four)
 template <int W>
 __global__ void __launch_bounds__(256) k_rc_mean(const RcParams P, const float* __restrict__ L0, float* __restrict__ J)
 {
@@ -280,14 +347,35 @@ __global__ void __launch_bounds__(256) k_rc_mean(const RcParams P, const float* 
     }
 }
 
+// Bounds of the exact early termination, in a part of the workspace that the
+// cascades leave free: every block's of every batch, then the batches'.
+template <int W, int ST>
+__global__ void __launch_bounds__(128) k_rc_scan(const RcParams P, float* __restrict__ parts)
+{
+    const int blk = blockIdx.x, b = blockIdx.y, a = P.block_offset[blk];
+    float m = 0.0f;
+    if (a >= 0 && a < P.cap_active)
+        m = join_cta(chain_bound<W, ST>(P.bricks + ((size_t)b * P.cap_active + a) * P.chain * RecFmt<W, ST>::kStride, P.chain));
+    if (threadIdx.x == 0) parts[(size_t)b * P.nbx * P.nbz + blk] = m;
+}
+
+__global__ void __launch_bounds__(1024) k_rc_bound(int n_blocks, const float* __restrict__ parts,
+                                                   float* __restrict__ bounds)
+{
+    float m = 0.0f;
+    for (int q = threadIdx.x; q < n_blocks; q += blockDim.x) m = join_bounds(m, parts[(size_t)blockIdx.x * n_blocks + q]);
+    m = join_cta(m);
+    if (threadIdx.x == 0) bounds[blockIdx.x] = m;
+}
+
 template <int W, int ST, int NB>
 void launch_rc_nb(cudaStream_t s, const RcParams& P, int n_units)
 {
     if (n_units == 0) return;
     const long long n = (long long)P.pnx * P.pnz * P.n_dir;
-    const dim3 grid((unsigned)((n + 255) / 256), (unsigned)n_units);
-    if (P.seg_count) k_rc_cascade<W, true, ST, NB><<<grid, 256, 0, s>>>(P);
-    else k_rc_cascade<W, false, ST, NB><<<grid, 256, 0, s>>>(P);
+    const dim3 grid((unsigned)((n + kRcThreads - 1) / kRcThreads), (unsigned)n_units);
+    if (P.seg_count) k_rc_cascade<W, true, ST, NB><<<grid, kRcThreads, 0, s>>>(P);
+    else k_rc_cascade<W, false, ST, NB><<<grid, kRcThreads, 0, s>>>(P);
 }
 
 template <int W, int ST>
@@ -318,6 +406,26 @@ cudaError_t launch_rc_cascade(cudaStream_t s, const RcParams& P)
         case 8 * 4 + kStoreF16: launch_rc_w<8, kStoreF16>(s, P); break;
         default: return cudaErrorInvalidValue;
     }
+    return cudaGetLastError();
+}
+
+cudaError_t launch_rc_scan(cudaStream_t s, const RcParams& P, float* scratch, const float** bounds)
+{
+    if (P.n_batch == 0) return cudaSuccess;
+    const int nb = P.nbx * P.nbz;
+    float* out = scratch + (size_t)nb * P.n_batch;
+    const dim3 grid((unsigned)nb, (unsigned)P.n_batch);
+    switch (P.W * 4 + P.storage) {
+        case 1 * 4 + kStoreF32: k_rc_scan<1, kStoreF32><<<grid, 128, 0, s>>>(P, scratch); break;
+        case 2 * 4 + kStoreF32: k_rc_scan<2, kStoreF32><<<grid, 128, 0, s>>>(P, scratch); break;
+        case 4 * 4 + kStoreF32: k_rc_scan<4, kStoreF32><<<grid, 128, 0, s>>>(P, scratch); break;
+        case 8 * 4 + kStoreF32: k_rc_scan<8, kStoreF32><<<grid, 128, 0, s>>>(P, scratch); break;
+        case 8 * 4 + kStoreBF16: k_rc_scan<8, kStoreBF16><<<grid, 128, 0, s>>>(P, scratch); break;
+        case 8 * 4 + kStoreF16: k_rc_scan<8, kStoreF16><<<grid, 128, 0, s>>>(P, scratch); break;
+        default: return cudaErrorInvalidValue;
+    }
+    k_rc_bound<<<(unsigned)P.n_batch, 1024, 0, s>>>(nb, scratch, out);
+    *bounds = out;
     return cudaGetLastError();
 }
 
