@@ -2,8 +2,8 @@
 // (Section 2.3, Algorithm 1; the paper's adapted grid generalises directly to
 // 3D with 8^3 blocks and levels 0..3).
 //
-// One CTA per (active block, wavelength batch); each thread takes probe cells of
-// the 8^3 block in turn, walking every quadrature direction.  The packed 3-bit block
+// Two CTAs per (active block, wavelength batch), one thread per probe cell of the 8^3
+// block, walking every quadrature direction.  The packed 3-bit block
 // states of the batch are staged in shared memory when they fit (else read
 // through L1 from global memory).
 //
@@ -23,7 +23,7 @@
 // exit plane sets DEX_ERR_TRAVERSAL_CAP.  (Clipping rays to the box around the
 // non-empty blocks, as the 2D solver does, bought nothing on the 256^3 workload
 // once the box had to be found in every CTA.)
-#include "dex_internal.h"
+#include "scan.cuh"
 
 namespace dex {
 
@@ -34,9 +34,12 @@ constexpr int kCells3 = B3 * B3 * B3;
 // threads per CTA and the CTAs per SM the register budget targets
 constexpr int kThreads3 = 256;
 constexpr int kMinBlocks3 = 3;
+constexpr int kParts3 = kCells3 / kThreads3;  // CTAs per block
 // state words staged in shared memory up to this many (64 KB); larger grids
 // read them from global memory
 constexpr int kMaxStagedWords = 8192;
+// grids of at most this many blocks stage one word per block instead (32 KB)
+constexpr int kMaxInfo3 = 8192;
 
 __host__ __device__ constexpr int level_offset3(int m) { return 585 - (585 >> (3 * m)); }
 
@@ -69,11 +72,14 @@ __device__ __forceinline__ int distance_cap3(const Hdda3Params& P, float t)
 // NB = 2: the ray carries two wavelength batches whose bricks lie `off` floats
 // apart (I, T of 2 W wavelengths, the second batch's from index W); both are
 // integrated over every voxel of the walk.
-template <int W, bool COUNT, int ST, int NB = 1>
+//
+// INFO: block look-ups read one staged word per block, offset * 8 + state (info);
+// otherwise the packed states (words) and the global offset table.
+template <int W, bool COUNT, int ST, int NB, bool INFO>
 __device__ __forceinline__ void trace_ray3(const Hdda3Params& P, const float* __restrict__ base, long long off,
                                            int i, int j, int k, int bx0, int by0, int bz0, int a0, int mip0, float dx,
-                                           float dy, float dz, const unsigned long long* words, float* I, float* T,
-                                           unsigned int& nseg, bool& capped)
+                                           float dy, float dz, const unsigned long long* words, const int* info,
+                                           float stop, float* I, float* T, unsigned int& nseg, bool& capped)
 {
     constexpr int REC = RecFmt<W, ST>::kStride;
     const float ox = (float)i + 0.5f, oy = (float)j + 0.5f, oz = (float)k + 0.5f;
@@ -139,13 +145,12 @@ __device__ __forceinline__ void trace_ray3(const Hdda3Params& P, const float* __
             segments<W>(r2.S, r2.chi, nl2, I + W, T + W);
         }
         if (COUNT) nseg += (cur_mip >= 0) & (th > th_prev);
-        if (last) break;
+        // early termination, tested every fourth step by all lanes together: the rest of
+        // the ray changes no bit of I
+        if (last || ((it & 3) == 3 && ray_done<NB * W>(I, T, stop))) break;
         th_prev = th;
         tl_prev = tl;
         if (cross) {  // entered another block
-            // early termination: once every transmission is exactly zero the rest of
-            // the ray adds exact zeros (bit-identical)
-            if (all_opaque<NB * W>(T)) break;
             const int bxn = bxc + (axis == 0 ? sx : 0), byn = byc + (axis == 1 ? sy : 0),
                       bzn = bzc + (axis == 2 ? sz : 0);
             if ((unsigned)bxn >= (unsigned)P.nbx || (unsigned)byn >= (unsigned)P.nby ||
@@ -154,7 +159,8 @@ __device__ __forceinline__ void trace_ray3(const Hdda3Params& P, const float* __
                 break;
             }
             const int blk = (bzn * P.nby + byn) * P.nbx + bxn;
-            const int st = block_state3(words, blk) - 1;
+            const int key = INFO ? info[blk] : 0;
+            const int st = (INFO ? key & 7 : block_state3(words, blk)) - 1;
             const int mip_new = st < 0 ? -1 : min(st, distance_cap3(P, th));
             if (mip_new == mip) {
                 if (axis == 0) lx = negx ? side - 1 : 0;
@@ -185,7 +191,7 @@ __device__ __forceinline__ void trace_ray3(const Hdda3Params& P, const float* __
             bxc = bxn;
             byc = byn;
             bzc = bzn;
-            rp = mip >= 0 ? base + ((size_t)P.block_offset[blk] * P.chain + level_offset3(mip) +
+            rp = mip >= 0 ? base + ((size_t)(INFO ? key >> 3 : P.block_offset[blk]) * P.chain + level_offset3(mip) +
                                     (lz * side + ly) * side + lx) * REC
                           : g_zero_record3;
             if constexpr (NB == 2) rp2 = mip >= 0 ? rp + off : g_zero_record3;
@@ -207,22 +213,31 @@ __device__ __forceinline__ unsigned long long min_states(unsigned long long a, u
     return m;
 }
 
-// NB = 1: one CTA per (active block, wavelength batch).  NB = 2: one CTA per
+// NB = 1: two CTAs per (active block, wavelength batch).  NB = 2: two CTAs per
 // (active block, pair of batches, pair_batches), walking once for both on the
 // smaller of their levels (the state words must fit in shared memory).
-template <int W, bool COUNT, int ST, int NB>
+// INFO: the CTA stages one word per block (grids of at most kMaxInfo3 blocks).
+template <int W, bool COUNT, int ST, int NB, bool INFO>
 __global__ void __launch_bounds__(kThreads3, NB == 1 ? kMinBlocks3 : 2) k_solve_hdda3(const Hdda3Params P)
 {
     extern __shared__ unsigned long long s_words[];
     __shared__ float s_J3[NB == 2 ? 2 * W : 1][kThreads3];
-    const int a0 = blockIdx.x;
+    const int a0 = blockIdx.x / kParts3, part = blockIdx.x - a0 * kParts3;
     if (a0 >= *P.n_active) return;
     int b = blockIdx.y, b2 = b;
     if constexpr (NB == 2) pair_batches(blockIdx.y, P.n_batch, P.pair_group, b, b2);
     const int tid = threadIdx.x;
     const unsigned long long* gw = P.words + (size_t)b * P.n_words;
-    const bool staged = NB == 2 || P.n_words <= kMaxStagedWords;
-    if (staged) {
+    int* s_info = reinterpret_cast<int*>(s_words);
+    const bool staged = !INFO && (NB == 2 || P.n_words <= kMaxStagedWords);
+    if constexpr (INFO) {
+        const unsigned long long* gw2 = P.words + (size_t)b2 * P.n_words;
+        for (int q = tid; q < P.nbx * P.nby * P.nbz; q += kThreads3) {
+            const int st = block_state3(gw, q);
+            s_info[q] = pack_block_info(P.block_offset[q], NB == 2 ? min(st, block_state3(gw2, q)) : st);
+        }
+        __syncthreads();
+    } else if (staged) {
         if constexpr (NB == 2) {
             const unsigned long long* gw2 = P.words + (size_t)b2 * P.n_words;
             for (int q = tid; q < P.n_words; q += kThreads3) s_words[q] = min_states(gw[q], gw2[q]);
@@ -234,7 +249,7 @@ __global__ void __launch_bounds__(kThreads3, NB == 1 ? kMinBlocks3 : 2) k_solve_
     const unsigned long long* words = staged ? s_words : gw;
     const int blk0 = P.active[a0];
     const int bx0 = blk0 % P.nbx, by0 = (blk0 / P.nbx) % P.nby, bz0 = blk0 / (P.nbx * P.nby);
-    const int state0 = block_state3(words, blk0) - 1;
+    const int state0 = (INFO ? s_info[blk0] & 7 : block_state3(words, blk0)) - 1;
     if (state0 < 0) {  // state words do not describe this active block
         raise_status(P.status, DEX_ERR_TRAVERSAL_CAP);
         return;
@@ -247,8 +262,8 @@ __global__ void __launch_bounds__(kThreads3, NB == 1 ? kMinBlocks3 : 2) k_solve_
     unsigned int nseg = 0;
     bool capped = false;
 
-    // each thread takes kCells3 / kThreads3 probes of the block, one after the other
-    for (int pc = tid; pc < kCells3; pc += kThreads3) {
+    {
+        const int pc = part * kThreads3 + tid;
         const int i = bx0 * B3 + (pc & 7), j = by0 * B3 + ((pc >> 3) & 7), k = bz0 * B3 + (pc >> 6);
         const size_t cell = ((size_t)k * P.ny + j) * P.nx + i;
         // J of the probe: registers for one batch, shared memory for a pair (whose
@@ -257,12 +272,18 @@ __global__ void __launch_bounds__(kThreads3, NB == 1 ? kMinBlocks3 : 2) k_solve_
         auto Jw = [&](int w) -> float& { return NB == 1 ? Jr[NB == 1 ? w : 0] : s_J3[w][tid]; };
 #pragma unroll
         for (int w = 0; w < NB * W; ++w) Jw(w) = 0.0f;
+        float stop = -1.0f;
+        if (!COUNT && P.scanned) {  // the bounds wait where this probe's J will go
+            float m = P.J[(size_t)(b * W) * P.n_cells + cell];
+            if (NB == 2) m = join_bounds(m, P.J[(size_t)(b2 * W) * P.n_cells + cell]);
+            stop = stop_factor(m, P.i_bc);
+        }
         for (int q = 0; q < P.quad.n_dir; ++q) {
             float I[NB * W], T[NB * W];
 #pragma unroll
             for (int w = 0; w < NB * W; ++w) { I[w] = 0.0f; T[w] = 1.0f; }
-            trace_ray3<W, COUNT, ST, NB>(P, base, off, i, j, k, bx0, by0, bz0, a0, mip0, P.quad.dx[q], P.quad.dy[q],
-                                         P.quad.dz[q], words, I, T, nseg, capped);
+            trace_ray3<W, COUNT, ST, NB, INFO>(P, base, off, i, j, k, bx0, by0, bz0, a0, mip0, P.quad.dx[q], P.quad.dy[q],
+                                         P.quad.dz[q], words, s_info, stop, I, T, nseg, capped);
             const float wk = P.quad.w[q];
 #pragma unroll
             for (int w = 0; w < NB * W; ++w) {
@@ -281,6 +302,66 @@ __global__ void __launch_bounds__(kThreads3, NB == 1 ? kMinBlocks3 : 2) k_solve_
     if (capped) raise_status(P.status, DEX_ERR_TRAVERSAL_CAP);
     // the walk's segments, once per batch it carries
     if (COUNT && P.seg_count != nullptr) atomicAdd(P.seg_count, (unsigned long long)NB * nseg);
+}
+
+// Bounds of the exact early termination, as k_scan_bricks and k_spread_bounds.
+__device__ __forceinline__ size_t first_cell3(const Hdda3Params& P, int blk)
+{
+    const int bx = blk % P.nbx, by = blk / P.nbx % P.nby, bz = blk / (P.nbx * P.nby);
+    return ((size_t)(bz * B3) * P.ny + by * B3) * P.nx + bx * B3;
+}
+
+template <int W, int ST>
+__global__ void __launch_bounds__(128) k_scan_bricks3(const Hdda3Params P)
+{
+    constexpr int REC = RecFmt<W, ST>::kStride;
+    const int a = blockIdx.x, b = blockIdx.y;
+    if (a >= *P.n_active) return;
+    const float* brick = P.bricks + ((size_t)b * P.cap_active + a) * P.chain * REC;
+    float m = 0.0f;
+    for (int v = threadIdx.x; v < P.chain; v += blockDim.x) {
+        const Record<W> r = RecFmt<W, ST>::load(brick + (size_t)v * REC);
+#pragma unroll
+        for (int w = 0; w < W; ++w) m = join_bounds(m, bound_of(r.S[w], r.chi[w]));
+    }
+    m = join_cta(m);
+    if (threadIdx.x == 0) P.J[(size_t)(b * W) * P.n_cells + first_cell3(P, P.active[a])] = m;
+}
+
+__global__ void __launch_bounds__(256) k_spread_bounds3(const Hdda3Params P)
+{
+    float* J = P.J + (size_t)(blockIdx.y * P.W) * P.n_cells;
+    const int na = *P.n_active;
+    float m = 0.0f;
+    for (int a = threadIdx.x; a < na; a += blockDim.x) m = join_bounds(m, __ldcg(J + first_cell3(P, P.active[a])));
+    m = join_cta(m);
+    for (int a = blockIdx.x; a < na; a += gridDim.x) {
+        float* c0 = J + first_cell3(P, P.active[a]);
+        for (int q = threadIdx.x; q < kCells3; q += blockDim.x)
+            c0[((size_t)(q >> 6) * P.ny + ((q >> 3) & 7)) * P.nx + (q & 7)] = m;
+    }
+}
+
+cudaError_t scan_bricks3(cudaStream_t s, Hdda3Params& P)
+{
+    const dim3 grid((unsigned)P.cap_active, (unsigned)P.n_batch);
+    switch (P.W * 4 + P.storage) {
+#define DEX_SCAN3(WW, ST) \
+    case WW * 4 + ST: k_scan_bricks3<WW, ST><<<grid, 128, 0, s>>>(P); break;
+        DEX_SCAN3(1, kStoreF32)
+        DEX_SCAN3(2, kStoreF32)
+        DEX_SCAN3(4, kStoreF32)
+        DEX_SCAN3(8, kStoreF32)
+        DEX_SCAN3(4, kStoreBF16)
+        DEX_SCAN3(8, kStoreBF16)
+        DEX_SCAN3(4, kStoreF16)
+        DEX_SCAN3(8, kStoreF16)
+#undef DEX_SCAN3
+        default: return cudaErrorInvalidValue;
+    }
+    k_spread_bounds3<<<dim3((unsigned)(P.cap_active < 152 ? P.cap_active : 152), (unsigned)P.n_batch), 256, 0, s>>>(P);
+    P.scanned = 1;
+    return cudaSuccess;
 }
 
 template <typename K>
@@ -308,18 +389,25 @@ cudaError_t launch_solve_hdda3(cudaStream_t s, const Hdda3Params& P0)
     for (int q = 0; q < 4; ++q)
         P.band[q] = P0.n_band < 0 ? 0.0f : (q < P0.n_band ? P0.band[q] : __builtin_huge_valf());
     if (P.cap_active == 0 || P.n_batch == 0) return cudaSuccess;
-    const size_t smem = P.n_words <= kMaxStagedWords ? sizeof(unsigned long long) * (size_t)P.n_words : 0;
+    const long long n_blocks = (long long)P.nbx * P.nby * P.nbz;
+    const bool info = P.W == 8 && n_blocks <= kMaxInfo3;
+    const size_t smem = info                           ? sizeof(int) * (size_t)n_blocks
+                        : P.n_words <= kMaxStagedWords ? sizeof(unsigned long long) * (size_t)P.n_words
+                                                       : 0;
     cudaError_t e = cudaSuccess;
+    if (P.traversal == DEX_TRAVERSAL_PAIRED && !solve_hdda3_paired_applies(P)) return cudaErrorNotSupported;
+    if (!P.scanned && !P.seg_count && (e = scan_bricks3(s, P)) != cudaSuccess) return e;
     if (P.traversal == DEX_TRAVERSAL_PAIRED) {
-        if (!solve_hdda3_paired_applies(P)) return cudaErrorNotSupported;
         const int n_pairs = pair_count(P.n_batch, P.pair_group);
         if (n_pairs > 0) {
-            const dim3 grid2((unsigned)P.cap_active, (unsigned)n_pairs);
+            const dim3 grid2((unsigned)P.cap_active * kParts3, (unsigned)n_pairs);
             switch (P.storage) {
 #define DEX_LAUNCH3P(ST)                                                                     \
     case ST:                                                                                 \
-        e = P.seg_count ? launch3(k_solve_hdda3<8, true, ST, 2>, grid2, smem, s, P)          \
-                        : launch3(k_solve_hdda3<8, false, ST, 2>, grid2, smem, s, P);        \
+        e = P.seg_count ? launch3(info ? k_solve_hdda3<8, true, ST, 2, true> : k_solve_hdda3<8, true, ST, 2, false>, \
+                                  grid2, smem, s, P)                                         \
+                        : launch3(info ? k_solve_hdda3<8, false, ST, 2, true> : k_solve_hdda3<8, false, ST, 2, false>, \
+                                  grid2, smem, s, P);                                        \
         break;
                 DEX_LAUNCH3P(kStoreF32)
                 DEX_LAUNCH3P(kStoreBF16)
@@ -335,6 +423,7 @@ cudaError_t launch_solve_hdda3(cudaStream_t s, const Hdda3Params& P0)
         for (int q = 0; q < pair_lone_count(P.n_batch, P.pair_group); ++q) {
             const int m = pair_lone_batch(q, P.n_batch, P.pair_group);
             Hdda3Params Q = P0;
+            Q.scanned = P.scanned;
             Q.traversal = DEX_TRAVERSAL_PER_BATCH;
             Q.n_batch = 1;
             Q.n_lambda = min(8, P.n_lambda - m * 8);
@@ -346,22 +435,28 @@ cudaError_t launch_solve_hdda3(cudaStream_t s, const Hdda3Params& P0)
         }
         return cudaSuccess;
     }
-    const dim3 grid((unsigned)P.cap_active, (unsigned)P.n_batch);
+    const dim3 grid((unsigned)P.cap_active * kParts3, (unsigned)P.n_batch);
     switch (P.W * 4 + P.storage) {
+#define DEX_LAUNCH3_(WW, ST, INFO)                                                          \
+    e = P.seg_count ? launch3(k_solve_hdda3<WW, true, ST, 1, INFO>, grid, smem, s, P)       \
+                    : launch3(k_solve_hdda3<WW, false, ST, 1, INFO>, grid, smem, s, P);
 #define DEX_LAUNCH3(WW, ST)                                                                 \
-    case WW * 4 + ST:                                                                       \
-        e = P.seg_count ? launch3(k_solve_hdda3<WW, true, ST, 1>, grid, smem, s, P)         \
-                        : launch3(k_solve_hdda3<WW, false, ST, 1>, grid, smem, s, P);       \
+    case WW * 4 + ST: DEX_LAUNCH3_(WW, ST, false) break;
+#define DEX_LAUNCH3I(ST)                                                                    \
+    case 8 * 4 + ST:                                                                        \
+        if (info) { DEX_LAUNCH3_(8, ST, true) } else { DEX_LAUNCH3_(8, ST, false) }         \
         break;
         DEX_LAUNCH3(1, kStoreF32)
         DEX_LAUNCH3(2, kStoreF32)
         DEX_LAUNCH3(4, kStoreF32)
-        DEX_LAUNCH3(8, kStoreF32)
+        DEX_LAUNCH3I(kStoreF32)
         DEX_LAUNCH3(4, kStoreBF16)
-        DEX_LAUNCH3(8, kStoreBF16)
+        DEX_LAUNCH3I(kStoreBF16)
         DEX_LAUNCH3(4, kStoreF16)
-        DEX_LAUNCH3(8, kStoreF16)
+        DEX_LAUNCH3I(kStoreF16)
+#undef DEX_LAUNCH3I
 #undef DEX_LAUNCH3
+#undef DEX_LAUNCH3_
         default: return cudaErrorInvalidValue;
     }
     if (e != cudaSuccess) return e;

@@ -103,3 +103,69 @@ def test_sparse(walk, nx, nz, L, W, storage):
             same(full[1], fast[1])
         ctx.set_own_cell(True)
     ctx.check()
+
+
+@pytest.mark.parametrize("walk", ["per_batch", "paired"])
+@pytest.mark.parametrize("L,W,storage,n_cascades,i_bc", [(20, 8, 0, 4, 0.0), (16, 8, 1, 3, 0.6), (5, 2, 0, 4, 0.3)])
+def test_cascades(walk, L, W, storage, n_cascades, i_bc):
+    from paper_2511_08498_gb300 import api
+    ctx = ctx_()
+    nx, nz = 96, 64
+    eta, chi = thick_medium(nx, nz, L, 840 + L)
+    eta.view(L, nz, nx)[:, :16, :16] = 0.0  # cell 0 in an empty block
+    chi.view(L, nz, nx)[:, :16, :16] = 0.0
+    grid = api.grid_build(ctx, nx, nz, eta, chi)
+    ctx.set_traversal(api.TRAVERSAL_PAIRED if walk == "paired" else api.TRAVERSAL_PER_BATCH)
+    mips = api.mips_build(ctx, grid, eta, chi, W, 3, 1.0, 1.0, storage=storage)
+    full, _ = api.rc_solve(ctx, grid, mips, n_cascades, 4, 1.5, i_bc=i_bc, count_segments=True)
+    fast, _ = api.rc_solve(ctx, grid, mips, n_cascades, 4, 1.5, i_bc=i_bc)
+    same(full, fast)
+    assert not fast[:, 0].any()
+    ctx.check()
+
+
+@pytest.mark.parametrize("walk", ["per_batch", "paired"])
+@pytest.mark.parametrize("L,W,storage", [(20, 8, 0), (24, 8, 1), (9, 8, 2), (3, 1, 0), (6, 4, 0)])
+def test_sparse_3d(walk, L, W, storage):
+    from paper_2511_08498_gb300 import api
+    if walk == "paired" and W != 8:
+        pytest.skip("the paired walk needs W = 8")
+    ctx = ctx_()
+    nx, ny, nz = 32, 24, 40
+    m = synth.random_medium3(nx, ny, nz, L, seed=synth.SEED_BASE + 850 + L, log_chi_range=(-2.5, 2.5),
+                             emitter_frac=0.02 if storage == 0 else 0.0)
+    m["eta"][:, 32:], m["chi"][:, 32:] = 0.0, 0.0
+    eta, chi = (torch.from_numpy(m[k].reshape(L, -1)).cuda() for k in ("eta", "chi"))
+    grid = api.grid3_build(ctx, nx, ny, nz, eta, chi)
+    dirs, w = synth.directions3(6, 2)
+    ctx.set_traversal(api.TRAVERSAL_PAIRED if walk == "paired" else api.TRAVERSAL_PER_BATCH)
+    for iod, band, i_bc in ((1e-2, BAND, 0.0), (1e30, None, 0.4)):
+        mips = api.mips3_build(ctx, grid, eta, chi, W, 3, iod, iod, storage=storage)
+        full = api.formal_solve_hdda3(ctx, grid, mips, dirs, w, band=band, i_bc=i_bc, want_intensity=True,
+                                      count_segments=True)
+        fast = api.formal_solve_hdda3(ctx, grid, mips, dirs, w, band=band, i_bc=i_bc, want_intensity=True)
+        same(full[0], fast[0])
+        same(full[1], fast[1])
+    ctx.check()
+
+
+@pytest.mark.parametrize("kind", ["cav", "vel"])
+@pytest.mark.parametrize("L,W,i_bc", [(12, 8, 0.0), (16, 8, 0.8), (5, 2, 0.0), (9, 4, 0.2)])
+def test_moving(kind, L, W, i_bc):
+    from paper_2511_08498_gb300 import api
+    ctx = ctx_()
+    nx, nz = 96, 128
+    m = synth.dynamic_line_atmosphere(nx, nz, n_lambda=L, seed=synth.SEED_BASE + 860 + L, empty_frac=0.2)
+    f = {k: torch.from_numpy(np.ascontiguousarray(m[k]).reshape(-1)).cuda() for k in api.CAV_FIELDS}
+    for k in ("chi_c", "eta_c"):  # a continuum that ends rays within the grid
+        f[k] *= 200.0
+    grid = api.cav_grid_build(ctx, nx, nz, f)
+    build, solve = ((api.cav_mips_build, api.formal_solve_cav) if kind == "cav"
+                    else (api.vel_mips_build, api.formal_solve_velinterp))
+    mips = build(ctx, grid, f, m["dv"], m["c_kms"], W, 3, 1.0, 1.0)
+    dirs, w = synth.directions(8)
+    full = solve(ctx, grid, mips, dirs, w, band=BAND, i_bc=i_bc, want_intensity=True, count_segments=True)
+    fast = solve(ctx, grid, mips, dirs, w, band=BAND, i_bc=i_bc, want_intensity=True)
+    same(full[0], fast[0])
+    same(full[1], fast[1])
+    ctx.check()
