@@ -96,12 +96,17 @@ struct PathBuilder {
     // Crossing r: m x planes and r - m z planes precede it in the merged order (x
     // first on ties).  Within rounding m is r |dx| / (|dx| + |dz|); the two loops
     // correct it to the order of the rounded parameters (0 to 2 steps).
-    __device__ __forceinline__ PathStep next(int c0, int lane)
+    __device__ __forceinline__ int x_planes(int r) const
     {
-        const int r = c0 + lane;
         int m = min(max(__float2int_rn((float)r * fx), 0), r);
         while (m > 0 && !(tx(m - 1) <= tz(r - m))) --m;
         while (m < r && tx(m) <= tz(r - m - 1)) ++m;
+        return m;
+    }
+    __device__ __forceinline__ PathStep next(int c0, int lane, int& m)
+    {
+        const int r = c0 + lane;
+        m = x_planes(r);
         const int n = r - m;
         const float tnx = tx(m), tnz = tz(n);
         const bool on_x = tnx <= tnz;
@@ -148,7 +153,8 @@ __device__ __forceinline__ void dense_ray(const DenseParams& P, PathStep* path, 
     for (int w = 0; w < W; ++w) { I[w] = 0.0f; T[w] = 1.0f; }
     // a ray crosses at most nx + nz planes
     for (int c0 = 0; c0 < P.nx + P.nz; c0 += 32) {
-        const PathStep mine = B.next(c0, lane);
+        int m;
+        const PathStep mine = B.next(c0, lane, m);
         __syncwarp();  // every lane is done with the previous crossings
         path[lane] = mine;
         __syncwarp();
@@ -178,6 +184,133 @@ __device__ __forceinline__ void dense_ray(const DenseParams& P, PathStep* path, 
             }
         }
         if (!__any_sync(0xffffffffu, live)) break;
+    }
+}
+
+// Every cell a probe, W = 8, grids that fill the chip: CTAs of 32 x 12 probes stage
+// the records that their rays cross in the next 32 crossings -- the tile, widened by
+// the crossings' x and z steps -- in shared memory (cp.async, at most 38 x 38 cells),
+// and read them there.  In planes, S and chi lie side by side per cell, so the two
+// 256-bit loads of a warp each touch every line of its 2 KB and take 16 passes of the
+// L1 data pipe each where 8 would do: that pipe was 82% busy and bound k_solve_dense.
+// Here the four 16-byte pieces of a record lie in four planes, so that lanes at
+// neighbouring cells read neighbouring pieces: 16 passes per warp and step, plus a
+// tenth for the staging (43% busy).  Two CTAs per SM: one stages while the other
+// integrates.  601 x 437, 20 wavelengths, 24 directions: 24.3 -> 22.9 ms; what is left
+// is the update itself (the FP32 pipe, 14 ms) and the shared loads' latency, which
+// 80 registers (12 rows, the next record read a step ahead) hide better than 64 (16
+// rows, 23.1 ms) and than two probes per thread at 123 (26.1 ms).
+constexpr int kTileRows = 12, kTileThreads = 32 * kTileRows;
+// the most of (32 + a) (kTileRows + b) over a + b = 32
+constexpr int tile_cells()
+{
+    int most = 0;
+    for (int a = 0; a <= 32; ++a)
+        most = (32 + a) * (kTileRows + 32 - a) > most ? (32 + a) * (kTileRows + 32 - a) : most;
+    return most;
+}
+constexpr int kTilePlane = ((tile_cells() * 16 + 127) / 128) * 128 + 32;  // bytes of one piece of every cell
+
+template <bool EXT>
+__global__ void __launch_bounds__(kTileThreads, 2) k_solve_dense_tile(const DenseParams P)
+{
+    extern __shared__ __align__(128) unsigned char s_rec[];  // four planes of pieces, then 32 crossings
+    PathStep* s_path = reinterpret_cast<PathStep*>(s_rec + 4 * kTilePlane);
+    const int b = blockIdx.y, warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int tiles_x = (P.nx + 31) >> 5;
+    const int i0 = blockIdx.x % tiles_x * 32, j0 = blockIdx.x / tiles_x * kTileRows;
+    const int i = i0 + lane, j = j0 + warp;
+    const bool probe = i < P.nx && j < P.nz;
+    const int p = j * P.nx + i;
+    const unsigned char* base = reinterpret_cast<const unsigned char*>(P.planes + (size_t)b * P.n_cells * 16);
+    const float stop = P.scanned && probe ? stop_factor(P.J[(size_t)(b * 8) * P.n_probe + p], P.i_bc) : -1.0f;
+    const uint32_t rec = (uint32_t)__cvta_generic_to_shared(s_rec) + (lane & 3) * kTilePlane + (lane >> 2) * 16;
+    float Jw[8];
+#pragma unroll
+    for (int w = 0; w < 8; ++w) Jw[w] = 0.0f;
+    for (int k = 0; k < P.quad.n_dir; ++k) {
+        const float dx = P.quad.dx[k], dz = P.quad.dz[k];
+        PathBuilder B(dx, dz, P.nx);
+        const float Ex = dx < 0.0f ? (float)(-i) - 0.5f : (float)(P.nx - i) - 0.5f;
+        const float Ez = dz < 0.0f ? (float)(-j) - 0.5f : (float)(P.nz - j) - 0.5f;
+        const float t2 = fminf(Ex * B.ax.ih, Ez * B.az.ih);
+        bool live = probe;
+        float I[8], T[8];
+#pragma unroll
+        for (int w = 0; w < 8; ++w) { I[w] = 0.0f; T[w] = 1.0f; }
+        int m0 = 0;
+        for (int c0 = 0; c0 < P.nx + P.nz; c0 += 32) {
+            // x and z planes crossed before this chunk and before the next: the records of
+            // the chunk's segments lie within these steps of the tile
+            const int n0 = c0 - m0, m1 = B.x_planes(c0 + 32), n1 = c0 + 32 - m1;
+            const int rw = 32 + m1 - m0, rh = kTileRows + n1 - n0;
+            const int x0 = dx < 0.0f ? i0 - m1 : i0 + m0, z0 = dz < 0.0f ? j0 - n1 : j0 + n0;
+            if (!__syncthreads_or(live)) break;  // and every warp is done with the previous records
+            for (int r = warp; r < rh; r += kTileRows) {
+                const int z = z0 + r;
+                if ((unsigned)z >= (unsigned)P.nz) continue;
+                const unsigned char* src = base + ((long long)z * P.nx + x0) * 64 + lane * 16;
+                const uint32_t dst = rec + r * rw * 16;
+                // eight cells (lanes: four pieces of each) at a time
+                for (int x = 0; x < rw; x += 8)
+                    if (x + (lane >> 2) < rw && (unsigned)(x0 + x + (lane >> 2)) < (unsigned)P.nx)
+                        asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst + x * 16), "l"(src + x * 64)
+                                     : "memory");
+            }
+            if (warp == 0) {
+                int m;
+                PathStep mine = B.next(c0, lane, m);
+                const int n = c0 + lane - m;
+                mine.off = ((dz < 0.0f ? n1 - n : n - n0) * rw + (dx < 0.0f ? m1 - m : m - m0)) * 16;
+                s_path[lane] = mine;
+                if (lane == 0) s_path[32] = mine;  // read ahead, never used
+            }
+            asm volatile("cp.async.wait_all;" ::: "memory");
+            __syncthreads();
+            m0 = m1;
+            if (live) {
+                const unsigned char* q0 = s_rec + (warp * rw + lane) * 16;
+                // the next step's record is read before this one is integrated
+                auto piece = [&](int off, int c) { return *reinterpret_cast<const float4*>(q0 + off + c * kTilePlane); };
+                PathStep ns = s_path[0];
+                float4 n0_ = piece(ns.off, 0), n1_ = piece(ns.off, 1), n2_ = piece(ns.off, 2), n3_ = piece(ns.off, 3);
+#pragma unroll 4
+                for (int q = 0; q < 32; ++q) {
+                    const PathStep s = ns;
+                    const float S[8] = {n0_.x, n0_.y, n0_.z, n0_.w, n1_.x, n1_.y, n1_.z, n1_.w};
+                    const float chi[8] = {n2_.x, n2_.y, n2_.z, n2_.w, n3_.x, n3_.y, n3_.z, n3_.w};
+                    ns = s_path[q + 1];
+                    n0_ = piece(ns.off, 0);
+                    n1_ = piece(ns.off, 1);
+                    n2_ = piece(ns.off, 2);
+                    n3_ = piece(ns.off, 3);
+                    segments<8>(S, chi, s.nl2, I, T);
+                    if constexpr (EXT) {
+                        if (c0 + q == 0) {
+#pragma unroll
+                            for (int w = 0; w < 8; ++w) I[w] = 0.0f;
+                        }
+                    }
+                    if (s.th >= t2 || ((q & 7) == 7 && ray_done<8>(I, T, stop))) {
+                        live = false;
+                        break;
+                    }
+                }
+            }
+        }
+        const float wk = P.quad.w[k];
+#pragma unroll
+        for (int w = 0; w < 8; ++w) {
+            const float Iw = fmaf(T[w], P.i_bc, I[w]);
+            Jw[w] = fmaf(wk, Iw, Jw[w]);
+            const int l = b * 8 + w;
+            if (P.I != nullptr && probe && l < P.n_lambda) P.I[((size_t)l * P.quad.n_dir + k) * P.n_probe + p] = Iw;
+        }
+    }
+#pragma unroll
+    for (int w = 0; w < 8; ++w) {
+        const int l = b * 8 + w;
+        if (probe && l < P.n_lambda) P.J[(size_t)l * P.n_probe + p] = Jw[w];
     }
 }
 
@@ -320,15 +453,30 @@ __global__ void __launch_bounds__(256) k_dense_spread(const DenseParams P, int n
     for (int p = blockIdx.x * blockDim.x + threadIdx.x; p < P.n_probe; p += gridDim.x * blockDim.x) J[p] = m;
 }
 
+cudaError_t launch_dense_tile(cudaStream_t s, const DenseParams& P)
+{
+    const dim3 grid((unsigned)(((P.nx + 31) / 32) * ((P.nz + kTileRows - 1) / kTileRows)), (unsigned)P.n_batch);
+    auto kernel = P.exclude_own ? k_solve_dense_tile<true> : k_solve_dense_tile<false>;
+    const size_t smem = 4 * kTilePlane + 33 * sizeof(PathStep);
+    cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (e != cudaSuccess) return e;
+    kernel<<<grid, kTileThreads, smem, s>>>(P);
+    return cudaGetLastError();
+}
+
+template <int W>
+void launch_dense_scan(cudaStream_t s, const DenseParams& P)
+{
+    const int parts = P.n_probe < kScanCtas ? P.n_probe : kScanCtas;
+    k_dense_scan<W><<<dim3((unsigned)parts, (unsigned)P.n_batch), 256, 0, s>>>(P);
+    const int ctas = (P.n_probe + 1023) / 1024;
+    k_dense_spread<<<dim3((unsigned)(ctas < 304 ? ctas : 304), (unsigned)P.n_batch), 256, 0, s>>>(P, parts);
+}
+
 template <int W>
 void launch_dense_w(bool split, dim3 grid, cudaStream_t s, const DenseParams& P)
 {
-    if (P.scanned) {
-        const int parts = P.n_probe < kScanCtas ? P.n_probe : kScanCtas;
-        k_dense_scan<W><<<dim3((unsigned)parts, (unsigned)P.n_batch), 256, 0, s>>>(P);
-        const int ctas = (P.n_probe + 1023) / 1024;
-        k_dense_spread<<<dim3((unsigned)(ctas < 304 ? ctas : 304), (unsigned)P.n_batch), 256, 0, s>>>(P, parts);
-    }
+    if (P.scanned) launch_dense_scan<W>(s, P);
 #define DEX_LAUNCH_DENSE(K)                                               \
     if (P.exclude_own) {                                                  \
         if (P.seg_count) K<W, true, true><<<grid, 256, 0, s>>>(P);        \
@@ -371,6 +519,10 @@ cudaError_t launch_solve_dense(cudaStream_t s, const DenseParams& P0)
     // fill the chip
     const long long warps = (P.n_probe + 31LL) / 32 * P.n_batch;
     const bool split = warps < kSplitWarps;
+    if (!split && P.W == 8 && P.probes == nullptr && !P.seg_count) {
+        if (P.scanned) launch_dense_scan<8>(s, P);
+        return launch_dense_tile(s, P);
+    }
     const int rows = split ? 1 : 8;
     const unsigned tiles = P.probes == nullptr ? (unsigned)(((P.nx + 31) / 32) * ((P.nz + rows - 1) / rows))
                                                : (unsigned)((P.n_probe + 32 * rows - 1) / (32 * rows));
