@@ -1500,11 +1500,11 @@ int dex_rc_solve(dex_ctx* ctx, int nx, int nz, int n_lambda, int W, int max_mip,
     const size_t n_cells = (size_t)nx * nz;
     const size_t half = (size_t)P.n_batch * (size_t)n0 * n_cells * (size_t)W;
     cudaError_t e = cudaMemsetAsync(J, 0, sizeof(float) * (size_t)n_lambda * n_cells, ctx->stream);
-    // counting solves run rays to exactly zero transmission; the others' bounds lie in
-    // the half of the workspace that cascade 0 does not use, beyond the quarter of it
-    // that an upper cascade fills
-    if (e == cudaSuccess && !seg_count)
-        e = dex::launch_rc_scan(ctx->stream, P, workspace + (n_cascades % 2 == 1 ? half : 0) + half / 2, &P.bounds);
+    // tables in the half of the workspace that cascade 0 does not use, beyond the quarter
+    // of it that an upper cascade fills; counting solves run rays to exactly zero
+    // transmission, so they take no bounds
+    if (e == cudaSuccess)
+        e = dex::launch_rc_tables(ctx->stream, P, workspace + (n_cascades % 2 == 1 ? half : 0) + half / 2, !seg_count);
     // direction offsets: cascade i starts at n0 (4^i - 1) / 3
     const float* upper = nullptr;
     float* out = nullptr;

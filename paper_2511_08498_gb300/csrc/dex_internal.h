@@ -332,6 +332,7 @@ struct RcParams {
     int paired, pair_group;                    // W = 8: one walk per pair of batches (pair_batches)
     int siblings;                              // sibling directions in neighbouring lanes: 4, or 1
     float* J;                                  // cascade 0 of four directions: their mean goes here, else nullptr
+    const int* info;                           // word per block of every walk (launch_rc_tables)
     const float* bounds;                       // the batches' bounds of the early termination, or nullptr
     float t_s, t_e, i_bc;                      // radiance interval, boundary intensity
     const float* bricks;
@@ -344,7 +345,9 @@ struct RcParams {
     unsigned int* status;
 };
 cudaError_t launch_rc_cascade(cudaStream_t s, const RcParams& P);
-cudaError_t launch_rc_scan(cudaStream_t s, const RcParams& P, float* scratch, const float** bounds);
+// the walks' words per block and, if asked, the batches' bounds, in scratch (at most
+// 2 n_batch n_blocks + n_batch floats); sets P.info and P.bounds
+cudaError_t launch_rc_tables(cudaStream_t s, RcParams& P, float* scratch, bool bounds);
 cudaError_t launch_rc_mean(cudaStream_t s, const RcParams& P, const float* L0, float* J);
 
 // ------------------------------------------------------------------- 3D --

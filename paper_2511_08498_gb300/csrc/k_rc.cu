@@ -41,24 +41,16 @@ __device__ __forceinline__ int rc_block_state(const unsigned long long* words, i
     return (int)((words[wi] >> sh) & 7ull);
 }
 
-// Block state of the walk: NB = 1 the batch's own, NB = 2 the smaller of the
-// two batches' states (0 = empty wins).
-template <int NB>
-__device__ __forceinline__ int rc_walk_state(const unsigned long long* w1, const unsigned long long* w2, int blk)
-{
-    const int s1 = rc_block_state(w1, blk);
-    return NB == 2 ? min(s1, rc_block_state(w2, blk)) : s1;
-}
-
 // Emission I and transmission T of the interval [t_s, t_e] of the ray o + t d
 // through the sparse mipmapped grid; returns true when the ray leaves the grid
-// before t_e.  NB = 2: two wavelength batches (bricks `off` floats apart, state
-// words words2) along one walk on the smaller of their levels; I and T hold
-// 2 W values, the second batch's from index W.
+// before t_e.  NB = 2: two wavelength batches (bricks `off` floats apart) along one
+// walk on the smaller of their levels; I and T hold 2 W values, the second batch's
+// from index W.  info: the walk's word per block, offset * 8 + state
+// (k_rc_info): one load per block entered, where the packed states of one or two
+// batches and the offset table took three in a row and two divisions by 21.
 template <int W, bool COUNT, int ST, int NB = 1>
 __device__ __forceinline__ bool rc_interval(const RcParams& P, const float* __restrict__ base, long long off,
-                                            const unsigned long long* __restrict__ words,
-                                            const unsigned long long* __restrict__ words2, float ox, float oz,
+                                            const int* __restrict__ info, float ox, float oz,
                                             float dx, float dz, float stop, float* I, float* T,
                                             unsigned int& nseg, bool& capped)
 {
@@ -78,7 +70,7 @@ __device__ __forceinline__ bool rc_interval(const RcParams& P, const float* __re
     const int cz = min(max(__float2int_rd(fmaf(P.t_s, dz, oz)), 0), P.nz - 1);
     int bxc = cx >> 4, bzc = cz >> 4;
     int blk = bzc * P.nbx + bxc;
-    int st = rc_walk_state<NB>(words, words2, blk) - 1;
+    int key = __ldg(info + blk), st = (key & 7) - 1;
     int mip = st < 0 ? -1 : min(st, P.level_cap);
     int shift = mip >= 0 ? mip : 4;
     int vox = 1 << shift, side = DEX_BLOCK >> shift;
@@ -87,7 +79,7 @@ __device__ __forceinline__ bool rc_interval(const RcParams& P, const float* __re
     float Pz = (float)(bzc * DEX_BLOCK + (lz + (negz ? 0 : 1)) * vox) - oz;
     const float* rp = base;
     if (mip >= 0)
-        rp = base + BF::offset((long long)P.block_offset[blk] * P.chain + rc_level_offset(mip), lz, lx, side);
+        rp = base + BF::offset((long long)(key >> 3) * P.chain + rc_level_offset(mip), lz, lx, side);
     float th_prev = P.t_s, tl_prev = 0.0f;
 
     Record<W> r, r2;
@@ -131,7 +123,8 @@ __device__ __forceinline__ bool rc_interval(const RcParams& P, const float* __re
                     break;
                 }
                 blk = bzn * P.nbx + bxn;
-                st = rc_walk_state<NB>(words, words2, blk) - 1;
+                key = __ldg(info + blk);
+                st = (key & 7) - 1;
                 const int mip_new = st < 0 ? -1 : min(st, P.level_cap);
                 if (mip_new == mip) {
                     if (on_x) lx = negx ? side - 1 : 0;
@@ -162,7 +155,7 @@ __device__ __forceinline__ bool rc_interval(const RcParams& P, const float* __re
                 bxc = bxn;
                 bzc = bzn;
                 if (mip >= 0)
-                    rp = base + BF::offset((long long)P.block_offset[blk] * P.chain + rc_level_offset(mip), lz, lx, side);
+                    rp = base + BF::offset((long long)(key >> 3) * P.chain + rc_level_offset(mip), lz, lx, side);
             }
         }
         if (cur_mip >= 0) {
@@ -217,6 +210,32 @@ __device__ __forceinline__ float sibling_sum(float v)
     return ((v + s1) + s2) + s3;
 }
 
+// Walks (units) of a solve: the batches, or with P.paired the pairs, then the lone
+// batches.
+template <int NB>
+__device__ __forceinline__ int rc_first_unit(const RcParams& P)
+{
+    return NB == 1 && P.paired ? pair_count(P.n_batch, P.pair_group) : 0;
+}
+
+// The word per block of every walk.
+__global__ void __launch_bounds__(256) k_rc_info(const RcParams P, int n_pairs, int* __restrict__ info)
+{
+    const int nb = P.nbx * P.nbz, u = blockIdx.y;
+    int b = u, b2;
+    if (P.paired) {
+        if (u < n_pairs) pair_batches(u, P.n_batch, P.pair_group, b, b2);
+        else b = b2 = pair_lone_batch(u - n_pairs, P.n_batch, P.pair_group);
+    } else {
+        b2 = b;
+    }
+    const unsigned long long *w1 = P.words + (size_t)b * P.n_words, *w2 = P.words + (size_t)b2 * P.n_words;
+    const int blk = blockIdx.x * blockDim.x + threadIdx.x;
+    if (blk < nb)
+        info[(size_t)u * nb + blk] =
+            pack_block_info(P.block_offset[blk], min(rc_block_state(w1, blk), rc_block_state(w2, blk)));
+}
+
 // NB = 1: blockIdx.y is the batch (with P.paired: the lone batch
 // pair_lone_batch(blockIdx.y)); NB = 2: the pair pair_batches(blockIdx.y), one
 // walk for both batches on the smaller of their levels.
@@ -244,10 +263,9 @@ __global__ void __launch_bounds__(kRcThreads, (NB == 1 ? 1024 : 512) / kRcThread
     }
     const int k = j * sib + s;
     const int px = p % P.pnx, pz = p / P.pnx;
-    const unsigned long long* words = P.words + (size_t)b * P.n_words;
-    const unsigned long long* words2 = P.words + (size_t)b2 * P.n_words;
+    const int* info = P.info + (size_t)(rc_first_unit<NB>(P) + blockIdx.y) * (P.nbx * P.nbz);
     if (live && P.spacing == 1)  // cascade 0: probes only in non-empty blocks
-        live = rc_block_state(words, (pz >> 4) * P.nbx + (px >> 4)) != 0;
+        live = (__ldg(info + (pz >> 4) * P.nbx + (px >> 4)) & 7) != 0;
     constexpr int REC = RecFmt<W, ST>::kStride;
     const size_t batch_floats = (size_t)P.cap_active * P.chain * REC;
     const float* base = P.bricks + (size_t)b * batch_floats;
@@ -266,7 +284,7 @@ __global__ void __launch_bounds__(kRcThreads, (NB == 1 ? 1024 : 512) / kRcThread
             if (NB == 2) m = join_bounds(m, __ldg(P.bounds + b2));
             stop = stop_factor(m, P.i_bc);
         }
-        left = rc_interval<W, COUNT, ST, NB>(P, base, off, words, words2, ox, oz, P.dirs[2 * k], P.dirs[2 * k + 1], stop,
+        left = rc_interval<W, COUNT, ST, NB>(P, base, off, info, ox, oz, P.dirs[2 * k], P.dirs[2 * k + 1], stop,
                                              I, T, nseg, capped);
     }
 
@@ -347,8 +365,8 @@ __global__ void __launch_bounds__(256) k_rc_mean(const RcParams P, const float* 
     }
 }
 
-// Bounds of the exact early termination, in a part of the workspace that the
-// cascades leave free: every block's of every batch, then the batches'.
+// Bounds of the exact early termination, in the workspace beside the walks' words:
+// every block's of every batch, then the batches'.
 template <int W, int ST>
 __global__ void __launch_bounds__(128) k_rc_scan(const RcParams P, float* __restrict__ parts)
 {
@@ -409,23 +427,30 @@ cudaError_t launch_rc_cascade(cudaStream_t s, const RcParams& P)
     return cudaGetLastError();
 }
 
-cudaError_t launch_rc_scan(cudaStream_t s, const RcParams& P, float* scratch, const float** bounds)
+cudaError_t launch_rc_tables(cudaStream_t s, RcParams& P, float* scratch, bool bounds)
 {
     if (P.n_batch == 0) return cudaSuccess;
     const int nb = P.nbx * P.nbz;
-    float* out = scratch + (size_t)nb * P.n_batch;
+    int* info = reinterpret_cast<int*>(scratch);
+    const int n_pairs = P.paired ? pair_count(P.n_batch, P.pair_group) : 0;
+    const int units = P.paired ? n_pairs + pair_lone_count(P.n_batch, P.pair_group) : P.n_batch;
+    k_rc_info<<<dim3((unsigned)((nb + 255) / 256), (unsigned)units), 256, 0, s>>>(P, n_pairs, info);
+    P.info = info;
+    if (!bounds) return cudaGetLastError();
+    float* parts = scratch + (size_t)nb * units;
+    float* out = parts + (size_t)nb * P.n_batch;
     const dim3 grid((unsigned)nb, (unsigned)P.n_batch);
     switch (P.W * 4 + P.storage) {
-        case 1 * 4 + kStoreF32: k_rc_scan<1, kStoreF32><<<grid, 128, 0, s>>>(P, scratch); break;
-        case 2 * 4 + kStoreF32: k_rc_scan<2, kStoreF32><<<grid, 128, 0, s>>>(P, scratch); break;
-        case 4 * 4 + kStoreF32: k_rc_scan<4, kStoreF32><<<grid, 128, 0, s>>>(P, scratch); break;
-        case 8 * 4 + kStoreF32: k_rc_scan<8, kStoreF32><<<grid, 128, 0, s>>>(P, scratch); break;
-        case 8 * 4 + kStoreBF16: k_rc_scan<8, kStoreBF16><<<grid, 128, 0, s>>>(P, scratch); break;
-        case 8 * 4 + kStoreF16: k_rc_scan<8, kStoreF16><<<grid, 128, 0, s>>>(P, scratch); break;
+        case 1 * 4 + kStoreF32: k_rc_scan<1, kStoreF32><<<grid, 128, 0, s>>>(P, parts); break;
+        case 2 * 4 + kStoreF32: k_rc_scan<2, kStoreF32><<<grid, 128, 0, s>>>(P, parts); break;
+        case 4 * 4 + kStoreF32: k_rc_scan<4, kStoreF32><<<grid, 128, 0, s>>>(P, parts); break;
+        case 8 * 4 + kStoreF32: k_rc_scan<8, kStoreF32><<<grid, 128, 0, s>>>(P, parts); break;
+        case 8 * 4 + kStoreBF16: k_rc_scan<8, kStoreBF16><<<grid, 128, 0, s>>>(P, parts); break;
+        case 8 * 4 + kStoreF16: k_rc_scan<8, kStoreF16><<<grid, 128, 0, s>>>(P, parts); break;
         default: return cudaErrorInvalidValue;
     }
-    k_rc_bound<<<(unsigned)P.n_batch, 1024, 0, s>>>(nb, scratch, out);
-    *bounds = out;
+    k_rc_bound<<<(unsigned)P.n_batch, 1024, 0, s>>>(nb, parts, out);
+    P.bounds = out;
     return cudaGetLastError();
 }
 
