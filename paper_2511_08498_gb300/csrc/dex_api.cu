@@ -1042,6 +1042,10 @@ static int batch_launch(dex_ctx* ctx, dex::BatchParams& P, const dex_batch_item*
     return ok(ctx);
 }
 
+// Default table of the batched solve: one word per block where every grid allows it
+// (eight atmospheres of up to 512^2: 39.4 ms against 40.9 with the packed states).
+static bool stage_info(size_t max_blocks) { return max_blocks <= (size_t)dex::kInfoMaxBlocks; }
+
 int dex_batch_solve(dex_ctx* ctx, int n_atm, const dex_batch_item* atms, int W, int ctas, unsigned int* queue,
                     unsigned long long* done_ns, unsigned long long* start_ns)
 {
@@ -1052,7 +1056,7 @@ int dex_batch_solve(dex_ctx* ctx, int n_atm, const dex_batch_item* atms, int W, 
     size_t max_words = 0, max_blocks = 0;
     int r = fill_batch(ctx, n_atm, atms, W, *P, max_words, 1, &max_blocks);
     if (!r) r = bind(ctx);
-    if (!r) r = batch_launch(ctx, *P, atms, W, ctas, max_words, queue, done_ns, start_ns, 256, false, max_blocks);
+    if (!r) r = batch_launch(ctx, *P, atms, W, ctas, max_words, queue, done_ns, start_ns, 256, stage_info(max_blocks), max_blocks);
     delete P;
     return r;
 }
@@ -1098,7 +1102,7 @@ int dex_batch_solve_noalloc(dex_ctx* ctx, int n_atm, const dex_batch_item* atms,
     unsigned int* scratch = nullptr;
     cudaError_t e = dex::noalloc_scratch(&scratch);
     if (e != cudaSuccess) return cuda_fail(ctx, e, "static scratch address");
-    return batch_launch(ctx, P, atms, W, ctas, max_words, scratch, done_ns, start_ns, 256, false, max_blocks);
+    return batch_launch(ctx, P, atms, W, ctas, max_words, scratch, done_ns, start_ns, 256, stage_info(max_blocks), max_blocks);
 }
 
 }  // extern "C"
