@@ -97,11 +97,21 @@ __device__ __forceinline__ void put_bf16(unsigned char* tile, int off, float v)
     *reinterpret_cast<__nv_bfloat16*>(tile + off) = __float2bfloat16_rn(v);
 }
 
+// A sample's inputs as stored.
+struct Sample {
+    float x, a, u;
+};
+
+__device__ __forceinline__ Sample load_sample(const float* xau, long long s)
+{
+    return {xau[3 * s], xau[3 * s + 1], xau[3 * s + 2]};
+}
+
 // input features: x / 16, log10(a) + 2, u / 16; false (and zeros) for a
 // non-finite input or a <= 0
-__device__ __forceinline__ bool features(const float* xau, long long s, float* f)
+__device__ __forceinline__ bool features(Sample v, float* f)
 {
-    const float x = xau[3 * s], a = xau[3 * s + 1], u = xau[3 * s + 2];
+    const float x = v.x, a = v.a, u = v.u;
     if (!(a > 0.0f) || !isfinite(a) || !isfinite(x) || !isfinite(u)) {
         f[0] = f[1] = f[2] = 0.0f;
         return false;
@@ -110,10 +120,18 @@ __device__ __forceinline__ bool features(const float* xau, long long s, float* f
     return true;
 }
 
+__device__ __forceinline__ unsigned int pack_bf16(float2 v)
+{
+    const __nv_bfloat162 b = __float22bfloat162_rn(v);
+    return *reinterpret_cast<const unsigned int*>(&b);
+}
+
 __device__ void stage_weights(SmemNet& net, unsigned char* W2, const float* __restrict__ p)
 {
     const int t = threadIdx.x;
-    for (int q = t; q < kH * kH; q += blockDim.x) put_bf16(W2, tile_offset(q / kH, q % kH, kH), p[kW2 + q]);
+    for (int q = 2 * t; q < kH * kH; q += 2 * blockDim.x)
+        *reinterpret_cast<unsigned int*>(W2 + tile_offset(q / kH, q % kH, kH)) =
+            pack_bf16(make_float2(p[kW2 + q], p[kW2 + q + 1]));
     for (int q = t; q < kH * 3; q += blockDim.x) net.w1t[q % 3][q / 3] = bf16_round(p[kW1 + q]);
     if (t < kH) {
         net.b1[t] = p[kB1 + t];
@@ -182,21 +200,18 @@ __device__ __forceinline__ void gelu4(float2 za, float2 zb, float2& ga, float2& 
     gb = __fmul2_rn(zb, __fmul2_rn(make_float2(rb, rb), make_float2(db.y, db.x)));
 }
 
-__device__ __forceinline__ unsigned int pack_bf16(float2 v)
+// z1 of units i .. i + 3
+__device__ __forceinline__ void layer1_z4(const SmemNet& net, const float* f, int i, float2& za, float2& zb)
 {
-    const __nv_bfloat162 b = __float22bfloat162_rn(v);
-    return *reinterpret_cast<const unsigned int*>(&b);
-}
-
-// z1 of units i, i + 1
-__device__ __forceinline__ float2 layer1_z(const SmemNet& net, const float* f, int i)
-{
-    const float2 b = *reinterpret_cast<const float2*>(&net.b1[i]);
-    const float2 w0 = *reinterpret_cast<const float2*>(&net.w1t[0][i]);
-    const float2 w1 = *reinterpret_cast<const float2*>(&net.w1t[1][i]);
-    const float2 w2 = *reinterpret_cast<const float2*>(&net.w1t[2][i]);
-    return __ffma2_rn(w2, make_float2(f[2], f[2]),
-                      __ffma2_rn(w1, make_float2(f[1], f[1]), __ffma2_rn(w0, make_float2(f[0], f[0]), b)));
+    const float4 b = *reinterpret_cast<const float4*>(&net.b1[i]);
+    const float4 w0 = *reinterpret_cast<const float4*>(&net.w1t[0][i]);
+    const float4 w1 = *reinterpret_cast<const float4*>(&net.w1t[1][i]);
+    const float4 w2 = *reinterpret_cast<const float4*>(&net.w1t[2][i]);
+    const float2 f0 = make_float2(f[0], f[0]), f1 = make_float2(f[1], f[1]), f2 = make_float2(f[2], f[2]);
+    za = __ffma2_rn(make_float2(w2.x, w2.y), f2,
+                    __ffma2_rn(make_float2(w1.x, w1.y), f1, __ffma2_rn(make_float2(w0.x, w0.y), f0, make_float2(b.x, b.y))));
+    zb = __ffma2_rn(make_float2(w2.z, w2.w), f2,
+                    __ffma2_rn(make_float2(w1.z, w1.w), f1, __ffma2_rn(make_float2(w0.z, w0.w), f0, make_float2(b.z, b.w))));
 }
 
 // one MMA chain: D (+)= A B^T over K/16 K-steps, issued by the calling thread
@@ -226,8 +241,8 @@ __device__ __forceinline__ bool wait_all(unsigned long long* mbar, uint32_t& pha
 }
 
 // ------------------------------------------------------------ inference --
-// Bound by the special-function units (208 operations per sample, of 16 per SM and
-// clock: 174 us for 2^22 samples); eight CTAs per
+// Bound by instruction issue (about 10 per activation) with the FP32 pipe and the
+// special-function units at 60% and 40%; eight CTAs per
 // SM, whose phases interleave, hide the barriers and the MMA's latency.
 __global__ void __launch_bounds__(128, 8) k_mlp_forward(const MlpParams P)
 {
@@ -242,11 +257,16 @@ __global__ void __launch_bounds__(128, 8) k_mlp_forward(const MlpParams P)
     uint32_t phase = 0;
     const long long n_tiles = (P.n + kTile - 1) / kTile;
     bool ok = true;
-    for (long long tile = blockIdx.x; tile < n_tiles; tile += gridDim.x) {
-        const long long s = tile * kTile + t;
+    // the next tile's inputs are on their way while this one is evaluated
+    const long long stride = (long long)gridDim.x * kTile;
+    long long s = blockIdx.x * (long long)kTile + t;
+    Sample next = s < P.n ? load_sample(P.xau, s) : Sample{0.0f, 1.0f, 0.0f};
+    for (long long tile = blockIdx.x; tile < n_tiles; tile += gridDim.x, s += stride) {
         bool valid = s < P.n;
         float f[3] = {0.0f, 0.0f, 0.0f};
-        if (valid && !features(P.xau, s, f)) {
+        const Sample now = next;
+        if (s + stride < P.n) next = load_sample(P.xau, s + stride);
+        if (valid && !features(now, f)) {
             raise_status(P.status, DEX_ERR_NUMERIC);
             valid = false;
         }
@@ -255,7 +275,12 @@ __global__ void __launch_bounds__(128, 8) k_mlp_forward(const MlpParams P)
             uint4 h;
             unsigned int* hw = reinterpret_cast<unsigned int*>(&h);
 #pragma unroll
-            for (int q = 0; q < 4; ++q) hw[q] = pack_bf16(gelu2(layer1_z(sm.net, f, i0 + 2 * q)));
+            for (int q = 0; q < 4; q += 2) {
+                float2 za, zb;
+                layer1_z4(sm.net, f, i0 + 2 * q, za, zb);
+                hw[q] = pack_bf16(gelu2(za));
+                hw[q + 1] = pack_bf16(gelu2(zb));
+            }
             *reinterpret_cast<uint4*>(sm.H1 + tile_offset(t, i0, kTile)) = h;
         }
         sync_for_mma();
@@ -344,7 +369,7 @@ __global__ void __launch_bounds__(256, 2) k_mlp_grad(const MlpParams P)
         float f[3] = {0.0f, 0.0f, 0.0f}, target = 0.0f;
         if (valid) {
             target = P.target[s];
-            if (!features(P.xau, s, f) || !isfinite(target)) {
+            if (!features(load_sample(P.xau, s), f) || !isfinite(target)) {
                 raise_status(P.status, DEX_ERR_NUMERIC);
                 valid = false;
                 f[0] = f[1] = f[2] = 0.0f;
@@ -357,11 +382,15 @@ __global__ void __launch_bounds__(256, 2) k_mlp_grad(const MlpParams P)
             uint4 h;
             unsigned int* hw = reinterpret_cast<unsigned int*>(&h);
 #pragma unroll
-            for (int q = 0; q < 4; ++q) {
-                const Gelu2 a(layer1_z(sm.net, f, h0 + i0 + 2 * q));
-                const float2 g = a.g();
-                hw[q] = pack_bf16(g);
-                dg1[i0 / 2 + q] = a.dg(g);
+            for (int q = 0; q < 4; q += 2) {
+                float2 za, zb;
+                layer1_z4(sm.net, f, h0 + i0 + 2 * q, za, zb);
+                const Gelu2 a(za), b(zb);
+                const float2 ga = a.g(), gb = b.g();
+                hw[q] = pack_bf16(ga);
+                hw[q + 1] = pack_bf16(gb);
+                dg1[i0 / 2 + q] = a.dg(ga);
+                dg1[i0 / 2 + q + 1] = b.dg(gb);
             }
             *reinterpret_cast<uint4*>(sm.H1 + tile_offset(t, h0 + i0, kTile)) = h;
         }
@@ -554,7 +583,10 @@ cudaError_t launch_mlp_forward(cudaStream_t s, const MlpParams& P)
                                  cudaSharedmemCarveoutMaxShared);
     if (e != cudaSuccess) return e;
     const long long tiles = (P.n + kTile - 1) / kTile;
-    const long long grid = tiles < 8LL * sms ? tiles : 8LL * sms;
+    // up to eight tiles per CTA: one CTA per slot for all of them left the younger CTAs
+    // of an SM behind (248 us for 2^22 samples against 221; four 228, sixteen 231)
+    const long long per = max(1LL, min(8LL, tiles / (8LL * sms)));
+    const long long grid = (tiles + per - 1) / per;
     k_mlp_forward<<<(unsigned)grid, 128, kSmemInfer, s>>>(P);
     return cudaGetLastError();
 }
