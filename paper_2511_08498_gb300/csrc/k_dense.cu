@@ -151,6 +151,8 @@ __device__ __forceinline__ void dense_ray(const DenseParams& P, PathStep* path, 
     const float t2 = fminf(Ex * B.ax.ih, Ez * B.az.ih);
 #pragma unroll
     for (int w = 0; w < W; ++w) { I[w] = 0.0f; T[w] = 1.0f; }
+    constexpr int GROUP = W == 1 ? 8 : (W == 2 ? 4 : (W == 4 ? 2 : 1));
+    float th_end = 0.0f;  // the last crossing of the chunk before
     // a ray crosses at most nx + nz planes
     for (int c0 = 0; c0 < P.nx + P.nz; c0 += 32) {
         int m;
@@ -159,29 +161,39 @@ __device__ __forceinline__ void dense_ray(const DenseParams& P, PathStep* path, 
         path[lane] = mine;
         __syncwarp();
         if (live) {
-#pragma unroll 4
-            for (int q = 0; q < 32; ++q) {
-                const PathStep s = path[q];
-                const Record<W> r = RecFmt<W, kStoreF32>::load(rec0 + (long long)s.off * REC);
-                segments<W>(r.S, r.chi, s.nl2, I, T);
-                if constexpr (EXT) {
-                    if (c0 + q == 0) {
+            // a few records at a time, loaded before the first of them is used: a step's
+            // latency, not its arithmetic, sets the time of small grids.  A segment beyond
+            // the ray's exit (the crossing before it is at or past t2) reads nothing.
+            float th_before = c0 == 0 ? 0.0f : th_end;
+            for (int q0 = 0; q0 < 32 && live; q0 += GROUP) {
+                PathStep s[GROUP];
+                Record<W> r[GROUP];
 #pragma unroll
-                        for (int w = 0; w < W; ++w) I[w] = 0.0f;
-                    }
+                for (int g = 0; g < GROUP; ++g) {
+                    s[g] = path[q0 + g];
+                    if (g == 0 || th_before < t2) r[g] = RecFmt<W, kStoreF32>::load(rec0 + (long long)s[g].off * REC);
+                    th_before = s[g].th;
                 }
-                if (COUNT) nseg += s.moved;
-                if (s.th >= t2) {
-                    live = false;
-                    break;
+#pragma unroll
+                for (int g = 0; g < GROUP; ++g) {
+                    segments<W>(r[g].S, r[g].chi, s[g].nl2, I, T);
+                    if constexpr (EXT) {
+                        if (c0 + q0 + g == 0) {
+#pragma unroll
+                            for (int w = 0; w < W; ++w) I[w] = 0.0f;
+                        }
+                    }
+                    if (COUNT) nseg += s[g].moved;
+                    if (s[g].th >= t2) {
+                        live = false;
+                        break;
+                    }
                 }
                 // the counting variant walks every cell: its count is the full-resolution
                 // segment count that throughput figures are normalised by
-                if (!COUNT && (q & 7) == 7 && ray_done<W>(I, T, stop)) {
-                    live = false;
-                    break;
-                }
+                if (!COUNT && live && ((q0 + GROUP) & 7) == 0 && ray_done<W>(I, T, stop)) live = false;
             }
+            th_end = th_before;
         }
         if (!__any_sync(0xffffffffu, live)) break;
     }
@@ -512,9 +524,11 @@ cudaError_t launch_solve_dense(cudaStream_t s, const DenseParams& P0)
 {
     if (P0.n_probe == 0 || P0.n_batch == 0) return cudaSuccess;
     DenseParams P = P0;
-    // scan the planes for the early termination's bound where the solve reads at
-    // least sixteen times as many records
-    P.scanned = !P.seg_count && (double)P.n_probe * P.quad.n_dir * 0.5 * ((double)P.nx + P.nz) >= 16.0 * (double)P.n_cells;
+    // scan the planes for the early termination's bound where the rays cross at least
+    // sixteen times as many records, and 2^27 of them (two launches cost 5 us, a tenth
+    // of the 128 x 128 solve with 16 directions, whose rays cross 2^25)
+    const double crossed = (double)P.n_probe * P.quad.n_dir * 0.5 * ((double)P.nx + P.nz);
+    P.scanned = !P.seg_count && crossed * P.n_batch >= 134217728.0 && crossed >= 16.0 * (double)P.n_cells;
     // one warp per 32 probes, or eight (one per direction) where those would not
     // fill the chip
     const long long warps = (P.n_probe + 31LL) / 32 * P.n_batch;
