@@ -1035,9 +1035,8 @@ static int batch_launch(dex_ctx* ctx, dex::BatchParams& P, const dex_batch_item*
                             ctx->stream);
     if (e == cudaSuccess && done_ns) e = cudaMemsetAsync(done_ns, 0, sizeof(unsigned long long) * P.n_atm, ctx->stream);
     if (e == cudaSuccess && start_ns) e = cudaMemsetAsync(start_ns, 0xff, sizeof(unsigned long long), ctx->stream);
-    // the paired walk stages one word per block (max_blocks: the largest grid)
-    const size_t smem = info || P.paired ? sizeof(int) * max_blocks : sizeof(unsigned long long) * max_words;
-    if (e == cudaSuccess) e = dex::launch_batch_solve(ctx->stream, P, ctas, W, packet, info, occupancy, smem);
+    if (e == cudaSuccess)
+        e = dex::launch_batch_solve(ctx->stream, P, ctas, W, packet, info, occupancy, max_words, max_blocks);
     if (e != cudaSuccess) return cuda_fail(ctx, e, "batch_solve launch");
     return ok(ctx);
 }

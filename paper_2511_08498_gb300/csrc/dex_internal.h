@@ -94,6 +94,13 @@ __host__ __device__ inline void pair_batches(int p, int n_batch, int group, int&
     b1 = b2 = -1;
 }
 
+// The batch paired with b, or b itself.
+__host__ __device__ inline int pair_partner(int b, int n_batch, int group)
+{
+    const int g = pair_group_size(n_batch, group), g0 = b / g * g;
+    return g0 + (n_batch - g0 < g ? n_batch - g0 : g) - 1 - (b - g0);
+}
+
 // Lone batches of the pairing: the middle batch of every group of odd size.
 __host__ __device__ inline int pair_lone_count(int n_batch, int group)
 {
@@ -124,6 +131,8 @@ struct HddaParams {
     int exclude_own; // leave out each probe's own-voxel emission (static model, W = 8, float32)
     int scanned;     // J holds the bounds of the exact early termination (scan.cuh)
     int split_at;    // float offset of the split kernels' intensities in dynamic shared memory
+    int twins;       // one walk per batch: pairs of batches whose blocks all have the same levels
+                     // are walked once (states_agree; k_solve_hdda_pair, then the others alone)
     float band[4];
     long long n_cells;
     const float* bricks;
@@ -262,6 +271,7 @@ struct BatchParams {
     long long n_items;
     int paired;             // W = 8: work units are pairs of batches (pair_batches) and lone batches
     int pair_group;         //   paired within groups of this many batches (0: one group)
+    int twins;              // one walk per batch, as HddaParams::twins
     int parts;              // work items per active block and batch: 256 / probes per item
     int chunk;              // work items claimed per queue increment
     unsigned int* queue;
@@ -274,9 +284,9 @@ struct BatchParams {
 // packet: probes per work item (256, 128 or 64); info: stage one word per block
 // (offset * 8 + state) instead of the packed state words; occupancy (W = 8): a
 // 64-register budget (four 256-thread CTAs per SM) instead of the compiler's;
-// smem_bytes: the largest table of the batch
+// max_words, max_blocks: of the batch's largest grid
 cudaError_t launch_batch_solve(cudaStream_t s, const BatchParams& P, int ctas, int W, int packet, bool info,
-                               bool occupancy, size_t smem_bytes);
+                               bool occupancy, size_t max_words, size_t max_blocks);
 // work units of one atmosphere: its batches, or with P.paired its pairs and lone batches
 inline int batch_units(const BatchParams& P, int n_batch)
 {
@@ -323,6 +333,8 @@ bool solve_hdda_shared_applies(const HddaParams& p);
 cudaError_t launch_solve_hdda_shared(cudaStream_t s, const HddaParams& p);
 bool solve_hdda_paired_applies(const HddaParams& p);
 cudaError_t launch_solve_hdda_paired(cudaStream_t s, const HddaParams& p);
+// the pairs of batches whose levels agree, for the per-batch walk (p.twins)
+cudaError_t launch_solve_hdda_twins(cudaStream_t s, const HddaParams& p);
 
 // --------------------------------------------------- radiance cascades --
 struct RcParams {

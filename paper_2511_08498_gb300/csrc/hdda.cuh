@@ -403,6 +403,15 @@ __device__ __forceinline__ void split_solve(const Quadrature& quad, float* s_I, 
         if (warp + q * NW < W) store(warp + q * NW, J[q]);
 }
 
+// Whether two batches have the same level in every block (all threads of the CTA).
+// A walk shared by the two then takes, at every step, the levels of each one's own.
+__device__ __forceinline__ bool states_agree(const unsigned long long* w1, const unsigned long long* w2, int n_words)
+{
+    bool differ = false;
+    for (int q = threadIdx.x; q < n_words; q += blockDim.x) differ |= __ldg(w1 + q) != __ldg(w2 + q);
+    return !__syncthreads_or(differ);
+}
+
 // kInfo: the CTA stages one word per block (offset * 8 + state, InfoLookup;
 // dynamic shared memory 4 * nbx * nbz bytes, grids of at most kInfoMaxBlocks
 // blocks); otherwise the packed state words (WordLookup; 8 * n_words bytes).
@@ -419,6 +428,13 @@ __global__ void __launch_bounds__(256, Model::kMinBlocks) k_solve_hdda_t(const H
     const int b = blockIdx.y;
     const int tid = threadIdx.x;
     const unsigned long long* words_b = P.words + (size_t)b * P.n_words;
+    if constexpr (Model::kPerBatch && W == 8 && !COUNT && !EXT) {
+        // walked with its partner (k_solve_hdda_pair) if their levels agree
+        if (P.twins) {
+            const int b2 = pair_partner(b, P.n_batch, P.pair_group);
+            if (b2 != b && states_agree(words_b, P.words + (size_t)b2 * P.n_words, P.n_words)) return;
+        }
+    }
     int* s_info = reinterpret_cast<int*>(s_dyn);
     if constexpr (kInfo) {
         const int n_blocks = P.nbx * P.nbz;

@@ -4,8 +4,10 @@
 // block), numbered atmosphere by atmosphere (item_base[a] + (batch * capacity_a
 // + rank) * parts + part).  A fixed grid of CTAs pulls `chunk` items at a time
 // from a device counter (the queue) until it runs dry; each item is the block
-// solve of k_solve_hdda_t (shared trace_ray) over 256 / parts of its probes.  Consecutive items mostly share an atmosphere and batch, so the
-// staged block states and quadrature are reused, and the L2 working set stays
+// solve of k_solve_hdda_t (shared trace_ray) over 256 / parts of its probes.  Where
+// pairs of batches may share a walk there are two such launches, the pairs' and the
+// other batches' (twins_apply).  Consecutive items mostly share an atmosphere and
+// batch, so the staged block states and quadrature are reused, and the L2 working set stays
 // one atmosphere batch wide.  Per-atmosphere completion times (globaltimer, ns)
 // are recorded when requested.
 
@@ -62,6 +64,9 @@ struct StaticRec {
 // kPair (W = 8): a work unit is a pair of batches (pair_batches) walked once on
 // the smaller of their two levels, 16 wavelengths per thread, or a lone batch
 // (pair_lone_batch) walked alone, as dex_formal_solve_hdda's paired walk.
+// P.twins: with kPair only the pairs whose blocks all have the same levels, without it
+// the batches of no such pair, as the TWIN walk of k_solve_hdda_pair and the per-batch
+// walk beside it.
 template <int W, int NT, bool kInfo, int kMinCtas, bool kPair = false>
 __global__ void __launch_bounds__(NT, kMinCtas) k_batch_solve(const BatchParams P)
 {
@@ -72,7 +77,7 @@ __global__ void __launch_bounds__(NT, kMinCtas) k_batch_solve(const BatchParams 
     constexpr int kParts = 256 / NT;
     int* s_info = reinterpret_cast<int*>(s_dyn);
     const int tid = threadIdx.x;
-    int cur_atm = -1, cur_batch = -1;
+    int cur_atm = -1, cur_batch = -1, skip_atm = -1, skip_batch = -1;
     unsigned int nseg_unused = 0;
     bool capped = false;
     if (P.start_ns != nullptr && tid == 0) atomicMin(P.start_ns, global_ns());
@@ -93,7 +98,7 @@ __global__ void __launch_bounds__(NT, kMinCtas) k_batch_solve(const BatchParams 
             const long long unit = local / kParts;
             const int part = (int)(local % kParts);
             const int b = (int)(unit / A.cap_active), r = (int)(unit % A.cap_active);
-            if (r >= *A.n_active) continue;
+            if (r >= *A.n_active || (a == skip_atm && b == skip_batch)) continue;
             // kPair: b numbers the atmosphere's pairs, then its lone batches
             int b1 = b, b2 = -1;
             if constexpr (kPair) {
@@ -103,6 +108,18 @@ __global__ void __launch_bounds__(NT, kMinCtas) k_batch_solve(const BatchParams 
             }
             __syncthreads();  // every thread is done with the previous item's shared data
             if (a != cur_atm || b != cur_batch) {
+                if constexpr (W == 8) {
+                    if (P.twins) {
+                        const int other = kPair ? (b2 >= 0 ? b2 : b1) : pair_partner(b, (A.n_lambda + W - 1) / W, P.pair_group);
+                        const bool twins = other != b1 && states_agree(A.words + (size_t)b1 * A.n_words,
+                                                                       A.words + (size_t)other * A.n_words, A.n_words);
+                        if (twins != kPair) {
+                            skip_atm = a;
+                            skip_batch = b;
+                            continue;
+                        }
+                    }
+                }
                 if constexpr (kPair) {
                     // one word per block, offset * 8 + the smaller of the pair's states
                     const int nb = A.nbx * A.nbz;
@@ -156,43 +173,62 @@ __global__ void __launch_bounds__(NT, kMinCtas) k_batch_solve(const BatchParams 
             const size_t cell = (size_t)j * A.nx + i;
             const size_t plane = (size_t)W * A.nx * A.nz;
             float bound = A.J[b1 * plane + cell];
-            if (kPair && b2 >= 0) bound = join_bounds(bound, A.J[b2 * plane + cell]);
-            G.stop = stop_factor(bound, A.i_bc);
-            const int mip0 = min(state0, distance_cap(G, 0.0f));
-            typename StaticRec<W>::Params M{};
-            for (int k = 0; k < A.n_dir; ++k) {
-                const float wk = s_w[k];
-                if (kPair && b2 >= 0) {
-                    // the pair: 16 wavelengths along one walk
-                    using PM = PairRecModel<kStoreF32, kMinCtas>;
-                    const typename PM::Params M2{(long long)(b2 - b1) * (long long)batch_floats};
-                    float I[2 * W], T[2 * W];
-#pragma unroll
-                    for (int w = 0; w < 2 * W; ++w) { I[w] = 0.0f; T[w] = 1.0f; }
-                    trace_ray<2 * W, false, PM>(G, M2, b1, i, j, bx0, bz0, r, mip0, s_dx[k], s_dz[k],
-                                                InfoLookup{s_info}, I, T, nseg_unused, capped);
-#pragma unroll
-                    for (int w = 0; w < 2 * W; ++w) s_J[w][tid] = fmaf(wk, fmaf(T[w], A.i_bc, I[w]), s_J[w][tid]);
+            [[maybe_unused]] float bound2 = 0.0f;
+            [[maybe_unused]] int second = -1;  // a batch to be walked by itself after b1
+            if (kPair && b2 >= 0) {
+                bound2 = A.J[b2 * plane + cell];
+                if (P.twins && join_bounds(bound, bound2) < 0.0f) {
+                    second = b2;
+                    b2 = b1;
                 } else {
-                    float I[W], T[W];
-#pragma unroll
-                    for (int w = 0; w < W; ++w) { I[w] = 0.0f; T[w] = 1.0f; }
-                    if constexpr (kInfo || kPair)
-                        trace_ray<W, false, StaticRec<W>>(G, M, b1, i, j, bx0, bz0, r, mip0, s_dx[k], s_dz[k],
-                                                           InfoLookup{s_info}, I, T, nseg_unused, capped);
-                    else
-                        trace_ray<W, false, StaticRec<W>>(G, M, b1, i, j, bx0, bz0, r, mip0, s_dx[k], s_dz[k],
-                                                           WordLookup{s_dyn, A.block_offset}, I, T, nseg_unused,
-                                                           capped);
-#pragma unroll
-                    for (int w = 0; w < W; ++w) s_J[w][tid] = fmaf(wk, fmaf(T[w], A.i_bc, I[w]), s_J[w][tid]);
+                    bound = join_bounds(bound, bound2);
                 }
             }
+            const int mip0 = min(state0, distance_cap(G, 0.0f));
+            typename StaticRec<W>::Params M{};
             const long long n_cells = (long long)A.nx * A.nz;
+            for (;;) {
+                G.stop = stop_factor(bound, A.i_bc);
+                for (int k = 0; k < A.n_dir; ++k) {
+                    const float wk = s_w[k];
+                    if (kPair && b2 >= 0) {
+                        // the pair: 16 wavelengths along one walk
+                        using PM = PairRecModel<kStoreF32, kMinCtas>;
+                        const typename PM::Params M2{(long long)(b2 - b1) * (long long)batch_floats};
+                        float I[2 * W], T[2 * W];
 #pragma unroll
-            for (int w = 0; w < (kPair ? 2 * W : W); ++w) {
-                const int l = w < W ? b1 * W + w : b2 * W + (w - W);
-                if ((w < W || b2 >= 0) && l < A.n_lambda) A.J[(size_t)l * n_cells + (size_t)j * A.nx + i] = s_J[w][tid];
+                        for (int w = 0; w < 2 * W; ++w) { I[w] = 0.0f; T[w] = 1.0f; }
+                        trace_ray<2 * W, false, PM>(G, M2, b1, i, j, bx0, bz0, r, mip0, s_dx[k], s_dz[k],
+                                                    InfoLookup{s_info}, I, T, nseg_unused, capped);
+#pragma unroll
+                        for (int w = 0; w < 2 * W; ++w) s_J[w][tid] = fmaf(wk, fmaf(T[w], A.i_bc, I[w]), s_J[w][tid]);
+                    } else {
+                        float I[W], T[W];
+#pragma unroll
+                        for (int w = 0; w < W; ++w) { I[w] = 0.0f; T[w] = 1.0f; }
+                        if constexpr (kInfo || kPair)
+                            trace_ray<W, false, StaticRec<W>>(G, M, b1, i, j, bx0, bz0, r, mip0, s_dx[k], s_dz[k],
+                                                               InfoLookup{s_info}, I, T, nseg_unused, capped);
+                        else
+                            trace_ray<W, false, StaticRec<W>>(G, M, b1, i, j, bx0, bz0, r, mip0, s_dx[k], s_dz[k],
+                                                               WordLookup{s_dyn, A.block_offset}, I, T, nseg_unused,
+                                                               capped);
+#pragma unroll
+                        for (int w = 0; w < W; ++w) s_J[w][tid] = fmaf(wk, fmaf(T[w], A.i_bc, I[w]), s_J[w][tid]);
+                    }
+                }
+#pragma unroll
+                for (int w = 0; w < (kPair ? 2 * W : W); ++w) {
+                    const int l = w < W ? b1 * W + w : b2 * W + (w - W);
+                    if ((w < W || b2 >= 0) && l < A.n_lambda) A.J[(size_t)l * n_cells + (size_t)j * A.nx + i] = s_J[w][tid];
+                }
+                if (!kPair || second < 0) break;
+                G.batch_base += (size_t)(second - b1) * batch_floats;
+                b1 = b2 = second;
+                second = -1;
+                bound = bound2;
+#pragma unroll
+                for (int w = 0; w < 2 * W; ++w) s_J[w][tid] = 0.0f;
             }
             if (P.done_ns != nullptr) {
                 __syncthreads();
@@ -296,9 +332,28 @@ cudaError_t noalloc_scratch(unsigned int** out)
     return cudaSuccess;
 }
 
-cudaError_t launch_batch_solve(cudaStream_t s, const BatchParams& P, int ctas, int W, int packet, bool info,
-                               bool occupancy, size_t smem_bytes)
+// Where pairs are looked for: W = 8, grids that the pair kernel's table covers, and
+// enough blocks of pairs that the second launch's start, after the last item of the
+// first, costs less than the shared walks give.  Eight to twelve atmospheres of static
+// lines (about half of the pairs agree), one walk per batch -> with pairs: 3168 blocks of
+// pairs 23.9 -> 22.0 ms, 3904 40.1 -> 35.8, 6784 73.9 -> 64.1; but 2816 13.95 -> 13.99,
+// 1968 13.6 -> 14.9, 352 3.5 -> 5.0.
+constexpr long long kTwinItems = 3040;  // ten rounds of the pair kernel's 304 resident CTAs
+
+static bool twins_apply(const BatchParams& P, int W, size_t max_blocks)
 {
+    if (W != 8 || max_blocks > (size_t)kInfoMaxBlocks) return false;
+    long long pairs = 0;
+    for (int a = 0; a < P.n_atm; ++a)
+        pairs += (long long)pair_count((P.atm[a].n_lambda + 7) / 8, P.pair_group) * P.atm[a].cap_active;
+    return pairs >= kTwinItems;
+}
+
+cudaError_t launch_batch_solve(cudaStream_t s, const BatchParams& P0, int ctas, int W, int packet, bool info,
+                               bool occupancy, size_t max_words, size_t max_blocks)
+{
+    BatchParams P = P0;
+    const size_t smem_bytes = info ? sizeof(int) * max_blocks : sizeof(unsigned long long) * max_words;
     cudaError_t e = cudaMemsetAsync(P.queue, 0, sizeof(unsigned int), s);
     if (e != cudaSuccess || P.n_items == 0) return e;
     if (occupancy && W != 8) return cudaErrorInvalidValue;
@@ -309,18 +364,31 @@ cudaError_t launch_batch_solve(cudaStream_t s, const BatchParams& P, int ctas, i
         case 8: scan_batch<8>(s, P); break;
         default: return cudaErrorInvalidValue;
     }
-    if (P.paired) {
-        // pairs of batches (W = 8): one word per block staged, the compiler's budget
-        // bounded at 128 registers (two 256-thread CTAs per SM)
-        if (W != 8) return cudaErrorInvalidValue;
+    // pairs of batches (W = 8): one word per block staged, the compiler's budget
+    // bounded at 128 registers (two 256-thread CTAs per SM)
+    auto launch_pairs = [&](const BatchParams& Q) {
         switch (packet) {
-            case 256: e = launch_batch_t<8, 256, true, 2, true>(s, P, ctas, smem_bytes); break;
-            case 128: e = launch_batch_t<8, 128, true, 4, true>(s, P, ctas, smem_bytes); break;
-            case 64: e = launch_batch_t<8, 64, true, 8, true>(s, P, ctas, smem_bytes); break;
+            case 256: return launch_batch_t<8, 256, true, 2, true>(s, Q, ctas, sizeof(int) * max_blocks);
+            case 128: return launch_batch_t<8, 128, true, 4, true>(s, Q, ctas, sizeof(int) * max_blocks);
+            case 64: return launch_batch_t<8, 64, true, 8, true>(s, Q, ctas, sizeof(int) * max_blocks);
             default: return cudaErrorInvalidValue;
         }
-        if (e != cudaSuccess) return e;
+    };
+    if (P.paired) {
+        if (W != 8) return cudaErrorInvalidValue;
+        if ((e = launch_pairs(P)) != cudaSuccess) return e;
         return cudaGetLastError();
+    }
+    P.twins = twins_apply(P, W, max_blocks);
+    if (P.twins) {
+        BatchParams Q = P;
+        Q.n_items = 0;
+        for (int a = 0; a < P.n_atm; ++a) {
+            Q.atm[a].item_base = Q.n_items;
+            Q.n_items += (long long)pair_count((P.atm[a].n_lambda + 7) / 8, P.pair_group) * P.atm[a].cap_active * P.parts;
+        }
+        if ((e = launch_pairs(Q)) != cudaSuccess) return e;
+        if ((e = cudaMemsetAsync(P.queue, 0, sizeof(unsigned int), s)) != cudaSuccess) return e;
     }
     switch (W) {
         case 1: e = launch_batch_w<1, false>(s, P, ctas, packet, info, smem_bytes); break;

@@ -94,6 +94,27 @@ static void scan_bricks(cudaStream_t s, HddaParams& P)
     P.scanned = 1;
 }
 
+// Whether the per-batch solve looks for pairs of batches that it may walk once (twins):
+// W = 8 and a grid that the pair kernel's table covers.  The pairs and the other batches
+// are two launches, so where some batch is certain to be left for the second (the middle
+// one of an odd number) the first must fill the chip: two rounds of the pair kernel's 304
+// resident CTAs, five where directions are split.  Static lines, 32 directions, one walk
+// per batch -> with pairs:
+//   768^2, 32 wavelengths  35.2 -> 28.7 ms    256^2, 32 (split)  3.38 -> 2.98 ms
+//   512^2, 16              14.5 -> 11.8       96^2, 16 (split)   0.284 -> 0.250
+//   512^2, 24              15.4 -> 14.2       384^2, 24          7.80 -> 9.00 (not taken)
+//   320^2, 24 (split)      4.12 -> 3.79       160^2, 24 (split)  0.741 -> 0.782 (not taken)
+// bfloat16 pairs run 128-thread CTAs and gain nothing when split (160^2, 32: 1.04 ->
+// 1.15).  Where the levels differ the check costs 0.3% (768^2, 20: 36.6 both ways).
+static bool twins_apply(const HddaParams& P, bool split)
+{
+    if (P.W != 8 || P.seg_count || !P.scanned || (long long)P.nbx * P.nbz > kPairInfoMaxBlocks) return false;
+    if (split && P.storage == kStoreBF16) return false;
+    const int pairs = pair_count(P.n_batch, P.pair_group);
+    if (pair_lone_count(P.n_batch, P.pair_group) == 0) return pairs > 0;
+    return (long long)P.cap_active * pairs * (split ? 8 : 1) >= (split ? 1520 : 608);
+}
+
 cudaError_t launch_solve_hdda(cudaStream_t s, const HddaParams& P0)
 {
     if (P0.cap_active == 0 || P0.n_batch == 0) return cudaSuccess;
@@ -129,6 +150,8 @@ cudaError_t launch_solve_hdda(cudaStream_t s, const HddaParams& P0)
     const size_t smem = sizeof(float) * ((size_t)P.split_at + (split ? (size_t)split_chunk<8>() * P.W * 32 : 0));
     const dim3 grid((unsigned)P.cap_active * (split ? 8u : 1u), (unsigned)P.n_batch);
     cudaError_t e = cudaSuccess;
+    P.twins = twins_apply(P, split);
+    if (P.twins && (e = launch_solve_hdda_twins(s, P)) != cudaSuccess) return e;
     switch (P.W * 4 + P.storage) {
 #define DEX_LAUNCH_(WW, ST, INFO)                                                                                     \
     {                                                                                                                 \

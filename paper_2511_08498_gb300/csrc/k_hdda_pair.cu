@@ -60,7 +60,12 @@ using PairModel = PairRecModel<ST, pair_min_blocks<ST>()>;
 // EXT: each probe's own-voxel emission is left out (the first segment of every
 // ray, as k_solve_hdda_t with EXT).
 // SPLIT: a CTA's warps share the directions of one 8 x 4 tile (split_solve).
-template <int ST, bool COUNT, bool EXT, bool SPLIT>
+// TWIN: for the solve that walks once per batch: only pairs whose blocks all have
+// the same levels (states_agree), for which the shared walk is each batch's own.
+// Where a batch's records have no bound (a source function that overflowed, say) each
+// batch is walked by itself, as a pair with itself: there a ray must end where its
+// own batch's transmissions do.
+template <int ST, bool COUNT, bool EXT, bool SPLIT, bool TWIN = false>
 __global__ void __launch_bounds__(pair_threads<ST>(), pair_min_blocks<ST>()) k_solve_hdda_pair(const HddaParams P)
 {
     using Model = PairModel<ST>;
@@ -75,6 +80,9 @@ __global__ void __launch_bounds__(pair_threads<ST>(), pair_min_blocks<ST>()) k_s
     const int tid = threadIdx.x;
     const unsigned long long* w1 = P.words + (size_t)b1 * P.n_words;
     const unsigned long long* w2 = P.words + (size_t)b2 * P.n_words;
+    if constexpr (TWIN) {
+        if (!states_agree(w1, w2, P.n_words)) return;
+    }
     const int n_blocks = P.nbx * P.nbz;
     for (int q = tid; q < n_blocks; q += blockDim.x)
         s_info[q] = pack_block_info(P.block_offset[q], min(block_state(w1, q), block_state(w2, q)));
@@ -138,10 +146,13 @@ __global__ void __launch_bounds__(pair_threads<ST>(), pair_min_blocks<ST>()) k_s
 #pragma unroll
     for (int q = 0; q < 4; ++q) G.band[q] = P.band[q];
     G.stop = -1.0f;
+    [[maybe_unused]] float bound1 = 0.0f, bound2 = 0.0f;
     if (!COUNT && P.scanned) {
-        G.stop = stop_factor(join_bounds(P.J[(size_t)(b1 * 8) * P.n_cells + cell], P.J[(size_t)(b2 * 8) * P.n_cells + cell]), P.i_bc);
+        bound1 = P.J[(size_t)(b1 * 8) * P.n_cells + cell];
+        bound2 = P.J[(size_t)(b2 * 8) * P.n_cells + cell];
+        G.stop = stop_factor(join_bounds(bound1, bound2), P.i_bc);
     }
-    const typename Model::Params M{(long long)(b2 - b1) * (long long)batch_floats};
+    typename Model::Params M{(long long)(b2 - b1) * (long long)batch_floats};
     const int mip0 = min(state0, distance_cap(G, 0.0f));
     unsigned int nseg = 0;
     bool capped = false;
@@ -160,38 +171,64 @@ __global__ void __launch_bounds__(pair_threads<ST>(), pair_min_blocks<ST>()) k_s
         if (P.I != nullptr && lambda(w) < P.n_lambda)
             P.I[((size_t)lambda(w) * P.quad.n_dir + k) * P.n_cells + cell] = Iw;
     };
-    if constexpr (SPLIT) {
-        __shared__ int s_next;
-        split_solve<16, NW>(
-            P.quad, reinterpret_cast<float*>(s_info) + P.split_at, &s_next, wrp, lane,
-            [&](int k, float* out) {
+    [[maybe_unused]] __shared__ int s_next;
+    auto solve = [&]() {
+        if constexpr (SPLIT) {
+            split_solve<16, NW>(
+                P.quad, reinterpret_cast<float*>(s_info) + P.split_at, &s_next, wrp, lane,
+                [&](int k, float* out) {
+                    float I[16], T[16];
+                    ray(k, I, T);
+#pragma unroll
+                    for (int w = 0; w < 16; ++w) {
+                        const float Iw = fmaf(T[w], P.i_bc, I[w]);
+                        out[w * 32] = Iw;
+                        store_I(w, k, Iw);
+                    }
+                },
+                [&](int w, float J) {
+                    if (lambda(w) < P.n_lambda) P.J[(size_t)lambda(w) * P.n_cells + cell] = J;
+                });
+        } else {
+            for (int k = 0; k < P.quad.n_dir; ++k) {
                 float I[16], T[16];
                 ray(k, I, T);
+                const float wk = P.quad.w[k];
 #pragma unroll
                 for (int w = 0; w < 16; ++w) {
                     const float Iw = fmaf(T[w], P.i_bc, I[w]);
-                    out[w * 32] = Iw;
+                    s_J[w][tid] = fmaf(wk, Iw, s_J[w][tid]);
                     store_I(w, k, Iw);
                 }
-            },
-            [&](int w, float J) {
-                if (lambda(w) < P.n_lambda) P.J[(size_t)lambda(w) * P.n_cells + cell] = J;
-            });
-    } else {
-        for (int k = 0; k < P.quad.n_dir; ++k) {
-            float I[16], T[16];
-            ray(k, I, T);
-            const float wk = P.quad.w[k];
+            }
 #pragma unroll
-            for (int w = 0; w < 16; ++w) {
-                const float Iw = fmaf(T[w], P.i_bc, I[w]);
-                s_J[w][tid] = fmaf(wk, Iw, s_J[w][tid]);
-                store_I(w, k, Iw);
+            for (int w = 0; w < 16; ++w)
+                if (lambda(w) < P.n_lambda) P.J[(size_t)lambda(w) * P.n_cells + cell] = s_J[w][tid];
+        }
+    };
+    if constexpr (TWIN) {
+        const int second = b2;
+        const long long off = M.off;
+        bool apart = join_bounds(bound1, bound2) < 0.0f;
+        if (apart) {
+            b2 = b1;
+            M.off = 0;
+            G.stop = stop_factor(bound1, P.i_bc);
+        }
+        for (;;) {
+            solve();
+            if (!apart) break;
+            apart = false;
+            b1 = b2 = second;
+            G.batch_base += off;
+            G.stop = stop_factor(bound2, P.i_bc);
+            if constexpr (!SPLIT) {
+#pragma unroll
+                for (int w = 0; w < 16; ++w) s_J[w][tid] = 0.0f;
             }
         }
-#pragma unroll
-        for (int w = 0; w < 16; ++w)
-            if (lambda(w) < P.n_lambda) P.J[(size_t)lambda(w) * P.n_cells + cell] = s_J[w][tid];
+    } else {
+        solve();
     }
     if (capped) raise_status(P.status, DEX_ERR_TRAVERSAL_CAP);
     // segments of the two batches
@@ -199,7 +236,7 @@ __global__ void __launch_bounds__(pair_threads<ST>(), pair_min_blocks<ST>()) k_s
 }
 
 template <int ST>
-cudaError_t launch_pair(cudaStream_t s, const HddaParams& P0)
+cudaError_t launch_pair(cudaStream_t s, const HddaParams& P0, bool twin = false)
 {
     HddaParams P = P0;
     const unsigned pairs = (unsigned)pair_count(P.n_batch, P.pair_group);
@@ -209,6 +246,8 @@ cudaError_t launch_pair(cudaStream_t s, const HddaParams& P0)
     const dim3 grid((unsigned)P.cap_active * (split ? 8u : (unsigned)pair_parts<ST>()), pairs);
     auto kernel = P.seg_count ? (P.exclude_own ? k_solve_hdda_pair<ST, true, true, false>
                                                : k_solve_hdda_pair<ST, true, false, false>)
+                  : twin      ? (split ? k_solve_hdda_pair<ST, false, false, true, true>
+                                       : k_solve_hdda_pair<ST, false, false, false, true>)
                   : split     ? (P.exclude_own ? k_solve_hdda_pair<ST, false, true, true>
                                                : k_solve_hdda_pair<ST, false, false, true>)
                               : (P.exclude_own ? k_solve_hdda_pair<ST, false, true, false>
@@ -228,6 +267,16 @@ bool solve_hdda_paired_applies(const HddaParams& P)
     const long long n_blocks = (long long)P.nbx * P.nbz;
     return P.traversal == DEX_TRAVERSAL_PAIRED && P.W == 8 && n_blocks <= kPairInfoMaxBlocks &&
            (!P.exclude_own || P.storage == kStoreF32);
+}
+
+cudaError_t launch_solve_hdda_twins(cudaStream_t s, const HddaParams& P)
+{
+    switch (P.storage) {
+        case kStoreF32: return launch_pair<kStoreF32>(s, P, true);
+        case kStoreBF16: return launch_pair<kStoreBF16>(s, P, true);
+        case kStoreF16: return launch_pair<kStoreF16>(s, P, true);
+        default: return cudaErrorInvalidValue;
+    }
 }
 
 cudaError_t launch_solve_hdda_paired(cudaStream_t s, const HddaParams& P)
