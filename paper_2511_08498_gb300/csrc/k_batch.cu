@@ -64,10 +64,10 @@ struct StaticRec {
 // kPair (W = 8): a work unit is a pair of batches (pair_batches) walked once on
 // the smaller of their two levels, 16 wavelengths per thread, or a lone batch
 // (pair_lone_batch) walked alone, as dex_formal_solve_hdda's paired walk.
-// P.twins: with kPair only the pairs whose blocks all have the same levels, without it
-// the batches of no such pair, as the TWIN walk of k_solve_hdda_pair and the per-batch
-// walk beside it.
-template <int W, int NT, bool kInfo, int kMinCtas, bool kPair = false>
+// kTwin (W = 8): with kPair the pairs whose blocks all have the same levels, as the TWIN
+// walk of k_solve_hdda_pair, without it the batches of no such pair (kernels of their
+// own: the check in the others' loop cost the small launches 2 to 3%).
+template <int W, int NT, bool kInfo, int kMinCtas, bool kPair = false, bool kTwin = false>
 __global__ void __launch_bounds__(NT, kMinCtas) k_batch_solve(const BatchParams P)
 {
     extern __shared__ unsigned long long s_dyn[];
@@ -77,7 +77,8 @@ __global__ void __launch_bounds__(NT, kMinCtas) k_batch_solve(const BatchParams 
     constexpr int kParts = 256 / NT;
     int* s_info = reinterpret_cast<int*>(s_dyn);
     const int tid = threadIdx.x;
-    int cur_atm = -1, cur_batch = -1, skip_atm = -1, skip_batch = -1;
+    int cur_atm = -1, cur_batch = -1;
+    [[maybe_unused]] int skip_atm = -1, skip_batch = -1;
     unsigned int nseg_unused = 0;
     bool capped = false;
     if (P.start_ns != nullptr && tid == 0) atomicMin(P.start_ns, global_ns());
@@ -98,7 +99,7 @@ __global__ void __launch_bounds__(NT, kMinCtas) k_batch_solve(const BatchParams 
             const long long unit = local / kParts;
             const int part = (int)(local % kParts);
             const int b = (int)(unit / A.cap_active), r = (int)(unit % A.cap_active);
-            if (r >= *A.n_active || (a == skip_atm && b == skip_batch)) continue;
+            if (r >= *A.n_active || (kTwin && a == skip_atm && b == skip_batch)) continue;
             // kPair: b numbers the atmosphere's pairs, then its lone batches
             int b1 = b, b2 = -1;
             if constexpr (kPair) {
@@ -108,16 +109,14 @@ __global__ void __launch_bounds__(NT, kMinCtas) k_batch_solve(const BatchParams 
             }
             __syncthreads();  // every thread is done with the previous item's shared data
             if (a != cur_atm || b != cur_batch) {
-                if constexpr (W == 8) {
-                    if (P.twins) {
-                        const int other = kPair ? (b2 >= 0 ? b2 : b1) : pair_partner(b, (A.n_lambda + W - 1) / W, P.pair_group);
-                        const bool twins = other != b1 && states_agree(A.words + (size_t)b1 * A.n_words,
-                                                                       A.words + (size_t)other * A.n_words, A.n_words);
-                        if (twins != kPair) {
-                            skip_atm = a;
-                            skip_batch = b;
-                            continue;
-                        }
+                if constexpr (kTwin) {
+                    const int other = kPair ? (b2 >= 0 ? b2 : b1) : pair_partner(b, (A.n_lambda + W - 1) / W, P.pair_group);
+                    const bool twins = other != b1 && states_agree(A.words + (size_t)b1 * A.n_words,
+                                                                   A.words + (size_t)other * A.n_words, A.n_words);
+                    if (twins != kPair) {
+                        skip_atm = a;
+                        skip_batch = b;
+                        continue;
                     }
                 }
                 if constexpr (kPair) {
@@ -174,24 +173,24 @@ __global__ void __launch_bounds__(NT, kMinCtas) k_batch_solve(const BatchParams 
             const size_t plane = (size_t)W * A.nx * A.nz;
             float bound = A.J[b1 * plane + cell];
             [[maybe_unused]] float bound2 = 0.0f;
-            [[maybe_unused]] int second = -1;  // a batch to be walked by itself after b1
+            [[maybe_unused]] int second = -1;  // kTwin: a batch to be walked by itself after b1
             if (kPair && b2 >= 0) {
                 bound2 = A.J[b2 * plane + cell];
-                if (P.twins && join_bounds(bound, bound2) < 0.0f) {
+                if (kTwin && join_bounds(bound, bound2) < 0.0f) {
                     second = b2;
                     b2 = b1;
                 } else {
                     bound = join_bounds(bound, bound2);
                 }
             }
+            G.stop = stop_factor(bound, A.i_bc);
             const int mip0 = min(state0, distance_cap(G, 0.0f));
             typename StaticRec<W>::Params M{};
             const long long n_cells = (long long)A.nx * A.nz;
-            for (;;) {
-                G.stop = stop_factor(bound, A.i_bc);
+            auto solve = [&]() {
                 for (int k = 0; k < A.n_dir; ++k) {
                     const float wk = s_w[k];
-                    if (kPair && b2 >= 0) {
+                    if ((kPair && kTwin) || (kPair && b2 >= 0)) {
                         // the pair: 16 wavelengths along one walk
                         using PM = PairRecModel<kStoreF32, kMinCtas>;
                         const typename PM::Params M2{(long long)(b2 - b1) * (long long)batch_floats};
@@ -222,13 +221,20 @@ __global__ void __launch_bounds__(NT, kMinCtas) k_batch_solve(const BatchParams 
                     const int l = w < W ? b1 * W + w : b2 * W + (w - W);
                     if ((w < W || b2 >= 0) && l < A.n_lambda) A.J[(size_t)l * n_cells + (size_t)j * A.nx + i] = s_J[w][tid];
                 }
-                if (!kPair || second < 0) break;
-                G.batch_base += (size_t)(second - b1) * batch_floats;
-                b1 = b2 = second;
-                second = -1;
-                bound = bound2;
+            };
+            if constexpr (kPair && kTwin) {
+                for (;;) {
+                    solve();
+                    if (second < 0) break;
+                    G.batch_base += (size_t)(second - b1) * batch_floats;
+                    b1 = b2 = second;
+                    second = -1;
+                    G.stop = stop_factor(bound2, A.i_bc);
 #pragma unroll
-                for (int w = 0; w < 2 * W; ++w) s_J[w][tid] = 0.0f;
+                    for (int w = 0; w < 2 * W; ++w) s_J[w][tid] = 0.0f;
+                }
+            } else {
+                solve();
             }
             if (P.done_ns != nullptr) {
                 __syncthreads();
@@ -290,10 +296,10 @@ void scan_batch(cudaStream_t s, const BatchParams& P)
     k_spread_batch<W><<<spread, 256, 0, s>>>(P);
 }
 
-template <int W, int NT, bool kInfo, int kMinCtas, bool kPair = false>
+template <int W, int NT, bool kInfo, int kMinCtas, bool kPair = false, bool kTwin = false>
 cudaError_t launch_batch_t(cudaStream_t s, const BatchParams& P, int ctas, size_t smem)
 {
-    auto kernel = k_batch_solve<W, NT, kInfo, kMinCtas, kPair>;
+    auto kernel = k_batch_solve<W, NT, kInfo, kMinCtas, kPair, kTwin>;
     if (smem > 16 * 1024) {
         cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         if (e != cudaSuccess) return e;
@@ -302,16 +308,16 @@ cudaError_t launch_batch_t(cudaStream_t s, const BatchParams& P, int ctas, size_
     return cudaSuccess;
 }
 
-template <int W, bool kOcc>
+template <int W, bool kOcc, bool kTwin = false>
 cudaError_t launch_batch_w(cudaStream_t s, const BatchParams& P, int ctas, int packet, bool info, size_t smem)
 {
     switch (packet * 2 + (info ? 1 : 0)) {
-        case 256 * 2: return launch_batch_t<W, 256, false, kOcc ? 4 : 3>(s, P, ctas, smem);
-        case 256 * 2 + 1: return launch_batch_t<W, 256, true, kOcc ? 4 : 3>(s, P, ctas, smem);
-        case 128 * 2: return launch_batch_t<W, 128, false, kOcc ? 8 : 6>(s, P, ctas, smem);
-        case 128 * 2 + 1: return launch_batch_t<W, 128, true, kOcc ? 8 : 6>(s, P, ctas, smem);
-        case 64 * 2: return launch_batch_t<W, 64, false, kOcc ? 16 : 12>(s, P, ctas, smem);
-        case 64 * 2 + 1: return launch_batch_t<W, 64, true, kOcc ? 16 : 12>(s, P, ctas, smem);
+        case 256 * 2: return launch_batch_t<W, 256, false, kOcc ? 4 : 3, false, kTwin>(s, P, ctas, smem);
+        case 256 * 2 + 1: return launch_batch_t<W, 256, true, kOcc ? 4 : 3, false, kTwin>(s, P, ctas, smem);
+        case 128 * 2: return launch_batch_t<W, 128, false, kOcc ? 8 : 6, false, kTwin>(s, P, ctas, smem);
+        case 128 * 2 + 1: return launch_batch_t<W, 128, true, kOcc ? 8 : 6, false, kTwin>(s, P, ctas, smem);
+        case 64 * 2: return launch_batch_t<W, 64, false, kOcc ? 16 : 12, false, kTwin>(s, P, ctas, smem);
+        case 64 * 2 + 1: return launch_batch_t<W, 64, true, kOcc ? 16 : 12, false, kTwin>(s, P, ctas, smem);
         default: return cudaErrorInvalidValue;
     }
 }
@@ -336,8 +342,8 @@ cudaError_t noalloc_scratch(unsigned int** out)
 // enough blocks of pairs that the second launch's start, after the last item of the
 // first, costs less than the shared walks give.  Eight to twelve atmospheres of static
 // lines (about half of the pairs agree), one walk per batch -> with pairs: 3168 blocks of
-// pairs 23.9 -> 22.0 ms, 3904 40.1 -> 35.8, 6784 73.9 -> 64.1; but 2816 13.95 -> 13.99,
-// 1968 13.6 -> 14.9, 352 3.5 -> 5.0.
+// pairs 23.4 -> 22.1 ms, 3904 39.4 -> 36.5, 6784 72.6 -> 64.9; but 2816 13.6 -> 14.2,
+// 1968 13.5 -> 15.4, 352 3.5 -> 5.1.
 constexpr long long kTwinItems = 3040;  // ten rounds of the pair kernel's 304 resident CTAs
 
 static bool twins_apply(const BatchParams& P, int W, size_t max_blocks)
@@ -349,10 +355,9 @@ static bool twins_apply(const BatchParams& P, int W, size_t max_blocks)
     return pairs >= kTwinItems;
 }
 
-cudaError_t launch_batch_solve(cudaStream_t s, const BatchParams& P0, int ctas, int W, int packet, bool info,
+cudaError_t launch_batch_solve(cudaStream_t s, const BatchParams& P, int ctas, int W, int packet, bool info,
                                bool occupancy, size_t max_words, size_t max_blocks)
 {
-    BatchParams P = P0;
     const size_t smem_bytes = info ? sizeof(int) * max_blocks : sizeof(unsigned long long) * max_words;
     cudaError_t e = cudaMemsetAsync(P.queue, 0, sizeof(unsigned int), s);
     if (e != cudaSuccess || P.n_items == 0) return e;
@@ -366,28 +371,30 @@ cudaError_t launch_batch_solve(cudaStream_t s, const BatchParams& P0, int ctas, 
     }
     // pairs of batches (W = 8): one word per block staged, the compiler's budget
     // bounded at 128 registers (two 256-thread CTAs per SM)
-    auto launch_pairs = [&](const BatchParams& Q) {
+    auto launch_pairs = [&](const BatchParams& Q, auto twin) {
+        constexpr bool kTwin = decltype(twin)::value;
+        const size_t smem = sizeof(int) * max_blocks;
         switch (packet) {
-            case 256: return launch_batch_t<8, 256, true, 2, true>(s, Q, ctas, sizeof(int) * max_blocks);
-            case 128: return launch_batch_t<8, 128, true, 4, true>(s, Q, ctas, sizeof(int) * max_blocks);
-            case 64: return launch_batch_t<8, 64, true, 8, true>(s, Q, ctas, sizeof(int) * max_blocks);
+            case 256: return launch_batch_t<8, 256, true, 2, true, kTwin>(s, Q, ctas, smem);
+            case 128: return launch_batch_t<8, 128, true, 4, true, kTwin>(s, Q, ctas, smem);
+            case 64: return launch_batch_t<8, 64, true, 8, true, kTwin>(s, Q, ctas, smem);
             default: return cudaErrorInvalidValue;
         }
     };
     if (P.paired) {
         if (W != 8) return cudaErrorInvalidValue;
-        if ((e = launch_pairs(P)) != cudaSuccess) return e;
+        if ((e = launch_pairs(P, std::false_type{})) != cudaSuccess) return e;
         return cudaGetLastError();
     }
-    P.twins = twins_apply(P, W, max_blocks);
-    if (P.twins) {
+    const bool twins = twins_apply(P, W, max_blocks);
+    if (twins) {
         BatchParams Q = P;
         Q.n_items = 0;
         for (int a = 0; a < P.n_atm; ++a) {
             Q.atm[a].item_base = Q.n_items;
             Q.n_items += (long long)pair_count((P.atm[a].n_lambda + 7) / 8, P.pair_group) * P.atm[a].cap_active * P.parts;
         }
-        if ((e = launch_pairs(Q)) != cudaSuccess) return e;
+        if ((e = launch_pairs(Q, std::true_type{})) != cudaSuccess) return e;
         if ((e = cudaMemsetAsync(P.queue, 0, sizeof(unsigned int), s)) != cudaSuccess) return e;
     }
     switch (W) {
@@ -395,8 +402,12 @@ cudaError_t launch_batch_solve(cudaStream_t s, const BatchParams& P0, int ctas, 
         case 2: e = launch_batch_w<2, false>(s, P, ctas, packet, info, smem_bytes); break;
         case 4: e = launch_batch_w<4, false>(s, P, ctas, packet, info, smem_bytes); break;
         case 8:
-            e = occupancy ? launch_batch_w<8, true>(s, P, ctas, packet, info, smem_bytes)
-                          : launch_batch_w<8, false>(s, P, ctas, packet, info, smem_bytes);
+            if (twins)
+                e = occupancy ? launch_batch_w<8, true, true>(s, P, ctas, packet, info, smem_bytes)
+                              : launch_batch_w<8, false, true>(s, P, ctas, packet, info, smem_bytes);
+            else
+                e = occupancy ? launch_batch_w<8, true>(s, P, ctas, packet, info, smem_bytes)
+                              : launch_batch_w<8, false>(s, P, ctas, packet, info, smem_bytes);
             break;
         default: return cudaErrorInvalidValue;
     }
