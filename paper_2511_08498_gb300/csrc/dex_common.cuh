@@ -166,6 +166,15 @@ __device__ __forceinline__ bool ray_done(const float* I, const float* T, float s
     return !(m > 0.0f);
 }
 
+// Whether two batches have the same level in every block (all threads of the CTA).
+// A walk shared by the two then takes, at every step, the levels of each one's own.
+__device__ __forceinline__ bool states_agree(const unsigned long long* w1, const unsigned long long* w2, int n_words)
+{
+    bool differ = false;
+    for (int q = threadIdx.x; q < n_words; q += blockDim.x) differ |= __ldg(w1 + q) != __ldg(w2 + q);
+    return !__syncthreads_or(differ);
+}
+
 // All W wavelengths of a record: pairs on the packed pipe, an odd one alone.
 template <int W>
 __device__ __forceinline__ void segments(const float* S, const float* chi, float nl2, float* I, float* T)

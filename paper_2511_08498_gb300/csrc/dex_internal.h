@@ -271,7 +271,6 @@ struct BatchParams {
     long long n_items;
     int paired;             // W = 8: work units are pairs of batches (pair_batches) and lone batches
     int pair_group;         //   paired within groups of this many batches (0: one group)
-    int twins;              // one walk per batch, as HddaParams::twins
     int parts;              // work items per active block and batch: 256 / probes per item
     int chunk;              // work items claimed per queue increment
     unsigned int* queue;
@@ -407,6 +406,7 @@ struct Hdda3Params {
     int traversal;  // DEX_TRAVERSAL_PAIRED: one walk per pair of batches; otherwise one per batch
     int pair_group; // batches paired within groups of this many (0: one group), as HddaParams
     int scanned;    // J holds the bounds of the exact early termination, as HddaParams
+    int twins;      // as HddaParams
     int n_band;
     float band[4];
     long long n_cells;

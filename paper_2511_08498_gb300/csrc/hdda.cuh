@@ -403,15 +403,6 @@ __device__ __forceinline__ void split_solve(const Quadrature& quad, float* s_I, 
         if (warp + q * NW < W) store(warp + q * NW, J[q]);
 }
 
-// Whether two batches have the same level in every block (all threads of the CTA).
-// A walk shared by the two then takes, at every step, the levels of each one's own.
-__device__ __forceinline__ bool states_agree(const unsigned long long* w1, const unsigned long long* w2, int n_words)
-{
-    bool differ = false;
-    for (int q = threadIdx.x; q < n_words; q += blockDim.x) differ |= __ldg(w1 + q) != __ldg(w2 + q);
-    return !__syncthreads_or(differ);
-}
-
 // kInfo: the CTA stages one word per block (offset * 8 + state, InfoLookup;
 // dynamic shared memory 4 * nbx * nbz bytes, grids of at most kInfoMaxBlocks
 // blocks); otherwise the packed state words (WordLookup; 8 * n_words bytes).

@@ -217,7 +217,9 @@ __device__ __forceinline__ unsigned long long min_states(unsigned long long a, u
 // (active block, pair of batches, pair_batches), walking once for both on the
 // smaller of their levels (the state words must fit in shared memory).
 // INFO: the CTA stages one word per block (grids of at most kMaxInfo3 blocks).
-template <int W, bool COUNT, int ST, int NB, bool INFO>
+// TWIN (NB = 2): for the solve that walks once per batch, only the pairs whose blocks all
+// have the same levels, batch by batch where a batch has no bound, as k_solve_hdda_pair.
+template <int W, bool COUNT, int ST, int NB, bool INFO, bool TWIN = false>
 __global__ void __launch_bounds__(kThreads3, NB == 1 ? kMinBlocks3 : 2) k_solve_hdda3(const Hdda3Params P)
 {
     extern __shared__ unsigned long long s_words[];
@@ -228,6 +230,14 @@ __global__ void __launch_bounds__(kThreads3, NB == 1 ? kMinBlocks3 : 2) k_solve_
     if constexpr (NB == 2) pair_batches(blockIdx.y, P.n_batch, P.pair_group, b, b2);
     const int tid = threadIdx.x;
     const unsigned long long* gw = P.words + (size_t)b * P.n_words;
+    if constexpr (TWIN) {
+        if (!states_agree(gw, P.words + (size_t)b2 * P.n_words, P.n_words)) return;
+    } else if constexpr (NB == 1 && W == 8 && INFO && !COUNT) {
+        if (P.twins) {  // walked with its partner if their levels agree
+            const int other = pair_partner(b, P.n_batch, P.pair_group);
+            if (other != b && states_agree(gw, P.words + (size_t)other * P.n_words, P.n_words)) return;
+        }
+    }
     int* s_info = reinterpret_cast<int*>(s_words);
     const bool staged = !INFO && (NB == 2 || P.n_words <= kMaxStagedWords);
     if constexpr (INFO) {
@@ -257,7 +267,7 @@ __global__ void __launch_bounds__(kThreads3, NB == 1 ? kMinBlocks3 : 2) k_solve_
     constexpr int REC = RecFmt<W, ST>::kStride;
     const size_t batch_floats = (size_t)P.cap_active * P.chain * REC;
     const float* base = P.bricks + (size_t)b * batch_floats;
-    const long long off = (long long)(b2 - b) * (long long)batch_floats;
+    long long off = (long long)(b2 - b) * (long long)batch_floats;
     const int mip0 = min(state0, distance_cap3(P, 0.0f));
     unsigned int nseg = 0;
     bool capped = false;
@@ -270,33 +280,53 @@ __global__ void __launch_bounds__(kThreads3, NB == 1 ? kMinBlocks3 : 2) k_solve_
         // I and T take the registers)
         float Jr[NB == 1 ? W : 1];
         auto Jw = [&](int w) -> float& { return NB == 1 ? Jr[NB == 1 ? w : 0] : s_J3[w][tid]; };
-#pragma unroll
-        for (int w = 0; w < NB * W; ++w) Jw(w) = 0.0f;
         float stop = -1.0f;
+        [[maybe_unused]] bool apart = false;
+        [[maybe_unused]] float bound2 = 0.0f;
+        [[maybe_unused]] const int second = b2;
+        [[maybe_unused]] const long long off2 = off;
         if (!COUNT && P.scanned) {  // the bounds wait where this probe's J will go
             float m = P.J[(size_t)(b * W) * P.n_cells + cell];
-            if (NB == 2) m = join_bounds(m, P.J[(size_t)(b2 * W) * P.n_cells + cell]);
+            if constexpr (NB == 2) {
+                bound2 = P.J[(size_t)(b2 * W) * P.n_cells + cell];
+                if (TWIN && join_bounds(m, bound2) < 0.0f) {  // each batch by itself, as a pair with itself
+                    apart = true;
+                    b2 = b;
+                    off = 0;
+                } else {
+                    m = join_bounds(m, bound2);
+                }
+            }
             stop = stop_factor(m, P.i_bc);
         }
-        for (int q = 0; q < P.quad.n_dir; ++q) {
-            float I[NB * W], T[NB * W];
+        for (;;) {
 #pragma unroll
-            for (int w = 0; w < NB * W; ++w) { I[w] = 0.0f; T[w] = 1.0f; }
-            trace_ray3<W, COUNT, ST, NB, INFO>(P, base, off, i, j, k, bx0, by0, bz0, a0, mip0, P.quad.dx[q], P.quad.dy[q],
-                                         P.quad.dz[q], words, s_info, stop, I, T, nseg, capped);
-            const float wk = P.quad.w[q];
+            for (int w = 0; w < NB * W; ++w) Jw(w) = 0.0f;
+            for (int q = 0; q < P.quad.n_dir; ++q) {
+                float I[NB * W], T[NB * W];
+#pragma unroll
+                for (int w = 0; w < NB * W; ++w) { I[w] = 0.0f; T[w] = 1.0f; }
+                trace_ray3<W, COUNT, ST, NB, INFO>(P, base, off, i, j, k, bx0, by0, bz0, a0, mip0, P.quad.dx[q], P.quad.dy[q],
+                                             P.quad.dz[q], words, s_info, stop, I, T, nseg, capped);
+                const float wk = P.quad.w[q];
+#pragma unroll
+                for (int w = 0; w < NB * W; ++w) {
+                    const float Iw = fmaf(T[w], P.i_bc, I[w]);
+                    Jw(w) = fmaf(wk, Iw, Jw(w));
+                    const int l = w < W ? b * W + w : b2 * W + (w - W);
+                    if (P.I != nullptr && l < P.n_lambda) P.I[((size_t)l * P.quad.n_dir + q) * P.n_cells + cell] = Iw;
+                }
+            }
 #pragma unroll
             for (int w = 0; w < NB * W; ++w) {
-                const float Iw = fmaf(T[w], P.i_bc, I[w]);
-                Jw(w) = fmaf(wk, Iw, Jw(w));
                 const int l = w < W ? b * W + w : b2 * W + (w - W);
-                if (P.I != nullptr && l < P.n_lambda) P.I[((size_t)l * P.quad.n_dir + q) * P.n_cells + cell] = Iw;
+                if (l < P.n_lambda) P.J[(size_t)l * P.n_cells + cell] = Jw(w);
             }
-        }
-#pragma unroll
-        for (int w = 0; w < NB * W; ++w) {
-            const int l = w < W ? b * W + w : b2 * W + (w - W);
-            if (l < P.n_lambda) P.J[(size_t)l * P.n_cells + cell] = Jw(w);
+            if (!TWIN || !apart) break;
+            apart = false;
+            b = b2 = second;
+            base += off2;
+            stop = stop_factor(bound2, P.i_bc);
         }
     }
     if (capped) raise_status(P.status, DEX_ERR_TRAVERSAL_CAP);
@@ -377,6 +407,17 @@ cudaError_t launch3(K kernel, dim3 grid, size_t smem, cudaStream_t s, const Hdda
 
 }  // namespace
 
+// Where the per-batch walk looks for pairs it may walk once: grids with the block table
+// whose pairs alone fill the chip one and a half times (304 resident CTAs).  Static
+// lines, 16 directions, one walk per batch -> with pairs: 128 x 96 x 80, 32 wavelengths
+// 13.5 -> 11.0 ms, 24 (a lone batch) 9.08 -> 8.09; 48 x 40 x 40, 32 (600 CTAs) 0.882 ->
+// 0.830, 16 (300) 0.524 -> 0.537; 32^3, 32 (256) 0.488 -> 0.518.  Where the levels differ
+// the check costs under 1%.
+static bool twins_apply3(const Hdda3Params& P)
+{
+    return (long long)P.cap_active * kParts3 * pair_count(P.n_batch, P.pair_group) >= 456;
+}
+
 bool solve_hdda3_paired_applies(const Hdda3Params& P)
 {
     return P.W == 8 && P.n_words <= kMaxStagedWords;
@@ -436,6 +477,18 @@ cudaError_t launch_solve_hdda3(cudaStream_t s, const Hdda3Params& P0)
         return cudaSuccess;
     }
     const dim3 grid((unsigned)P.cap_active * kParts3, (unsigned)P.n_batch);
+    if (info && P.scanned && twins_apply3(P)) {
+        P.twins = 1;
+        const dim3 pairs((unsigned)P.cap_active * kParts3, (unsigned)pair_count(P.n_batch, P.pair_group));
+        switch (P.storage) {
+            case kStoreF32: e = launch3(k_solve_hdda3<8, false, kStoreF32, 2, true, true>, pairs, smem, s, P); break;
+            case kStoreBF16: e = launch3(k_solve_hdda3<8, false, kStoreBF16, 2, true, true>, pairs, smem, s, P); break;
+            case kStoreF16: e = launch3(k_solve_hdda3<8, false, kStoreF16, 2, true, true>, pairs, smem, s, P); break;
+            default: return cudaErrorInvalidValue;
+        }
+        if (e != cudaSuccess) return e;
+        if ((e = cudaGetLastError()) != cudaSuccess) return e;
+    }
     switch (P.W * 4 + P.storage) {
 #define DEX_LAUNCH3_(WW, ST, INFO)                                                          \
     e = P.seg_count ? launch3(k_solve_hdda3<WW, true, ST, 1, INFO>, grid, smem, s, P)       \

@@ -88,6 +88,23 @@ def test_records_without_a_bound(nx, nz, batch):
     ctx.check()
 
 
+@pytest.mark.parametrize("nx,ny,nz,L,storage", [(64, 48, 40, 16, 0), (40, 48, 64, 32, 1), (64, 48, 40, 20, 2),
+                                                (64, 64, 72, 24, 0)])
+def test_3d(nx, ny, nz, L, storage):
+    from paper_2511_08498_gb300 import api
+    ctx = ctx_()
+    dirs, w = synth.directions3(4, 2)
+    for mirrored, iod, band, i_bc, bad in ((True, 1e-2, BAND, 0.0, False), (False, 0.3, BAND, 0.2, False),
+                                           (False, 1e30, None, 0.4, False), (True, 1e-2, BAND, 0.3, storage == 0)):
+        eta, chi = medium(nx, nz, L, 930 + L, mirrored, log_chi=(-3.0, -2.0) if bad else (-3.0, 2.0), ny=ny)
+        grid = api.grid3_build(ctx, nx, ny, nz, eta, chi)
+        mips = api.mips3_build(ctx, grid, eta, chi, 8, 3, iod, iod, storage=storage)
+        if bad:
+            mips.bricks.view((L + 7) // 8, -1)[0, 0] = float("inf")
+        both(api.formal_solve_hdda3, ctx, grid, mips, dirs, w, band=band, i_bc=i_bc)
+    ctx.check()
+
+
 # enough blocks of pairs (3040) for the persistent launch to look for them: packets,
 # packed states and one word per block, queue chunks; an atmosphere of one batch among them
 @pytest.mark.parametrize("cfg", [None, dict(packet=64, staging=1, chunk=3), dict(packet=128, staging=0, occupancy=1)])
