@@ -190,7 +190,7 @@ class Workload:
         self.grid = None
         self.mips = None
         self.mips_by_storage = {}
-        self.launches_per_step = 5  # synth, block flags, block layout, mips build, hdda solve
+        self.launches_per_step = 7  # synth, block flags, block layout, mips build, bounds scan and spread, hdda solve
 
     def synth(self):
         d = self.dev
@@ -449,6 +449,9 @@ def native(args):
                      "peak_fp32_lane_ops_per_sm_clk": fp32_rate / n_sm / (sm_clock_mhz * 1e6),
                      "peak_ex2_per_sm_clk": ex2_rate / n_sm / (sm_clock_mhz * 1e6),
                      "kernel_ms": hdda_s * 1e3, "executed_seg_lambda": exec_seg_lambda,
+                     "executed_basis": "the counting solve's segments: it follows each ray until its "
+                                       "transmissions are exactly zero, the timed solve until the rest cannot "
+                                       "change a bit of I, so achieved and frac are upper bounds",
                      "hbm_algorithmic_gbs": exec_seg_lambda * 8 / hdda_s / 1e9,
                      "hbm_peak_gbs": float(peaks.get("hbm_gbs", 6800.0)), "peak_source": peak_src,
                      "hbm_binds": False,

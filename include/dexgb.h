@@ -312,7 +312,12 @@ int dex_mips_build(dex_ctx* ctx, int nx, int nz, int n_lambda, int W, const floa
  *       probe, coarser levels only further out; n_band = 0 forces level 0)
  *   J   device [n_lambda][nz][nx] output; zeroed by the call, written at probe cells
  *   I   device [n_lambda][n_dir][nz][nx] output or NULL (zeroed by the call)
- *   seg_count  device uint64 accumulator or NULL: adds the voxel segments integrated
+ *   seg_count  device uint64 accumulator or NULL: adds the voxel segments integrated.
+ *       A counting call follows every ray until its transmissions are exactly zero;
+ *       without a count rays end as soon as the rest cannot change a bit of I (J and I
+ *       are the same), so a timed call integrates fewer segments than are counted
+ * With one walk per batch (the default) and W = 8, two mirrored batches whose blocks all
+ * have the same levels share a walk; J and I are the same bit for bit.
  */
 int dex_formal_solve_hdda(dex_ctx* ctx, int nx, int nz, int n_lambda, int W, int max_mip, int storage,
                           const float* bricks,
@@ -432,9 +437,11 @@ int dex_max_rel_change(dex_ctx* ctx, int n_level, int n_cells, const float* temp
 
 /* ------------------------------------------------------------------ Voigt --
  *
- * Section 3.2: the Voigt function H(a, x) = Re w(x + i a) by HUM1WEI24
- * (Humlicek 1982 region I for |x| + a >= 15, Weideman 1994 with 24 terms
- * otherwise), float32; the form the Core-and-Voigt solver evaluates per segment.
+ * Section 3.2: the Voigt function H(a, x) = Re w(x + i a), float32, the form the
+ * Core-and-Voigt solver evaluates per segment: Humlicek's (1982) region I for
+ * |x| + a >= 15 as in HUM1WEI24; below that, for a < 0.25, Dawson's integral and the
+ * asymptotic series, in which nothing cancels in float32; for a >= 0.25 Weideman's
+ * (1994) 24 terms, with a continued fraction from |x| + a = 5.
  * a, x, h: device [n] (a >= 0).
  */
 int dex_voigt(dex_ctx* ctx, int n, const float* a, const float* x, float* h);
@@ -544,7 +551,8 @@ int dex_formal_solve_velinterp(dex_ctx* ctx, int nx, int nz, int n_lambda, int W
 
 /* ---------------------------------------------------- batched atmospheres --
  *
- * Many independent atmospheres solved by one persistent launch: a fixed grid of
+ * Many independent atmospheres solved by one persistent launch (two where enough
+ * wavelength batches may share walks, the pairs' and the others'): a fixed grid of
  * CTAs pulls work items (atmosphere, wavelength batch, active block) from a
  * device counter until none are left; each item is the 256-probe block solve of
  * dex_formal_solve_hdda (static records).  The atmospheres share the batch
@@ -595,8 +603,8 @@ int dex_batch_solve(dex_ctx* ctx, int n_atm, const dex_batch_item* atms, int W, 
  *            a thread, so that 1024 threads a SM are resident (some spilling)
  * Every probe accumulates J over the directions in one thread in the order of
  * dex_formal_solve_hdda, so J is bit-identical for every configuration.
- * dex_batch_solve is dex_batch_solve_config with {ctas, 256, 1, 0, 0}.  Invalid
- * values -> DEX_ERR_ARG.
+ * dex_batch_solve is dex_batch_solve_config with {ctas, 256, 1, s, 0}, s = 1 where
+ * every grid has at most 8192 blocks.  Invalid values -> DEX_ERR_ARG.
  * With the context's traversal set to DEX_TRAVERSAL_PAIRED (W = 8; every grid
  * of at most 8192 blocks, else DEX_ERR_UNSUPPORTED) the work units are each
  * atmosphere's pairs of batches (dex_ctx_set_pair_group) and lone batches, and
@@ -821,7 +829,8 @@ int dex_formal_solve_hdda3(dex_ctx* ctx, int nx, int ny, int nz, int n_lambda, i
  * at the lattice edge).  J = the mean of L over the n0 cascade-0 directions.
  */
 
-/* Floats of the workspace: 2 * n_batch * n0 * nx * nz * W (two cascades' merged radiance). */
+/* Floats of the workspace: 2 * n_batch * n0 * nx * nz * W (two cascades' merged radiance;
+ * the solve also keeps its tables of blocks in the part it does not need for them). */
 size_t dex_rc_workspace_floats(int nx, int nz, int n_lambda, int W, int n0);
 
 /*

@@ -30,22 +30,15 @@ namespace {
 // transmissions, two records loaded at the top of each step) takes about 125
 // registers with float32 records: 2 CTAs of 256 threads per SM.  Bfloat16
 // records hold half the registers and run at 5 CTAs of 128 threads (at most 102
-// registers).  Measured on the 1024^2 static-line solve (IoD 1e-2 / unlimited
-// averaging), float32 on brick rows:
-//   float32, 256 threads, 2 CTAs (this)          158.8 / 63.3 ms
-//   float32, 128 threads, 4 CTAs                 167.1 / 66.8 ms
-//   float32, 128 threads, 3 CTAs (160 registers) 168.0 / 67.5 ms
-//   float32, 64 threads, 8 CTAs                  167.6 / 67.4 ms
-//   float32, 256 threads, 1 CTA (194 registers)  204.5 / 82.0 ms
-// with float32 records of S and chi side by side (before the brick rows):
-//   float32, 256 threads, 2 CTAs                 173.6 / 62.8 ms
-//   float32, 128 threads, 5 CTAs (96 registers)  176.4 / 66.1 ms
-//   float32, 256 threads, 3 CTAs (80, spills)    294.4 / 106.1 ms
-//   bfloat16, 128 threads, 5 CTAs (this)         165.0 / 66.2 ms
-//   bfloat16, 256 threads, 2 CTAs                171.5 / 66.6 ms
-//   bfloat16, 128 threads, 6 CTAs (80 registers) 174.3 / 69.8 ms
-// and, for float32 at 256 threads, the step loop unrolled twice or not at all
-// +1.4%, records loaded after the stepping +3.7%.
+// registers).  Measured on the 1024^2 static-line solve at IoD 1e-2, float32 on
+// brick rows (the whole step, of which the solve is about 94%):
+//   256 threads, 2 CTAs (this)  94.9 ms     128 threads, 5 CTAs (96 registers)  98.2 ms
+//   128 threads, 4 CTAs         93.9        64 threads, 8 CTAs                  93.6
+// (every CTA stages the block table, 64 KB on the largest grids, of which two fit).
+// The bound: issue slots 63% and the FP32 pipe 58% busy at 16 warps, with 25 of 32
+// lanes active.  Before rays ended early on the bound of what is left the order was the
+// same, 158.8 ms for this shape and 294 ms at 3 CTAs (80 registers, spills); bfloat16
+// 165.0 (this), 171.5 at 256 threads and 2 CTAs, 174.3 at 128 and 6.
 template <int ST>
 constexpr int pair_threads() { return ST == kStoreBF16 ? 128 : 256; }
 template <int ST>

@@ -141,10 +141,9 @@ __device__ void stage_weights(SmemNet& net, unsigned char* W2, const float* __re
     if (t == 0) net.b3 = p[kB3];
 }
 
-// GELU of two hidden units on the packed FP32 pipe.  The special-function units
-// bound these kernels (2^x and a reciprocal per activation: 16 per SM and clock),
-// so the two logistic functions share one reciprocal, 1/a = b / (a b): three
-// special-function operations for two activations.  2^x is bounded at 2^60, below
+// GELU of two hidden units on the packed FP32 pipe.  The two logistic functions share
+// one reciprocal, 1/a = b / (a b): three special-function operations for two
+// activations instead of four, in kernels whose issue slots and FP32 pipe they share.  2^x is bounded at 2^60, below
 // which the product cannot overflow and above which the activation is 0 to 1e-17.
 struct Gelu2 {
     float2 z, z2, s;
