@@ -462,6 +462,8 @@ def native(args):
                                  "special-function units (see peak_basis)"},
         "plain": {"value": dense_seg_lambda / plain_s, "ms_per_step": plain_s * 1e3,
                   "kernel_ms": plain_kern_s * 1e3, "kernel_updates_per_s": plain_achieved * 1e9,
+                  "kernel_updates_basis": "dense-equivalent: rays end once the rest cannot change a bit of I, so "
+                                          "the rates and fractions are upper bounds",
                   "kernel_frac_of_peak": plain_achieved / peak,
                   "kernel_frac_of_sfu_peak": plain_achieved / sfu_peak,
                   "hbm_algorithmic_gbs": dense_seg_lambda * 8 / plain_kern_s / 1e9},

@@ -434,7 +434,8 @@ constexpr int kScanCtas = 304;
 
 // Grids of fewer warps (32 probes x batch) than two full loads of the chip's 152 x
 // 32 resident ones split the directions.  128 x 128, one wavelength, 16 directions:
-// 512 warps took 231 us one after the other, split 61 us.
+// 512 warps took 231 us one after the other, split 61 us (41 with a few records in
+// flight per ray).
 constexpr long long kSplitWarps = 2 * 152 * 32;
 
 
