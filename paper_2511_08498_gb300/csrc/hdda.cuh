@@ -104,6 +104,17 @@ struct Offset32Of<M, decltype((void)M::kOffset32)> {
     static constexpr bool value = M::kOffset32;
 };
 
+// Models for which pairs of batches may share a walk (k_solve_hdda_pair's) declare
+// kTwins = true.
+template <class M, class = void>
+struct TwinsOf {
+    static constexpr bool value = false;
+};
+template <class M>
+struct TwinsOf<M, decltype((void)M::kTwins)> {
+    static constexpr bool value = M::kTwins;
+};
+
 // Record load of a voxel model: Model::load(M, p) where the model declares it
 // (its records need the launch parameters, e.g. a second batch's offset),
 // Model::load(p) otherwise.
@@ -419,7 +430,7 @@ __global__ void __launch_bounds__(256, Model::kMinBlocks) k_solve_hdda_t(const H
     const int b = blockIdx.y;
     const int tid = threadIdx.x;
     const unsigned long long* words_b = P.words + (size_t)b * P.n_words;
-    if constexpr (Model::kPerBatch && W == 8 && !COUNT && !EXT) {
+    if constexpr (TwinsOf<Model>::value && W == 8 && !COUNT && !EXT) {
         // walked with its partner (k_solve_hdda_pair) if their levels agree
         if (P.twins) {
             const int b2 = pair_partner(b, P.n_batch, P.pair_group);

@@ -38,6 +38,7 @@ struct StaticModel {
     static constexpr int kSplitStride = BrickFmt<W, ST>::kX;
     static constexpr bool kPerBatch = true;
     static constexpr int kMinBlocks = 4;  // CTAs per SM the register budget targets
+    static constexpr bool kTwins = true;
     // record loaded at the top of each step: -3.3% (float32) on the 1024^2 benchmark
     // solve; +5% with the bfloat16 / float16 unpacking (register pressure)
     static constexpr bool kEarlyLoad = ST == kStoreF32;
