@@ -233,7 +233,7 @@ __global__ void __launch_bounds__(kTileThreads, 2) k_solve_dense_tile(const Dens
     const int i0 = blockIdx.x % tiles_x * 32, j0 = blockIdx.x / tiles_x * kTileRows;
     const int i = i0 + lane, j = j0 + warp;
     const bool probe = i < P.nx && j < P.nz;
-    const int p = j * P.nx + i;
+    const int p = (int)((unsigned)j * P.nx + i);
     const unsigned char* base = reinterpret_cast<const unsigned char*>(P.planes + (size_t)b * P.n_cells * 16);
     const float stop = P.scanned && probe ? stop_factor(P.J[(size_t)(b * 8) * P.n_probe + p], P.i_bc) : -1.0f;
     const uint32_t rec = (uint32_t)__cvta_generic_to_shared(s_rec) + (lane & 3) * kTilePlane + (lane >> 2) * 16;
@@ -336,7 +336,7 @@ __device__ __forceinline__ bool dense_probe(const DenseParams& P, int tile_rows,
         const int tx = blockIdx.x % tiles_x, tz = blockIdx.x / tiles_x;
         i = tx * 32 + lane;
         j = tz * tile_rows + row;
-        p = j * P.nx + i;
+        p = (int)((unsigned)j * P.nx + i);  // may wrap beyond the last row, where it is not used
         return i < P.nx && j < P.nz;
     }
     i = j = 0;
@@ -463,7 +463,9 @@ __global__ void __launch_bounds__(256) k_dense_spread(const DenseParams P, int n
     float m = 0.0f;
     for (int q = threadIdx.x; q < n_parts; q += blockDim.x) m = join_bounds(m, __ldcg(J + q));
     m = join_cta(m);
-    for (int p = blockIdx.x * blockDim.x + threadIdx.x; p < P.n_probe; p += gridDim.x * blockDim.x) J[p] = m;
+    // 64 bits: up to 2^31 - 1 probes, and the last step goes beyond them
+    for (long long p = blockIdx.x * (long long)blockDim.x + threadIdx.x; p < P.n_probe; p += gridDim.x * blockDim.x)
+        J[p] = m;
 }
 
 cudaError_t launch_dense_tile(cudaStream_t s, const DenseParams& P)
@@ -482,7 +484,7 @@ void launch_dense_scan(cudaStream_t s, const DenseParams& P)
 {
     const int parts = P.n_probe < kScanCtas ? P.n_probe : kScanCtas;
     k_dense_scan<W><<<dim3((unsigned)parts, (unsigned)P.n_batch), 256, 0, s>>>(P);
-    const int ctas = (P.n_probe + 1023) / 1024;
+    const long long ctas = (P.n_probe + 1023LL) / 1024;
     k_dense_spread<<<dim3((unsigned)(ctas < 304 ? ctas : 304), (unsigned)P.n_batch), 256, 0, s>>>(P, parts);
 }
 
@@ -540,7 +542,7 @@ cudaError_t launch_solve_dense(cudaStream_t s, const DenseParams& P0)
     }
     const int rows = split ? 1 : 8;
     const unsigned tiles = P.probes == nullptr ? (unsigned)(((P.nx + 31) / 32) * ((P.nz + rows - 1) / rows))
-                                               : (unsigned)((P.n_probe + 32 * rows - 1) / (32 * rows));
+                                               : (unsigned)((P.n_probe + 32LL * rows - 1) / (32 * rows));
     const dim3 grid(tiles, (unsigned)P.n_batch);
     switch (P.W) {
         case 1: launch_dense_w<1>(split, grid, s, P); break;
