@@ -63,18 +63,17 @@ __global__ void k_pack_planes(long long n_cells, int n_lambda, int W, int n_batc
 struct __align__(16) PathStep {
     float nl2;   // -length log2(e)
     float th;    // ray parameter of the crossed plane (rounded)
-    int off;     // cells from the probe's cell to the segment's
-    int moved;   // 1 where the segment's end is beyond its start (counted segments)
+    long long off;  // bytes from the probe's record to the segment's (grids of up to 2^32 cells)
 };
 
 // The crossings [c0, c0 + 32) of a direction, one per lane.
 struct PathBuilder {
     AxisParam ax, az;
     float sx, sz, fx;     // signs of the direction, |dx| / (|dx| + |dz|)
-    int stepx, stepz;     // cells per step
+    int stepx, stepz;     // bytes per step
     float th_last, tl_last;
 
-    __device__ __forceinline__ PathBuilder(float dx, float dz, int nx)
+    __device__ __forceinline__ PathBuilder(float dx, float dz, int nx, int rec_bytes)
     {
         // a zero component counts as positive, so its plane offsets are positive
         // and their parameters (offset * inf) are +inf: that axis never steps
@@ -83,8 +82,8 @@ struct PathBuilder {
         az = axis_param(dz);
         sx = negx ? -1.0f : 1.0f;
         sz = negz ? -1.0f : 1.0f;
-        stepx = negx ? -1 : 1;
-        stepz = negz ? -nx : nx;
+        stepx = negx ? -rec_bytes : rec_bytes;
+        stepz = stepx * (negx == negz ? nx : -nx);  // at most 64 x 65536 bytes
         fx = fabsf(dx) / (fabsf(dx) + fabsf(dz));
         th_last = tl_last = 0.0f;
     }
@@ -126,8 +125,7 @@ struct PathBuilder {
         PathStep s;
         s.nl2 = len * kNegLog2e;
         s.th = th;
-        s.off = m * stepx + n * stepz;
-        s.moved = th > th_prev;
+        s.off = (long long)m * stepx + (long long)n * stepz;
         return s;
     }
 };
@@ -145,7 +143,7 @@ __device__ __forceinline__ void dense_ray(const DenseParams& P, PathStep* path, 
                                           float* I, float* T, unsigned int& nseg)
 {
     constexpr int REC = 2 * W;
-    PathBuilder B(dx, dz, P.nx);
+    PathBuilder B(dx, dz, P.nx, REC * (int)sizeof(float));
     const float Ex = dx < 0.0f ? (float)(-i) - 0.5f : (float)(P.nx - i) - 0.5f;
     const float Ez = dz < 0.0f ? (float)(-j) - 0.5f : (float)(P.nz - j) - 0.5f;
     const float t2 = fminf(Ex * B.ax.ih, Ez * B.az.ih);
@@ -153,6 +151,7 @@ __device__ __forceinline__ void dense_ray(const DenseParams& P, PathStep* path, 
     for (int w = 0; w < W; ++w) { I[w] = 0.0f; T[w] = 1.0f; }
     constexpr int GROUP = W == 1 ? 8 : (W == 2 ? 4 : (W == 4 ? 2 : 1));
     float th_end = 0.0f;  // the last crossing of the chunk before
+    [[maybe_unused]] float th_count = 0.0f;
     // a ray crosses at most nx + nz planes
     for (int c0 = 0; c0 < P.nx + P.nz; c0 += 32) {
         int m;
@@ -171,7 +170,9 @@ __device__ __forceinline__ void dense_ray(const DenseParams& P, PathStep* path, 
 #pragma unroll
                 for (int g = 0; g < GROUP; ++g) {
                     s[g] = path[q0 + g];
-                    if (g == 0 || th_before < t2) r[g] = RecFmt<W, kStoreF32>::load(rec0 + (long long)s[g].off * REC);
+                    if (g == 0 || th_before < t2)
+                        r[g] = RecFmt<W, kStoreF32>::load(
+                            reinterpret_cast<const float*>(reinterpret_cast<const char*>(rec0) + s[g].off));
                     th_before = s[g].th;
                 }
 #pragma unroll
@@ -183,7 +184,10 @@ __device__ __forceinline__ void dense_ray(const DenseParams& P, PathStep* path, 
                             for (int w = 0; w < W; ++w) I[w] = 0.0f;
                         }
                     }
-                    if (COUNT) nseg += s[g].moved;
+                    if (COUNT) {
+                        nseg += s[g].th > th_count;  // segments whose end is beyond their start
+                        th_count = s[g].th;
+                    }
                     if (s[g].th >= t2) {
                         live = false;
                         break;
@@ -242,7 +246,7 @@ __global__ void __launch_bounds__(kTileThreads, 2) k_solve_dense_tile(const Dens
     for (int w = 0; w < 8; ++w) Jw[w] = 0.0f;
     for (int k = 0; k < P.quad.n_dir; ++k) {
         const float dx = P.quad.dx[k], dz = P.quad.dz[k];
-        PathBuilder B(dx, dz, P.nx);
+        PathBuilder B(dx, dz, P.nx, 64);
         const float Ex = dx < 0.0f ? (float)(-i) - 0.5f : (float)(P.nx - i) - 0.5f;
         const float Ez = dz < 0.0f ? (float)(-j) - 0.5f : (float)(P.nz - j) - 0.5f;
         const float t2 = fminf(Ex * B.ax.ih, Ez * B.az.ih);
@@ -284,18 +288,18 @@ __global__ void __launch_bounds__(kTileThreads, 2) k_solve_dense_tile(const Dens
                 const unsigned char* q0 = s_rec + (warp * rw + lane) * 16;
                 // the next step's record is read before this one is integrated
                 auto piece = [&](int off, int c) { return *reinterpret_cast<const float4*>(q0 + off + c * kTilePlane); };
-                PathStep ns = s_path[0];
-                float4 n0_ = piece(ns.off, 0), n1_ = piece(ns.off, 1), n2_ = piece(ns.off, 2), n3_ = piece(ns.off, 3);
+                PathStep ns = s_path[0];  // offsets within the staged planes
+                float4 n0_ = piece((int)ns.off, 0), n1_ = piece((int)ns.off, 1), n2_ = piece((int)ns.off, 2), n3_ = piece((int)ns.off, 3);
 #pragma unroll 4
                 for (int q = 0; q < 32; ++q) {
                     const PathStep s = ns;
                     const float S[8] = {n0_.x, n0_.y, n0_.z, n0_.w, n1_.x, n1_.y, n1_.z, n1_.w};
                     const float chi[8] = {n2_.x, n2_.y, n2_.z, n2_.w, n3_.x, n3_.y, n3_.z, n3_.w};
                     ns = s_path[q + 1];
-                    n0_ = piece(ns.off, 0);
-                    n1_ = piece(ns.off, 1);
-                    n2_ = piece(ns.off, 2);
-                    n3_ = piece(ns.off, 3);
+                    n0_ = piece((int)ns.off, 0);
+                    n1_ = piece((int)ns.off, 1);
+                    n2_ = piece((int)ns.off, 2);
+                    n3_ = piece((int)ns.off, 3);
                     segments<8>(S, chi, s.nl2, I, T);
                     if constexpr (EXT) {
                         if (c0 + q == 0) {

@@ -41,3 +41,18 @@ def test_probe_list():
     one, _ = solve(16, 16, planes, [[0.0, 1.0]], probes[:1])
     J, _ = solve(16, 16, planes, [[0.0, 1.0]], probes)
     assert J.min().item() == one.item() == J.max().item() > 0.0
+
+
+def test_rays_across_more_than_2_31_cells():
+    """A ray whose records lie more than 2^31 cells behind its probe's, straight and aslant."""
+    n = 65536
+    planes = torch.zeros((1, n, n, 2), device="cuda")
+    planes[0, 40000, :, 0], planes[0, 40000, :, 1] = 3.0, 10.0
+    planes[0, n - 1, :, 0], planes[0, n - 1, :, 1] = 1e4, 1.0
+    d = [[0.0, 1.0], [0.6, 0.8]]
+    J, I = solve(n, n, planes.view(1, n * n, 2), d, torch.tensor([5], dtype=torch.int32, device="cuda"))
+    for k, (_, dz) in enumerate(d):
+        t1, t2 = 10.0 / dz, 1.0 / dz
+        want = 3.0 * (1.0 - np.exp(-t1)) + np.exp(-t1) * 1e4 * (1.0 - np.exp(-t2))
+        # relative errors: 4e-6 per update, and float32 path lengths and 2^x in the exponents
+        assert abs(I[0, k, 0].item() - want) < 2e-5 * want
