@@ -7,7 +7,8 @@
 // is a prefix of it that ends on the ray's own exit plane.  A warp (32 probes,
 // one wavelength batch, one direction at a time) builds that list 32 crossings
 // at a time, one per lane, in shared memory; its lanes then only load a record
-// at a common offset from their own cell and integrate it.
+// at a common offset from their own cell and integrate it (with eight wavelengths per
+// batch only in k_solve_dense_tile: dense_ray).
 //
 // Plane crossings are evaluated from exact half-integer plane offsets,
 //   t = offset * fl(1/d)  (+ a low-order part, see AxisParam),
@@ -130,13 +131,21 @@ struct PathBuilder {
     }
 };
 
-// One direction's ray of every lane of a warp (cell (i, j), record rec0): I and T
-// over the list's prefix up to the lane's exit plane.  Every lane of the warp
-// calls it; `live` is false for lanes without a probe.
+// One direction's ray of every lane of a warp (cell (i, j), record rec0): I and T up to
+// the lane's exit plane.  Every lane of the warp calls it; `live` is false for lanes
+// without a probe.
+// W = 8: every lane walks its own ray, the record requested before the plane arithmetic
+// that hides its latency.  Other W: over a prefix of the warp's list of crossings, where
+// the plane arithmetic, several times the update of one or two wavelengths, is shared.
+// With eight the list only adds its read to every step's chain; 256 x 264, 6 directions,
+// split: 417 us on the list, 309 walking; 200 x 208, 96 wavelengths, 24 directions, a
+// probe list: 6.26 and 5.65 ms.
 // EXT: the probe's own-cell emission (the first segment of every ray) is left
 // out, so I and J hold the radiation arriving from beyond the cell, attenuated
 // by it -- the part of J that MALI's effective mean intensity needs without
 // subtracting the own-cell term from J (Section 4.1's preconditioning)
+// The counting variant walks every cell: its count is the full-resolution segment
+// count that throughput figures are normalised by.
 template <int W, bool COUNT, bool EXT>
 __device__ __forceinline__ void dense_ray(const DenseParams& P, PathStep* path, int lane, int i, int j,
                                           const float* __restrict__ rec0, float dx, float dz, float stop, bool live,
@@ -149,57 +158,88 @@ __device__ __forceinline__ void dense_ray(const DenseParams& P, PathStep* path, 
     const float t2 = fminf(Ex * B.ax.ih, Ez * B.az.ih);
 #pragma unroll
     for (int w = 0; w < W; ++w) { I[w] = 0.0f; T[w] = 1.0f; }
-    constexpr int GROUP = W == 1 ? 8 : (W == 2 ? 4 : (W == 4 ? 2 : 1));
-    float th_end = 0.0f;  // the last crossing of the chunk before
-    [[maybe_unused]] float th_count = 0.0f;
-    // a ray crosses at most nx + nz planes
-    for (int c0 = 0; c0 < P.nx + P.nz; c0 += 32) {
-        int m;
-        const PathStep mine = B.next(c0, lane, m);
-        __syncwarp();  // every lane is done with the previous crossings
-        path[lane] = mine;
-        __syncwarp();
-        if (live) {
-            // a few records at a time, loaded before the first of them is used: a step's
-            // latency, not its arithmetic, sets the time of small grids.  A segment beyond
-            // the ray's exit (the crossing before it is at or past t2) reads nothing.
-            float th_before = c0 == 0 ? 0.0f : th_end;
-            for (int q0 = 0; q0 < 32 && live; q0 += GROUP) {
-                PathStep s[GROUP];
-                Record<W> r[GROUP];
+    if constexpr (W == 8) {
+        if (!live) return;
+        const char* rp = reinterpret_cast<const char*>(rec0);
+        float Px = B.px(0), Pz = B.pz(0), th_prev = 0.0f, tl_prev = 0.0f;
+        // a ray crosses at most nx + nz planes
+        for (int it = 0; it < P.nx + P.nz; ++it) {
+            const Record<W> r = RecFmt<W, kStoreF32>::load(reinterpret_cast<const float*>(rp));
+            const float tnx = Px * B.ax.ih, tnz = Pz * B.az.ih;
+            const bool on_x = tnx <= tnz;
+            const float th = on_x ? tnx : tnz;
+            const float tl = plane_lo(on_x ? Px : Pz, on_x ? B.ax : B.az, th);
+            const float len = fmaxf((th - th_prev) + (tl - tl_prev), 0.0f);  // as PathBuilder::next
+            segments<W>(r.S, r.chi, len * kNegLog2e, I, T);
+            if constexpr (EXT) {
+                if (it == 0) {
 #pragma unroll
-                for (int g = 0; g < GROUP; ++g) {
-                    s[g] = path[q0 + g];
-                    if (g == 0 || th_before < t2)
-                        r[g] = RecFmt<W, kStoreF32>::load(
-                            reinterpret_cast<const float*>(reinterpret_cast<const char*>(rec0) + s[g].off));
-                    th_before = s[g].th;
+                    for (int w = 0; w < W; ++w) I[w] = 0.0f;
                 }
+            }
+            if (COUNT) nseg += th > th_prev;
+            if (th >= t2 || (!COUNT && (it & 7) == 7 && ray_done<W>(I, T, stop))) break;
+            th_prev = th;
+            tl_prev = tl;
+            if (on_x) {
+                Px += B.sx;
+                rp += B.stepx;
+            } else {
+                Pz += B.sz;
+                rp += B.stepz;
+            }
+        }
+    } else {
+        constexpr int GROUP = W == 1 ? 8 : (W == 2 ? 4 : 2);
+        float th_end = 0.0f;  // the last crossing of the chunk before
+        [[maybe_unused]] float th_count = 0.0f;
+        // a ray crosses at most nx + nz planes
+        for (int c0 = 0; c0 < P.nx + P.nz; c0 += 32) {
+            int m;
+            const PathStep mine = B.next(c0, lane, m);
+            __syncwarp();  // every lane is done with the previous crossings
+            path[lane] = mine;
+            __syncwarp();
+            if (live) {
+                // a few records at a time, loaded before the first of them is used: a step's
+                // latency, not its arithmetic, sets the time of small grids.  A segment beyond
+                // the ray's exit (the crossing before it is at or past t2) reads nothing.
+                float th_before = c0 == 0 ? 0.0f : th_end;
+                for (int q0 = 0; q0 < 32 && live; q0 += GROUP) {
+                    PathStep s[GROUP];
+                    Record<W> r[GROUP];
 #pragma unroll
-                for (int g = 0; g < GROUP; ++g) {
-                    segments<W>(r[g].S, r[g].chi, s[g].nl2, I, T);
-                    if constexpr (EXT) {
-                        if (c0 + q0 + g == 0) {
+                    for (int g = 0; g < GROUP; ++g) {
+                        s[g] = path[q0 + g];
+                        if (g == 0 || th_before < t2)
+                            r[g] = RecFmt<W, kStoreF32>::load(
+                                reinterpret_cast<const float*>(reinterpret_cast<const char*>(rec0) + s[g].off));
+                        th_before = s[g].th;
+                    }
 #pragma unroll
-                            for (int w = 0; w < W; ++w) I[w] = 0.0f;
+                    for (int g = 0; g < GROUP; ++g) {
+                        segments<W>(r[g].S, r[g].chi, s[g].nl2, I, T);
+                        if constexpr (EXT) {
+                            if (c0 + q0 + g == 0) {
+#pragma unroll
+                                for (int w = 0; w < W; ++w) I[w] = 0.0f;
+                            }
+                        }
+                        if (COUNT) {
+                            nseg += s[g].th > th_count;  // segments whose end is beyond their start
+                            th_count = s[g].th;
+                        }
+                        if (s[g].th >= t2) {
+                            live = false;
+                            break;
                         }
                     }
-                    if (COUNT) {
-                        nseg += s[g].th > th_count;  // segments whose end is beyond their start
-                        th_count = s[g].th;
-                    }
-                    if (s[g].th >= t2) {
-                        live = false;
-                        break;
-                    }
+                    if (!COUNT && live && ((q0 + GROUP) & 7) == 0 && ray_done<W>(I, T, stop)) live = false;
                 }
-                // the counting variant walks every cell: its count is the full-resolution
-                // segment count that throughput figures are normalised by
-                if (!COUNT && live && ((q0 + GROUP) & 7) == 0 && ray_done<W>(I, T, stop)) live = false;
+                th_end = th_before;
             }
-            th_end = th_before;
+            if (!__any_sync(0xffffffffu, live)) break;
         }
-        if (!__any_sync(0xffffffffu, live)) break;
     }
 }
 
@@ -389,22 +429,23 @@ __global__ void __launch_bounds__(256, 4) k_solve_dense(const DenseParams P)
     if (COUNT && P.seg_count != nullptr) atomicAdd(P.seg_count, (unsigned long long)nseg);
 }
 
-// Eight directions at a time of 32 probes, one per warp; warp w then adds the
-// eight intensities of wavelength w to J in the order of the directions.
+// Several directions at a time of 32 probes, one per warp; the CTA then adds their
+// intensities to J in the order of the directions, thread (warp, lane) the wavelengths
+// warp, warp + warps, ... of its probe.
 template <int W, bool COUNT, bool EXT = false>
 __global__ void __launch_bounds__(256, 4) k_solve_dense_split(const DenseParams P)
 {
     __shared__ PathStep s_path[8][32];
     __shared__ float s_I[8][W][32];
-    const int b = blockIdx.y, warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    __shared__ float s_J[W][32];
+    const int b = blockIdx.y, warp = threadIdx.x >> 5, lane = threadIdx.x & 31, n_warp = blockDim.x >> 5;
     int i, j, p;
     const bool live = dense_probe(P, 1, 0, lane, i, j, p);
     const float* rec0 = P.planes + ((size_t)b * P.n_cells + (size_t)j * P.nx + i) * (2 * W);
     const float stop = !COUNT && P.scanned && live ? stop_factor(P.J[(size_t)(b * W) * P.n_probe + p], P.i_bc) : -1.0f;
-    const int lw = b * W + warp;  // the wavelength whose J this warp sums
-    float Jw = 0.0f;
+    for (int w = warp; w < W; w += n_warp) s_J[w][lane] = 0.0f;
     unsigned int nseg = 0;
-    for (int k0 = 0; k0 < P.quad.n_dir; k0 += 8) {
+    for (int k0 = 0; k0 < P.quad.n_dir; k0 += n_warp) {
         if (k0 + warp < P.quad.n_dir) {
             float I[W], T[W];
             dense_ray<W, COUNT, EXT>(P, s_path[warp], lane, i, j, rec0, P.quad.dx[k0 + warp], P.quad.dz[k0 + warp],
@@ -413,19 +454,20 @@ __global__ void __launch_bounds__(256, 4) k_solve_dense_split(const DenseParams 
             for (int w = 0; w < W; ++w) s_I[warp][w][lane] = fmaf(T[w], P.i_bc, I[w]);
         }
         __syncthreads();
-        if (warp < W) {
-#pragma unroll
-            for (int g = 0; g < 8; ++g) {
-                if (k0 + g >= P.quad.n_dir) break;
-                const float Iw = s_I[g][warp][lane];
+        for (int w = warp; w < W; w += n_warp) {
+            const int l = b * W + w;
+            float Jw = s_J[w][lane];
+            for (int g = 0; g < n_warp && k0 + g < P.quad.n_dir; ++g) {
+                const float Iw = s_I[g][w][lane];
                 Jw = fmaf(P.quad.w[k0 + g], Iw, Jw);
-                if (P.I != nullptr && live && lw < P.n_lambda)
-                    P.I[((size_t)lw * P.quad.n_dir + k0 + g) * P.n_probe + p] = Iw;
+                if (P.I != nullptr && live && l < P.n_lambda) P.I[((size_t)l * P.quad.n_dir + k0 + g) * P.n_probe + p] = Iw;
             }
+            s_J[w][lane] = Jw;
         }
         __syncthreads();
     }
-    if (warp < W && live && lw < P.n_lambda) P.J[(size_t)lw * P.n_probe + p] = Jw;
+    for (int w = warp; w < W; w += n_warp)
+        if (live && b * W + w < P.n_lambda) P.J[(size_t)(b * W + w) * P.n_probe + p] = s_J[w][lane];
     if (COUNT && P.seg_count != nullptr) atomicAdd(P.seg_count, (unsigned long long)nseg);
 }
 
@@ -438,10 +480,17 @@ constexpr int kScanCtas = 304;
 
 // Grids of fewer warps (32 probes x batch) than two full loads of the chip's 152 x
 // 32 resident ones split the directions.  128 x 128, one wavelength, 16 directions:
-// 512 warps took 231 us one after the other, split 61 us (41 with a few records in
+// 512 warps took 231 us one after the other, split 61 us (39 with a few records in
 // flight per ray).
 constexpr long long kSplitWarps = 2 * 152 * 32;
 
+// Fewer than eight directions of a whole grid, W = 8: a split CTA is small and its rays
+// part at once, so k_solve_dense_tile takes over as soon as its CTAs fill the chip (two
+// per SM).  4 directions, split -> tile: 350 x 358, 16 wavelengths (360 CTAs) 1.36 ->
+// 1.19 ms; 200 x 208, 24 (378) 472 -> 468 us; 8 (126) 184, tile 218; 6 directions,
+// 256 x 264, 8 (176) 309, tile 421.  With more directions splitting stays ahead: 300 x
+// 308, 9, 24 directions 3.41, tile 3.85 ms; 250 x 258, 24, 10 directions 1.37, 1.50.
+constexpr long long kTileCtas = 2 * 152;
 
 template <int W>
 __global__ void __launch_bounds__(256) k_dense_scan(const DenseParams P)
@@ -472,9 +521,15 @@ __global__ void __launch_bounds__(256) k_dense_spread(const DenseParams P, int n
         J[p] = m;
 }
 
+// CTAs of k_solve_dense_tile
+long long tile_grid(const DenseParams& P)
+{
+    return (P.nx + 31LL) / 32 * ((P.nz + kTileRows - 1) / kTileRows) * P.n_batch;
+}
+
 cudaError_t launch_dense_tile(cudaStream_t s, const DenseParams& P)
 {
-    const dim3 grid((unsigned)(((P.nx + 31) / 32) * ((P.nz + kTileRows - 1) / kTileRows)), (unsigned)P.n_batch);
+    const dim3 grid((unsigned)(tile_grid(P) / P.n_batch), (unsigned)P.n_batch);
     auto kernel = P.exclude_own ? k_solve_dense_tile<true> : k_solve_dense_tile<false>;
     const size_t smem = 4 * kTilePlane + 33 * sizeof(PathStep);
     cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
@@ -498,13 +553,18 @@ void launch_dense_w(bool split, dim3 grid, cudaStream_t s, const DenseParams& P)
     if (P.scanned) launch_dense_scan<W>(s, P);
 #define DEX_LAUNCH_DENSE(K)                                               \
     if (P.exclude_own) {                                                  \
-        if (P.seg_count) K<W, true, true><<<grid, 256, 0, s>>>(P);        \
-        else K<W, false, true><<<grid, 256, 0, s>>>(P);                   \
+        if (P.seg_count) K<W, true, true><<<grid, threads, 0, s>>>(P);    \
+        else K<W, false, true><<<grid, threads, 0, s>>>(P);               \
     } else if (P.seg_count) {                                             \
-        K<W, true><<<grid, 256, 0, s>>>(P);                               \
+        K<W, true><<<grid, threads, 0, s>>>(P);                           \
     } else {                                                              \
-        K<W, false><<<grid, 256, 0, s>>>(P);                              \
+        K<W, false><<<grid, threads, 0, s>>>(P);                          \
     }
+    // split: as many warps as share the directions evenly over rounds of at most eight
+    // (idle ones would hold their registers: 350 x 358, 16 wavelengths, 4 directions on
+    // eight warps 3.10 ms, on four 1.77)
+    const int rounds = (P.quad.n_dir + 7) / 8;
+    const int threads = split ? 32 * ((P.quad.n_dir + rounds - 1) / rounds) : 256;
     if (split) {
         DEX_LAUNCH_DENSE(k_solve_dense_split)
     } else {
@@ -539,8 +599,9 @@ cudaError_t launch_solve_dense(cudaStream_t s, const DenseParams& P0)
     // one warp per 32 probes, or eight (one per direction) where those would not
     // fill the chip
     const long long warps = (P.n_probe + 31LL) / 32 * P.n_batch;
-    const bool split = warps < kSplitWarps;
-    if (!split && P.W == 8 && P.probes == nullptr && !P.seg_count) {
+    const bool tile = P.W == 8 && P.probes == nullptr && !P.seg_count;
+    const bool split = warps < kSplitWarps && !(tile && P.quad.n_dir < 8 && tile_grid(P) >= kTileCtas);
+    if (!split && tile) {
         if (P.scanned) launch_dense_scan<8>(s, P);
         return launch_dense_tile(s, P);
     }
