@@ -579,7 +579,7 @@ typedef struct {
 /*
  * Solve n_atm (<= DEX_MAX_BATCH_ATM) atmospheres in one persistent launch.
  *   atms     host [n_atm] descriptors (device pointers inside)
- *   ctas     persistent grid size (0: 3 per SM)
+ *   ctas     persistent grid size (0: 3 per SM; 6 of half the size for small batches)
  *   queue    device scratch: one unsigned int, the work counter (reset by the call)
  *   done_ns  device [n_atm] or NULL: completion time of each atmosphere's last item
  *            (GPU global timer, ns), start_ns device [1] or NULL: the earliest CTA start
@@ -604,7 +604,8 @@ int dex_batch_solve(dex_ctx* ctx, int n_atm, const dex_batch_item* atms, int W, 
  * Every probe accumulates J over the directions in one thread in the order of
  * dex_formal_solve_hdda, so J is bit-identical for every configuration.
  * dex_batch_solve is dex_batch_solve_config with {ctas, 256, 1, s, 0}, s = 1 where
- * every grid has at most 8192 blocks.  Invalid values -> DEX_ERR_ARG.
+ * every grid has at most 8192 blocks; with ctas = 0 and fewer than 6 packets of 256 per
+ * SM it is {6 per SM, 128, 1, s, 0}.  Invalid values -> DEX_ERR_ARG.
  * With the context's traversal set to DEX_TRAVERSAL_PAIRED (W = 8; every grid
  * of at most 8192 blocks, else DEX_ERR_UNSUPPORTED) the work units are each
  * atmosphere's pairs of batches (dex_ctx_set_pair_group) and lone batches, and

@@ -1013,6 +1013,13 @@ static int fill_batch(dex_ctx* ctx, int n_atm, const dex_batch_item* atms, int W
     return DEX_OK;
 }
 
+static int sm_count(dex_ctx* ctx)
+{
+    int sms = 0;
+    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, ctx->device);
+    return sms > 0 ? sms : 152;
+}
+
 // Zero every J, then launch the persistent solve with the given work counter.
 static int batch_launch(dex_ctx* ctx, dex::BatchParams& P, const dex_batch_item* atms, int W, int ctas,
                         size_t max_words, unsigned int* queue, unsigned long long* done_ns,
@@ -1024,11 +1031,7 @@ static int batch_launch(dex_ctx* ctx, dex::BatchParams& P, const dex_batch_item*
     P.done_ns = done_ns;
     P.start_ns = start_ns;
     P.status = ctx->status;
-    if (ctas <= 0) {
-        int sms = 0;
-        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, ctx->device);
-        ctas = 3 * (sms > 0 ? sms : 152);
-    }
+    if (ctas <= 0) ctas = 3 * sm_count(ctx);
     cudaError_t e = cudaSuccess;
     for (int a = 0; a < P.n_atm && e == cudaSuccess; ++a)
         e = cudaMemsetAsync(atms[a].J, 0, sizeof(float) * (size_t)atms[a].n_lambda * atms[a].nx * atms[a].nz,
@@ -1045,6 +1048,25 @@ static int batch_launch(dex_ctx* ctx, dex::BatchParams& P, const dex_batch_item*
 // (eight atmospheres of up to 512^2: 39.4 ms against 40.9 with the packed states).
 static bool stage_info(size_t max_blocks) { return max_blocks <= (size_t)dex::kInfoMaxBlocks; }
 
+// Fill the launch parameters for the default configuration: packets of 256 probes, or of
+// 128 with twice the CTAs where the grid is left to the library (ctas <= 0) and its 3
+// CTAs per SM would get fewer than two packets each.  The last packets then set the time,
+// and the warps of a large one wait for its slowest ray.  Static lines of 128 to 192 cells
+// a side, 32 wavelengths, 256 -> 128 probes: three atmospheres 3.53 -> 3.21 ms paired
+// (448 packets), 3.28 -> 2.91 one walk per batch (800); four, paired (704) 3.45 -> 3.13;
+// but three of up to 384 (1376) 4.35 -> 4.52.
+static int fill_default(dex_ctx* ctx, int n_atm, const dex_batch_item* atms, int W, dex::BatchParams& P,
+                        size_t& max_words, size_t& max_blocks, int& ctas, int& packet)
+{
+    packet = 256;
+    if (int r = fill_batch(ctx, n_atm, atms, W, P, max_words, 1, &max_blocks)) return r;
+    const long long resident = 3LL * sm_count(ctx);
+    if (ctas > 0 || P.n_items >= 2 * resident) return DEX_OK;
+    packet = 128;
+    ctas = (int)(2 * resident);
+    return fill_batch(ctx, n_atm, atms, W, P, max_words, 2, &max_blocks);
+}
+
 int dex_batch_solve(dex_ctx* ctx, int n_atm, const dex_batch_item* atms, int W, int ctas, unsigned int* queue,
                     unsigned long long* done_ns, unsigned long long* start_ns)
 {
@@ -1053,9 +1075,12 @@ int dex_batch_solve(dex_ctx* ctx, int n_atm, const dex_batch_item* atms, int W, 
     dex::BatchParams* P = new (std::nothrow) dex::BatchParams();
     if (!P) return fail(ctx, DEX_ERR_ARG, "host allocation failed");
     size_t max_words = 0, max_blocks = 0;
-    int r = fill_batch(ctx, n_atm, atms, W, *P, max_words, 1, &max_blocks);
+    int packet = 256;
+    int r = fill_default(ctx, n_atm, atms, W, *P, max_words, max_blocks, ctas, packet);
     if (!r) r = bind(ctx);
-    if (!r) r = batch_launch(ctx, *P, atms, W, ctas, max_words, queue, done_ns, start_ns, 256, stage_info(max_blocks), max_blocks);
+    if (!r)
+        r = batch_launch(ctx, *P, atms, W, ctas, max_words, queue, done_ns, start_ns, packet, stage_info(max_blocks),
+                         max_blocks);
     delete P;
     return r;
 }
@@ -1096,12 +1121,14 @@ int dex_batch_solve_noalloc(dex_ctx* ctx, int n_atm, const dex_batch_item* atms,
     if (!ctx) return DEX_ERR_ARG;
     dex::BatchParams P{};  // on the stack: this call makes no allocation at all
     size_t max_words = 0, max_blocks = 0;
-    if (int r = fill_batch(ctx, n_atm, atms, W, P, max_words, 1, &max_blocks)) return r;
+    int packet = 256;
+    if (int r = fill_default(ctx, n_atm, atms, W, P, max_words, max_blocks, ctas, packet)) return r;
     if (int r = bind(ctx)) return r;
     unsigned int* scratch = nullptr;
     cudaError_t e = dex::noalloc_scratch(&scratch);
     if (e != cudaSuccess) return cuda_fail(ctx, e, "static scratch address");
-    return batch_launch(ctx, P, atms, W, ctas, max_words, scratch, done_ns, start_ns, 256, stage_info(max_blocks), max_blocks);
+    return batch_launch(ctx, P, atms, W, ctas, max_words, scratch, done_ns, start_ns, packet, stage_info(max_blocks),
+                        max_blocks);
 }
 
 }  // extern "C"
