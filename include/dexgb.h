@@ -313,9 +313,10 @@ int dex_mips_build(dex_ctx* ctx, int nx, int nz, int n_lambda, int W, const floa
  *   J   device [n_lambda][nz][nx] output; zeroed by the call, written at probe cells
  *   I   device [n_lambda][n_dir][nz][nx] output or NULL (zeroed by the call)
  *   seg_count  device uint64 accumulator or NULL: adds the voxel segments integrated.
- *       A counting call follows every ray until its transmissions are exactly zero;
- *       without a count rays end as soon as the rest cannot change a bit of I (J and I
- *       are the same), so a timed call integrates fewer segments than are counted
+ *       A counting call follows every ray to the block crossing at which its transmissions
+ *       have all become exactly zero; without a count rays end as soon as the rest cannot
+ *       change a bit of I (J and I are the same), so a timed call integrates fewer segments
+ *       than are counted
  * With one walk per batch (the default) and W = 8, two mirrored batches whose blocks all
  * have the same levels share a walk; J and I are the same bit for bit.
  */

@@ -147,10 +147,12 @@ __device__ __forceinline__ void trace_ray3(const Hdda3Params& P, const float* __
         if (COUNT) nseg += (cur_mip >= 0) & (th > th_prev);
         // early termination, tested every fourth step by all lanes together: the rest of
         // the ray changes no bit of I
-        if (last || ((it & 3) == 3 && ray_done<NB * W>(I, T, stop))) break;
+        if (last || (!COUNT && (it & 3) == 3 && ray_done<NB * W>(I, T, stop))) break;
         th_prev = th;
         tl_prev = tl;
         if (cross) {  // entered another block
+            // counted segments run to the block in which every transmission has become zero
+            if (COUNT && all_opaque<NB * W>(T)) break;
             const int bxn = bxc + (axis == 0 ? sx : 0), byn = byc + (axis == 1 ? sy : 0),
                       bzn = bzc + (axis == 2 ? sz : 0);
             if ((unsigned)bxn >= (unsigned)P.nbx || (unsigned)byn >= (unsigned)P.nby ||

@@ -116,6 +116,8 @@ __device__ __forceinline__ bool rc_interval(const RcParams& P, const float* __re
                 rp += negz ? -side * REC : side * REC;
                 cross = (unsigned)lz >= (unsigned)side;
             }
+            // counted segments run to the block in which every transmission has become zero
+            if (COUNT && cross && all_opaque<NB * W>(T)) break;
             if (cross) {
                 const int bxn = bxc + (on_x ? sx : 0), bzn = bzc + (on_x ? 0 : sz);
                 if ((unsigned)bxn >= (unsigned)P.nbx || (unsigned)bzn >= (unsigned)P.nbz) {
@@ -164,7 +166,7 @@ __device__ __forceinline__ bool rc_interval(const RcParams& P, const float* __re
             if (COUNT) nseg += NB * (th > th_prev);
         }
         // the rest changes no bit of the radiance
-        if (last || ((it & 3) == 3 && ray_done<NB * W>(I, T, stop))) break;
+        if (last || (!COUNT && (it & 3) == 3 && ray_done<NB * W>(I, T, stop))) break;
         th_prev = th;
         tl_prev = tl;
     }
