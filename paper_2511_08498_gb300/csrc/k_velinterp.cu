@@ -89,8 +89,11 @@ struct VelModel {
 
 // CTA (a, b): the early termination's bound of active block a and batch b, to the
 // block's first cell.  Interpolated source functions lie between those of the two
-// samples; rounding can exceed them only where neighbouring opacities differ by
-// more than 2^20, which counts as no bound.
+// samples but for rounding: at the clamped speed the weight can come out as 1 + 2^-19
+// (two units of the quotient's rounding, times 7, less 6), which takes 2^-19 of the other
+// sample's opacity and emission off.  Where neighbouring opacities differ by at most 2^15
+// that is a sixteenth of this sample's opacity and of the bound's emission, well within
+// the factor of 16 below; a larger ratio counts as no bound.
 template <int W>
 __global__ void __launch_bounds__(128) k_scan_vel(const HddaParams P)
 {
@@ -105,7 +108,7 @@ __global__ void __launch_bounds__(128) k_scan_vel(const HddaParams P)
         float prev = p[W];
         for (int s = 0; s < kNV; ++s) {
             const float e = p[s * 2 * W], c = p[s * 2 * W + W];
-            const bool steep = fminf(c, prev) * 1048576.0f < fmaxf(c, prev);
+            const bool steep = fminf(c, prev) * 32768.0f < fmaxf(c, prev);  // 2^15
             const float v = c > 0.0f ? __fdividef(e, c) : 0.0f;
             m = join_bounds(m, steep ? -1.0f : bound_of(v, c));
             prev = c;
