@@ -192,7 +192,9 @@ size_t dex_planes_floats(int n_cells, int n_lambda, int W);
  *              1 <= n_dir <= DEX_MAX_DIRS
  *   n_probe    number of probes; n_probe < 0 means every cell (probes must be
  *              NULL, probe p = cell p); n_probe == 0 is a no-op
- *   probes     device [n_probe] cell indices (ignored when n_probe <= 0)
+ *   probes     device [n_probe] cell indices (ignored when n_probe <= 0); one outside the
+ *              grid sets DEX_ERR_TRAVERSAL_CAP in the device status word, and its J is not
+ *              a result
  *   J          device [n_lambda][n_probe] float32 output (overwritten)
  *   I          device [n_lambda][n_dir][n_probe] float32 output, or NULL
  *   seg_count  device uint64 accumulator, or NULL: adds the number of

@@ -490,6 +490,7 @@ __global__ void __launch_bounds__(256, Model::kMinBlocks) k_solve_hdda_t(const H
     const int state0 = (kInfo ? (s_info[blk0] & 7) : block_state(s_dyn, blk0)) - 1;
     if (state0 < 0) {  // state words do not describe this active block
         raise_status(P.status, DEX_ERR_TRAVERSAL_CAP);
+        if (P.scanned) P.J[(size_t)(b * W) * P.n_cells + (size_t)j * P.nx + i] = 0.0f;  // it held the bound
         return;
     }
     Geo G;

@@ -152,8 +152,12 @@ __global__ void __launch_bounds__(NT, kMinCtas) k_batch_solve(const BatchParams 
             const int i = bx0 * DEX_BLOCK + (wrp & 1) * 8 + (tid & 7);
             const int j = bz0 * DEX_BLOCK + part * (DEX_BLOCK / kParts) + (wrp >> 1) * 4 + ((tid & 31) >> 3);
             const int state0 = (kInfo || kPair ? (s_info[blk0] & 7) : block_state(s_dyn, blk0)) - 1;
+            const size_t cell = (size_t)j * A.nx + i;
+            const size_t plane = (size_t)W * A.nx * A.nz;
             if (state0 < 0) {
                 capped = true;
+                A.J[b1 * plane + cell] = 0.0f;  // it held the bound
+                if (kPair && b2 >= 0) A.J[b2 * plane + cell] = 0.0f;
                 continue;
             }
             Geo G;
@@ -169,8 +173,6 @@ __global__ void __launch_bounds__(NT, kMinCtas) k_batch_solve(const BatchParams 
 #pragma unroll
             for (int q = 0; q < 4; ++q) G.band[q] = A.band[q];
             // the batch's bound (k_scan_batch) waits where this thread's first J will go
-            const size_t cell = (size_t)j * A.nx + i;
-            const size_t plane = (size_t)W * A.nx * A.nz;
             float bound = A.J[b1 * plane + cell];
             [[maybe_unused]] float bound2 = 0.0f;
             [[maybe_unused]] int second = -1;  // kTwin: a batch to be walked by itself after b1

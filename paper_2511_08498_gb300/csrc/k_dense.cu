@@ -389,6 +389,7 @@ __device__ __forceinline__ bool dense_probe(const DenseParams& P, int tile_rows,
     const int c = P.probes[p];
     if (c < 0 || (long long)c >= P.n_cells) {
         raise_status(P.status, DEX_ERR_TRAVERSAL_CAP);
+        if (P.scanned) P.J[(size_t)(blockIdx.y * P.W) * P.n_probe + p] = 0.0f;  // it held the bound
         return false;
     }
     i = c % P.nx;

@@ -264,6 +264,11 @@ __global__ void __launch_bounds__(kThreads3, NB == 1 ? kMinBlocks3 : 2) k_solve_
     const int state0 = (INFO ? s_info[blk0] & 7 : block_state3(words, blk0)) - 1;
     if (state0 < 0) {  // state words do not describe this active block
         raise_status(P.status, DEX_ERR_TRAVERSAL_CAP);
+        if (P.scanned) {  // the probe's J held the bounds
+            const int pc = part * kThreads3 + tid;
+            float* J = P.J + ((size_t)(bz0 * B3 + (pc >> 6)) * P.ny + by0 * B3 + ((pc >> 3) & 7)) * P.nx + bx0 * B3 + (pc & 7);
+            J[(size_t)(b * W) * P.n_cells] = J[(size_t)(b2 * W) * P.n_cells] = 0.0f;
+        }
         return;
     }
     constexpr int REC = RecFmt<W, ST>::kStride;

@@ -121,6 +121,7 @@ __global__ void __launch_bounds__(pair_threads<ST>(), pair_min_blocks<ST>()) k_s
     const int state0 = (s_info[blk0] & 7) - 1;
     if (state0 < 0) {  // state words do not describe this active block
         raise_status(P.status, DEX_ERR_TRAVERSAL_CAP);
+        if (P.scanned) P.J[(size_t)(b1 * 8) * P.n_cells + cell] = P.J[(size_t)(b2 * 8) * P.n_cells + cell] = 0.0f;  // the bounds
         return;
     }
     const size_t batch_floats = (size_t)P.cap_active * P.chain * Model::kStride;
