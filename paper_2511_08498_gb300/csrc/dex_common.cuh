@@ -129,7 +129,7 @@ __device__ __forceinline__ bool all_opaque(const float* T)
     return bits == 0u;
 }
 
-// Exact early termination.  With B >= |S| of every record of the batch and B >=
+// Exact early termination.  With B >= S >= 0 of every record of the batch and B >=
 // |i_bc|, whatever a ray still adds to a wavelength is at most T B (1 + 2^-21) per
 // segment.  Where T B 2^26 <= I that is below a quarter of the spacing of floats
 // at I, so every later update, and the boundary term, rounds back to I: the rest
@@ -145,11 +145,12 @@ __device__ __forceinline__ float stop_factor(float bound, float i_bc)
 // The larger of two bounds, or -1 (none known) if either is.
 __device__ __forceinline__ float join_bounds(float a, float b) { return fminf(a, b) < 0.0f ? -1.0f : fmaxf(a, b); }
 
-// Bound of one wavelength's record, or -1 unless S is finite and chi finite and not negative.
+// Bound of one wavelength's record, or -1 unless S and chi are finite and not negative (a
+// negative I would never pass ray_done's test; such rays end where T is zero, as without a
+// bound).
 __device__ __forceinline__ float bound_of(float S, float chi)
 {
-    const float a = fabsf(S);
-    return a <= 3.402823466e38f && chi >= 0.0f && chi <= 3.402823466e38f ? a : -1.0f;
+    return S >= 0.0f && S <= 3.402823466e38f && chi >= 0.0f && chi <= 3.402823466e38f ? S : -1.0f;
 }
 
 template <int W>
