@@ -141,20 +141,29 @@ __device__ void stage_weights(SmemNet& net, unsigned char* W2, const float* __re
     if (t == 0) net.b3 = p[kB3];
 }
 
+// The larger of a and b, NaN if either is.
+__device__ __forceinline__ float max_nan(float a, float b)
+{
+    float m;
+    asm("max.NaN.f32 %0, %1, %2;" : "=f"(m) : "f"(a), "f"(b));
+    return m;
+}
+
 // GELU of two hidden units on the packed FP32 pipe.  The two logistic functions share
 // one reciprocal, 1/a = b / (a b): three special-function operations for two
-// activations instead of four, in kernels whose issue slots and FP32 pipe they share.  2^x is bounded at 2^60, below
-// which the product cannot overflow and above which the activation is 0 to 1e-17.
+// activations instead of four, in kernels whose issue slots and FP32 pipe they share.
+// Pre-activations count as at least -7.6, where 2^x is 2^62.7, so that the product of
+// two stays below 2^126 and its reciprocal is normal; there and below the activation
+// comes out as -1e-18 (its value is between that and 0).
 struct Gelu2 {
     float2 z, z2, s;
-    __device__ __forceinline__ explicit Gelu2(float2 zz) : z(zz)
+    __device__ __forceinline__ explicit Gelu2(float2 zz) : z(make_float2(max_nan(zz.x, -7.6f), max_nan(zz.y, -7.6f)))
     {
         // -2 log2(e) c (z + k z^3), c = sqrt(2 / pi), k = 0.044715
         constexpr float c1 = -2.3022081986f, c2 = -0.1029432397f;
         z2 = __fmul2_rn(z, z);
         const float2 a = __fmul2_rn(z, __ffma2_rn(make_float2(c2, c2), z2, make_float2(c1, c1)));
-        const float2 e = make_float2(mlp::mlp_ex2(fminf(a.x, 60.0f)), mlp::mlp_ex2(fminf(a.y, 60.0f)));
-        const float2 d = __fadd2_rn(make_float2(1.0f, 1.0f), e);
+        const float2 d = __fadd2_rn(make_float2(1.0f, 1.0f), make_float2(mlp::mlp_ex2(a.x), mlp::mlp_ex2(a.y)));
         const float r = mlp::mlp_rcp(d.x * d.y);
         s = __fmul2_rn(make_float2(r, r), make_float2(d.y, d.x));
     }
@@ -180,23 +189,6 @@ __device__ __forceinline__ float2 gelu2(float2 z)
     const float2 a = __fmul2_rn(u, make_float2(m2log2e, m2log2e));
     const float2 d = __fadd2_rn(make_float2(1.0f, 1.0f), make_float2(mlp::mlp_ex2(a.x), mlp::mlp_ex2(a.y)));
     return __fmul2_rn(z, make_float2(mlp::mlp_rcp(d.x), mlp::mlp_rcp(d.y)));
-}
-
-// GELU of four hidden units with one reciprocal: 1/(p q) gives q/(p q) and p/(p q) for
-// the two pairs' products, as in Gelu2.  2^x is bounded at 2^30 (the product below
-// 2^121): activations at z < -5.6 come out as z 2^-30, off by less than 6e-9.
-__device__ __forceinline__ void gelu4(float2 za, float2 zb, float2& ga, float2& gb)
-{
-    auto den = [](float2 z) {
-        constexpr float c1 = -2.3022081986f, c2 = -0.1029432397f;
-        const float2 a = __fmul2_rn(z, __ffma2_rn(make_float2(c2, c2), __fmul2_rn(z, z), make_float2(c1, c1)));
-        return __fadd2_rn(make_float2(1.0f, 1.0f),
-                          make_float2(mlp::mlp_ex2(fminf(a.x, 30.0f)), mlp::mlp_ex2(fminf(a.y, 30.0f))));
-    };
-    const float2 da = den(za), db = den(zb);
-    const float pa = da.x * da.y, pb = db.x * db.y, r = mlp::mlp_rcp(pa * pb), ra = r * pb, rb = r * pa;
-    ga = __fmul2_rn(za, __fmul2_rn(make_float2(ra, ra), make_float2(da.y, da.x)));
-    gb = __fmul2_rn(zb, __fmul2_rn(make_float2(rb, rb), make_float2(db.y, db.x)));
 }
 
 // z1 of units i .. i + 3
@@ -292,17 +284,16 @@ __global__ void __launch_bounds__(128, 8) k_mlp_forward(const MlpParams P)
         // output unit: two partial sums (even and odd hidden units) on the packed pipe
         float2 y2 = make_float2(sm.net.b3, 0.0f);
 #pragma unroll 1
-        for (int c = 0; c < kH; c += 16) {
+        for (int j = 0; j < kH; j += 16) {
             float z[16];
-            tmem_ld16(tmem_at(tm, warp * 32, kColD2 + c), z);
+            tmem_ld16(tmem_at(tm, warp * 32, kColD2 + j), z);
 #pragma unroll
             for (int q = 0; q < 16; q += 4) {
-                const float4 b = *reinterpret_cast<const float4*>(&sm.net.b2[c + q]);
-                const float4 w = *reinterpret_cast<const float4*>(&sm.net.w3[c + q]);
-                float2 ga, gb;
-                gelu4(__fadd2_rn(make_float2(z[q], z[q + 1]), make_float2(b.x, b.y)),
-                      __fadd2_rn(make_float2(z[q + 2], z[q + 3]), make_float2(b.z, b.w)), ga, gb);
-                y2 = __ffma2_rn(make_float2(w.z, w.w), gb, __ffma2_rn(make_float2(w.x, w.y), ga, y2));
+                const float4 b = *reinterpret_cast<const float4*>(&sm.net.b2[j + q]);
+                const float4 w = *reinterpret_cast<const float4*>(&sm.net.w3[j + q]);
+                const Gelu2 a(__fadd2_rn(make_float2(z[q], z[q + 1]), make_float2(b.x, b.y)));
+                const Gelu2 c(__fadd2_rn(make_float2(z[q + 2], z[q + 3]), make_float2(b.z, b.w)));
+                y2 = __ffma2_rn(make_float2(w.z, w.w), c.g(), __ffma2_rn(make_float2(w.x, w.y), a.g(), y2));
             }
         }
         const float y = y2.x + y2.y;
