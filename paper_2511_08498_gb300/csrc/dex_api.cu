@@ -146,7 +146,12 @@ int fill_atom(dex_ctx* ctx, const dex_atom* atom, int n_lambda, const double* la
     for (int k = 0; k < n_lambda; ++k) {
         P.off[k] = line_tag[k] >= 0 ? P.nu[k] - P.nu0[line_tag[k]] : 0.0;
         P.bx[k] = kH_ * P.nu[k] / kKB_;
-        P.by[k] = P.bx[k] * (256.0 / M_LN2);
+        // h nu / k * 256 / ln2 to twice the digits: every product and quotient with its remainder
+        constexpr double steps = 256.0 / M_LN2, steps_lo = 5.2109500776783445e-15;
+        const double p = kH_ * P.nu[k], p_lo = std::fma(kH_, P.nu[k], -p);
+        const double x_lo = (std::fma(-P.bx[k], kKB_, p) + p_lo) / kKB_;
+        P.by[k] = P.bx[k] * steps;
+        P.by_lo[k] = std::fma(P.bx[k], steps, -P.by[k]) + (x_lo * steps + P.bx[k] * steps_lo);
         P.bc[k] = 2.0 * kH_ * P.nu[k] * P.nu[k] * P.nu[k] / (kC_ * kC_);
     }
     for (int j = 0; j < 256; ++j) P.exp_table[j] = std::exp2(j / 256.0);

@@ -165,7 +165,8 @@ struct AtomParams {
     short first[DEX_MAX_LINES + 1];
     double off[DEX_MAX_ATOM_LAMBDA];   // nu - nu0 of the sample's line
     double bx[DEX_MAX_ATOM_LAMBDA];    // h nu / k (K)
-    double by[DEX_MAX_ATOM_LAMBDA];    // the same in units of ln2 / 256
+    double by[DEX_MAX_ATOM_LAMBDA];    // the same in units of ln2 / 256, and what its
+    double by_lo[DEX_MAX_ATOM_LAMBDA]; // rounding to double left off
     double bc[DEX_MAX_ATOM_LAMBDA];    // 2 h nu^3 / c^2
     double exp_table[256];             // 2^(j / 256)
     double nu0[DEX_MAX_LINES];
