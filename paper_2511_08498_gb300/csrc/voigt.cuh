@@ -24,10 +24,11 @@
 // of O(0.05) real parts in Weideman's form, and in float32 the complex sum loses
 // up to ~1e-3 of it.  In the three forms above nothing cancels: a float32 model of
 // them stays within 6e-7 relative of the Faddeeva function for a from 1e-4 to 0.25
-// and |x| + a < 15 (the Taylor series about the real axis built on Weideman's sum
-// that they replaced: 1.1e-5).  Cost: about 36 instructions in the core and 25 in
-// the wing against 165 and 60; the Core-and-Voigt solve, whose warps meet both,
-// ran at the rate it fetched them.
+// and |x| + a < 15, the kernel within 6.4e-7 (8.2e-7 down to a = 1e-6; the Taylor
+// series about the real axis built on Weideman's sum that they replaced: 9e-6 and, at
+// a = 1e-6, 6e-4).  Cost: about 36 instructions in the core and 25 in the wing against
+// 165 and 60; the Core-and-Voigt solve, whose warps meet both, ran at the rate it
+// fetched them.
 // The coefficients (a_n: Fourier coefficients of exp(-t^2)(L^2 + t^2), t = L
 // tan(theta/2); D's Taylor coefficients) are computed on the host and passed as a
 // kernel parameter; D's are read at a node per lane, so kernels copy them to
