@@ -114,7 +114,6 @@ int fill_atom(dex_ctx* ctx, const dex_atom* atom, int n_lambda, const double* la
         if (!(lambda_nm[k] > 0.0)) return fail(ctx, DEX_ERR_ARG, "wavelength %d must be > 0", k);
         if (line_tag[k] < -1 || line_tag[k] >= atom->n_line) return fail(ctx, DEX_ERR_ARG, "bad line tag %d", k);
         P.nu[k] = kC_ / (lambda_nm[k] * 1e-7);
-        P.tag[k] = (signed char)line_tag[k];
         P.wq[k] = 0.0;
     }
     for (int l = 0; l < atom->n_line; ++l) {

@@ -158,7 +158,6 @@ struct AtomParams {
     int n_lambda;
     double nu[DEX_MAX_ATOM_LAMBDA];    // sample frequencies (Hz)
     double wq[DEX_MAX_ATOM_LAMBDA];    // trapezoid weight in frequency within the sample's line
-    signed char tag[DEX_MAX_ATOM_LAMBDA];
     // samples grouped by line (line li: order[first[li]] .. order[first[li + 1] - 1]),
     // those without a line last, up to n_lambda
     short order[DEX_MAX_ATOM_LAMBDA];

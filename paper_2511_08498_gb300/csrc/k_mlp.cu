@@ -92,11 +92,6 @@ static_assert(sizeof(SmemTrain) <= kSmemTrain && 3 * kSmemTrain > 228 * 1024, "t
 
 __device__ __forceinline__ float bf16_round(float x) { return __bfloat162float(__float2bfloat16_rn(x)); }
 
-__device__ __forceinline__ void put_bf16(unsigned char* tile, int off, float v)
-{
-    *reinterpret_cast<__nv_bfloat16*>(tile + off) = __float2bfloat16_rn(v);
-}
-
 // A sample's inputs as stored.
 struct Sample {
     float x, a, u;
