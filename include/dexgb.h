@@ -602,8 +602,8 @@ int dex_batch_solve(dex_ctx* ctx, int n_atm, const dex_batch_item* atms, int W, 
  *            memory: 0 the packed 3-bit state words (plus the global offset
  *            table), 1 one word per block, offset * 8 + state (every grid of
  *            the batch at most 8192 blocks)
- *   occupancy  0: the compiler's register budget; 1 (W = 8 only): 64 registers
- *            a thread, so that 1024 threads a SM are resident (some spilling)
+ *   occupancy  0: at most 80 registers a thread, so that 768 threads a SM are resident;
+ *            1 (W = 8 only): 64 registers, 1024 threads (more spilling)
  * Every probe accumulates J over the directions in one thread in the order of
  * dex_formal_solve_hdda, so J is bit-identical for every configuration.
  * dex_batch_solve is dex_batch_solve_config with {ctas, 256, 1, s, 0}, s = 1 where

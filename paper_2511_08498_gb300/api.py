@@ -505,7 +505,7 @@ def mali_iteration(ctx: Context, atom: Atom, lam_nm, tag, T, ne, nh, nx: int, nz
 
 
 def voigt(ctx: Context, a: torch.Tensor, x: torch.Tensor, out=None):
-    """H(a, x) by HUM1WEI24 (``dex_voigt``); a, x float32 CUDA tensors of equal size."""
+    """The Voigt function H(a, x) (``dex_voigt``); a, x float32 CUDA tensors of equal size."""
     if out is None:
         out = torch.empty_like(x)
     ctx._rc(lib().dex_voigt(ctx.handle, x.numel(), _ptr(a), _ptr(x), _ptr(out)))

@@ -135,6 +135,8 @@ __device__ __forceinline__ bool all_opaque(const float* T)
 // at I, so every later update, and the boundary term, rounds back to I: the rest
 // of the ray cannot change a bit of it.  A ray is done when this holds for all of
 // its wavelengths, near tau = 18 where exact underflow of T takes 87 to 104.
+// Wavelengths that pad a batch up to W have S = chi = 0 and keep T = 1: rays of such a
+// batch, and of the one sharing its walk, end at the edge only.
 // stop = B 2^26, or negative where no bound is known (then T = 0 everywhere).
 __device__ __forceinline__ float stop_factor(float bound, float i_bc)
 {

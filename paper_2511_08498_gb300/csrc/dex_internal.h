@@ -282,7 +282,7 @@ struct BatchParams {
 
 // packet: probes per work item (256, 128 or 64); info: stage one word per block
 // (offset * 8 + state) instead of the packed state words; occupancy (W = 8): a
-// 64-register budget (four 256-thread CTAs per SM) instead of the compiler's;
+// 64-register budget (four 256-thread CTAs per SM) instead of 80 (three);
 // max_words, max_blocks: of the batch's largest grid
 cudaError_t launch_batch_solve(cudaStream_t s, const BatchParams& P, int ctas, int W, int packet, bool info,
                                bool occupancy, size_t max_words, size_t max_blocks);

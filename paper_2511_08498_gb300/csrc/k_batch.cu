@@ -52,9 +52,10 @@ struct StaticRec {
     }
 };
 
-// kMinCtas: CTAs per SM the register budget is sized for (1: the compiler's
-// choice, 97 registers at W = 8; 1024 / NT: 64 registers, four 256-thread CTAs
-// of residency, with some spilling).
+// kMinCtas: CTAs per SM the register budget is sized for (768 / NT: 80 registers, three
+// 256-thread CTAs of residency, at W = 8 with up to 48 bytes spilled, 150 where shared
+// walks are looked for; 1024 / NT: 64 registers, four, 120 and 230 bytes; pairs 512 / NT:
+// 128 registers, two).
 // NT threads per CTA = probes per work item (a 16 x (NT / 16) part of a block,
 // warps on 8 x 4 tiles as in k_solve_hdda_t); a CTA claims `chunk` consecutive
 // items per queue increment.  kInfo: the block table is staged as one word per
