@@ -56,6 +56,18 @@ def run_config(ctx, items, W, cfg, queue=None, **kw):
         ctx.set_traversal(api.TRAVERSAL_PER_BATCH)
 
 
+def default_config(items, W, sms, walk="per_batch"):
+    """The launch that ``dex_batch_solve`` makes of ``items`` when the grid is left to it."""
+    packets = 0
+    for it in items:
+        n = -(-it.n_lambda // W)
+        packets += it.capacity * (n if walk == "per_batch" else -(-n // 2))  # pairs and a lone batch
+    small = packets < 6 * sms
+    staging = int(all((it.nx // 16) * (it.nz // 16) <= 8192 for it in items))
+    return dict(ctas=(6 if small else 3) * sms, packet=128 if small else 256, chunk=1, staging=staging, occupancy=0,
+                walk=walk)
+
+
 def tune_batch(ctx, items, W, reps=3, rounds=2):
     """Coordinate descent over the launch knobs of ``dex_batch_solve_config`` --
     persistent grid size, probes per work item (packet), work items per queue
@@ -65,7 +77,7 @@ def tune_batch(ctx, items, W, reps=3, rounds=2):
     Returns ``{"best", "best_ms", "default", "default_ms", "trials"}``."""
     sms = torch.cuda.get_device_properties(ctx.device).multi_processor_count
     queue = torch.zeros(1, dtype=torch.int32, device=torch.device("cuda", ctx.device))
-    default = dict(ctas=3 * sms, packet=256, chunk=1, staging=0, occupancy=0, walk="per_batch")
+    default = default_config(items, W, sms)
     space = [("walk", ["per_batch", "paired"] if W == 8 else ["per_batch"]),
              ("ctas", [k * sms for k in (1, 2, 3, 4, 6, 8)]), ("packet", [256, 128, 64]), ("chunk", [1, 2, 4, 8, 16]),
              ("staging", [0, 1]), ("occupancy", [0, 1] if W == 8 else [0])]
