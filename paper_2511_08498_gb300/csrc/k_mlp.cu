@@ -568,10 +568,16 @@ cudaError_t launch_mlp_forward(cudaStream_t s, const MlpParams& P)
                                  cudaSharedmemCarveoutMaxShared);
     if (e != cudaSuccess) return e;
     const long long tiles = (P.n + kTile - 1) / kTile;
-    // up to eight tiles per CTA: one CTA per slot for all of them left the younger CTAs
-    // of an SM behind (248 us for 2^22 samples against 221; four 228, sixteen 231)
-    const long long per = max(1LL, min(8LL, tiles / (8LL * sms)));
-    const long long grid = (tiles + per - 1) / per;
+    // Setting up a CTA (weights, tensor memory) costs about as much as two tiles, so small
+    // numbers of tiles go to as few CTAs per SM as get 2.3 tiles each, from two to the
+    // eight that fit: 311000 samples 38.6 us with one tile per CTA, 27.2 with six CTAs per
+    // SM; 117000 19.1, 17.0 with three; 78000 15.9, 13.9 with two.  From sixteen tiles per
+    // slot on CTAs of eight tiles each: one CTA per slot for all of them left the younger
+    // CTAs of an SM behind (2^22 samples 225 us against 216), while 1.5 million samples
+    // take 87.7 us with one per slot, 89.6 with CTAs of eight tiles.
+    const long long slots = 8LL * sms;
+    const long long k = llround((double)tiles / (2.3 * sms));
+    const long long grid = tiles >= 16 * slots ? (tiles + 7) / 8 : min(tiles, max(2LL, min(8LL, k)) * sms);
     k_mlp_forward<<<(unsigned)grid, 128, kSmemInfer, s>>>(P);
     return cudaGetLastError();
 }
