@@ -53,6 +53,13 @@ constexpr int kPairInfoMaxBlocks = 16384;
 // 160, 21 wavelengths, paired (270): 0.85 -> 0.33 ms; but 784 x 288, 29 wavelengths
 // (3528): 5.07 -> 5.52 ms, and the 1024^2 paired solve 101 -> 115 ms.
 constexpr long long kSplitCtas = 1216;
+// That counts the grid's blocks, of which the host does not know how many are empty.  One
+// walk per batch on grids of up to kSplitSparseCtas is launched both ways, and the device
+// runs the split one below kSplitActiveCtas active (block, batch) pairs, one and a half
+// loads; the other launch ends at once (480 x 320, 32 wavelengths, 70% empty, 720 of 2400:
+// 2.06 -> 1.66 ms; 272 x 304, 31, 1163 of 1292: 5.00, split 4.73; 640 x 480, 16, 1440 of
+// 2400: 5.12, split 6.04).
+constexpr long long kSplitSparseCtas = 3648, kSplitActiveCtas = 912;
 
 // Distance thresholds of levels 1..4 padded to four, as the traversal compares
 // them (the number of thresholds band[m-1] <= t is the highest level allowed):
@@ -131,8 +138,11 @@ struct HddaParams {
     int exclude_own; // leave out each probe's own-voxel emission (static model, W = 8, float32)
     int scanned;     // J holds the bounds of the exact early termination (scan.cuh)
     int split_at;    // float offset of the split kernels' intensities in dynamic shared memory
-    int twins;       // one walk per batch: pairs of batches whose blocks all have the same levels
-                     // are walked once (states_agree; k_solve_hdda_pair, then the others alone)
+    int twins;       // one walk per batch: from this many active blocks on (0: never) pairs of
+                     // batches whose blocks all have the same levels are walked once
+                     // (states_agree; k_solve_hdda_pair, then the others alone)
+    int active_from, active_to;  // k_solve_hdda_t does nothing with fewer active blocks, or with
+                                 // active_to (unless 0) or more
     float band[4];
     long long n_cells;
     const float* bricks;
@@ -333,7 +343,7 @@ cudaError_t launch_solve_hdda_shared(cudaStream_t s, const HddaParams& p);
 bool solve_hdda_paired_applies(const HddaParams& p);
 cudaError_t launch_solve_hdda_paired(cudaStream_t s, const HddaParams& p);
 // the pairs of batches whose levels agree, for the per-batch walk (p.twins)
-cudaError_t launch_solve_hdda_twins(cudaStream_t s, const HddaParams& p);
+cudaError_t launch_solve_hdda_twins(cudaStream_t s, const HddaParams& p, bool split);
 
 // --------------------------------------------------- radiance cascades --
 struct RcParams {

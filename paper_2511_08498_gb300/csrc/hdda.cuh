@@ -428,13 +428,14 @@ __global__ void __launch_bounds__(256, Model::kMinBlocks) k_solve_hdda_t(const H
     extern __shared__ unsigned long long s_dyn[];
     __shared__ float s_J[SPLIT ? 1 : W][256];
     const int a0 = SPLIT ? blockIdx.x >> 3 : blockIdx.x;
-    if (a0 >= *P.n_active) return;
+    const int n_active = *P.n_active;
+    if (a0 >= n_active || n_active < P.active_from || (P.active_to && n_active >= P.active_to)) return;
     const int b = blockIdx.y;
     const int tid = threadIdx.x;
     const unsigned long long* words_b = P.words + (size_t)b * P.n_words;
     if constexpr (TwinsOf<Model>::value && W == 8 && !COUNT && !EXT) {
         // walked with its partner (k_solve_hdda_pair) if their levels agree
-        if (P.twins) {
+        if (P.twins && n_active >= P.twins) {
             const int b2 = pair_partner(b, P.n_batch, P.pair_group);
             if (b2 != b && states_agree(words_b, P.words + (size_t)b2 * P.n_words, P.n_words)) return;
         }

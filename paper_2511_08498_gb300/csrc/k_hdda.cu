@@ -95,25 +95,76 @@ static void scan_bricks(cudaStream_t s, HddaParams& P)
     P.scanned = 1;
 }
 
-// Whether the per-batch solve looks for pairs of batches that it may walk once (twins):
+// Where the per-batch solve looks for pairs of batches that it may walk once (twins):
 // W = 8 and a grid that the pair kernel's table covers.  The pairs and the other batches
 // are two launches, so where some batch is certain to be left for the second (the middle
 // one of an odd number) the first must fill the chip: two rounds of the pair kernel's 304
-// resident CTAs, five where directions are split.  Static lines, 32 directions, one walk
-// per batch -> with pairs:
+// resident CTAs, five where directions are split; with an even number, of which some pairs
+// may differ, one and a half (256 x 320, 31 wavelengths, 60% empty, 256 blocks of pairs:
+// 2.90 ms instead of 2.24), and always where split.  That is counted in active blocks, which
+// the device knows (HddaParams::twins: from how many on; 0 never): by the grid's blocks,
+// 384 x 400 cells, 40 wavelengths, 60% of them empty, took 4.73 ms instead of 3.76.
+// Static lines, 32 directions, 40% empty, one walk per batch -> with pairs:
 //   768^2, 32 wavelengths  35.2 -> 28.7 ms    256^2, 32 (split)  3.38 -> 2.98 ms
 //   512^2, 16              14.5 -> 11.8       96^2, 16 (split)   0.284 -> 0.250
 //   512^2, 24              15.4 -> 14.2       384^2, 24          7.80 -> 9.00 (not taken)
 //   320^2, 24 (split)      4.12 -> 3.79       160^2, 24 (split)  0.741 -> 0.782 (not taken)
-// bfloat16 pairs run 128-thread CTAs and gain nothing when split (160^2, 32: 1.04 ->
-// 1.15).  Where the levels differ the check costs 0.3% (768^2, 20: 36.6 both ways).
-static bool twins_apply(const HddaParams& P, bool split)
+// bfloat16 pairs run 128-thread CTAs, 760 resident, and gain nothing when split (160^2,
+// 32: 1.04 -> 1.15) or below two rounds (400 x 336, 32, 578 blocks of pairs: 4.76 -> 5.14).
+// Where the levels differ the check costs 0.3% (768^2, 20: 36.6 both ways).
+static int twins_from(const HddaParams& P, bool split)
 {
-    if (P.W != 8 || P.seg_count || !P.scanned || (long long)P.nbx * P.nbz > kPairInfoMaxBlocks) return false;
-    if (split && P.storage == kStoreBF16) return false;
+    if (P.W != 8 || P.seg_count || !P.scanned || (long long)P.nbx * P.nbz > kPairInfoMaxBlocks) return 0;
+    if (split && P.storage == kStoreBF16) return 0;
     const int pairs = pair_count(P.n_batch, P.pair_group);
-    if (pair_lone_count(P.n_batch, P.pair_group) == 0) return pairs > 0;
-    return (long long)P.cap_active * pairs * (split ? 8 : 1) >= (split ? 1520 : 608);
+    if (pairs == 0) return 0;
+    const bool even = pair_lone_count(P.n_batch, P.pair_group) == 0;
+    const int unsplit = P.storage == kStoreBF16 ? 760 : even ? 456 : 608;
+    const int ctas = split ? (even ? 1 : 190) : unsplit;
+    const int from = max((ctas + pairs - 1) / pairs, P.active_from);
+    return (P.active_to ? min(P.active_to - 1, P.cap_active) : P.cap_active) >= from ? from : 0;
+}
+
+// One walk per batch, directions split or not.
+static cudaError_t launch_per_batch(cudaStream_t s, HddaParams P, bool info, bool split)
+{
+    const size_t smem = sizeof(float) * ((size_t)P.split_at + (split ? (size_t)split_chunk<8>() * P.W * 32 : 0));
+    const int blocks = P.active_to ? min(P.active_to, P.cap_active) : P.cap_active;
+    const dim3 grid((unsigned)blocks * (split ? 8u : 1u), (unsigned)P.n_batch);
+    cudaError_t e = cudaSuccess;
+    P.twins = twins_from(P, split);
+    if (P.twins && (e = launch_solve_hdda_twins(s, P, split)) != cudaSuccess) return e;
+    switch (P.W * 4 + P.storage) {
+#define DEX_LAUNCH_(WW, ST, INFO)                                                                                     \
+    {                                                                                                                 \
+        using M_ = StaticModel<WW, ST>;                                                                               \
+        if (P.seg_count) e = launch_hdda_kernel(k_solve_hdda_t<WW, true, M_, INFO>, grid, smem, s, P, M_::Params{});  \
+        else if (split)                                                                                               \
+            e = launch_hdda_kernel(k_solve_hdda_t<WW, false, M_, INFO, false, true>, grid, smem, s, P, M_::Params{}); \
+        else e = launch_hdda_kernel(k_solve_hdda_t<WW, false, M_, INFO>, grid, smem, s, P, M_::Params{});             \
+    }
+#define DEX_LAUNCH(WW, ST) \
+    case WW * 4 + ST: DEX_LAUNCH_(WW, ST, false) break;
+#define DEX_LAUNCH_INFO(ST)                  \
+    case 8 * 4 + ST:                         \
+        if (info) DEX_LAUNCH_(8, ST, true)   \
+        else DEX_LAUNCH_(8, ST, false)       \
+        break;
+        DEX_LAUNCH(1, kStoreF32)
+        DEX_LAUNCH(2, kStoreF32)
+        DEX_LAUNCH(4, kStoreF32)
+        DEX_LAUNCH_INFO(kStoreF32)
+        DEX_LAUNCH(4, kStoreBF16)
+        DEX_LAUNCH_INFO(kStoreBF16)
+        DEX_LAUNCH(4, kStoreF16)
+        DEX_LAUNCH_INFO(kStoreF16)
+#undef DEX_LAUNCH_INFO
+#undef DEX_LAUNCH
+#undef DEX_LAUNCH_
+        default: return cudaErrorInvalidValue;
+    }
+    if (e != cudaSuccess) return e;
+    return cudaGetLastError();
 }
 
 cudaError_t launch_solve_hdda(cudaStream_t s, const HddaParams& P0)
@@ -148,42 +199,14 @@ cudaError_t launch_solve_hdda(cudaStream_t s, const HddaParams& P0)
     const bool info = P.W == 8 && n_blocks <= kInfoMaxBlocks;
     P.split_at = (int)(((info ? n_blocks : 2LL * P.n_words) + 3) & ~3LL);
     const bool split = split_directions(P);
-    const size_t smem = sizeof(float) * ((size_t)P.split_at + (split ? (size_t)split_chunk<8>() * P.W * 32 : 0));
-    const dim3 grid((unsigned)P.cap_active * (split ? 8u : 1u), (unsigned)P.n_batch);
-    cudaError_t e = cudaSuccess;
-    P.twins = twins_apply(P, split);
-    if (P.twins && (e = launch_solve_hdda_twins(s, P)) != cudaSuccess) return e;
-    switch (P.W * 4 + P.storage) {
-#define DEX_LAUNCH_(WW, ST, INFO)                                                                                     \
-    {                                                                                                                 \
-        using M_ = StaticModel<WW, ST>;                                                                               \
-        if (P.seg_count) e = launch_hdda_kernel(k_solve_hdda_t<WW, true, M_, INFO>, grid, smem, s, P, M_::Params{});  \
-        else if (split)                                                                                               \
-            e = launch_hdda_kernel(k_solve_hdda_t<WW, false, M_, INFO, false, true>, grid, smem, s, P, M_::Params{}); \
-        else e = launch_hdda_kernel(k_solve_hdda_t<WW, false, M_, INFO>, grid, smem, s, P, M_::Params{});             \
+    const long long ctas = (long long)P.cap_active * P.n_batch;
+    if (!split && !P.seg_count && ctas < kSplitSparseCtas && P.split_at <= 24576) {
+        HddaParams Q = P;
+        P.active_from = Q.active_to = (int)((kSplitActiveCtas + P.n_batch - 1) / P.n_batch);
+        const cudaError_t e = launch_per_batch(s, Q, info, true);
+        if (e != cudaSuccess) return e;
     }
-#define DEX_LAUNCH(WW, ST) \
-    case WW * 4 + ST: DEX_LAUNCH_(WW, ST, false) break;
-#define DEX_LAUNCH_INFO(ST)                  \
-    case 8 * 4 + ST:                         \
-        if (info) DEX_LAUNCH_(8, ST, true)   \
-        else DEX_LAUNCH_(8, ST, false)       \
-        break;
-        DEX_LAUNCH(1, kStoreF32)
-        DEX_LAUNCH(2, kStoreF32)
-        DEX_LAUNCH(4, kStoreF32)
-        DEX_LAUNCH_INFO(kStoreF32)
-        DEX_LAUNCH(4, kStoreBF16)
-        DEX_LAUNCH_INFO(kStoreBF16)
-        DEX_LAUNCH(4, kStoreF16)
-        DEX_LAUNCH_INFO(kStoreF16)
-#undef DEX_LAUNCH_INFO
-#undef DEX_LAUNCH
-#undef DEX_LAUNCH_
-        default: return cudaErrorInvalidValue;
-    }
-    if (e != cudaSuccess) return e;
-    return cudaGetLastError();
+    return launch_per_batch(s, P, info, split);
 }
 
 }  // namespace dex

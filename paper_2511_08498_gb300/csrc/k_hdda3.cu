@@ -233,9 +233,9 @@ __global__ void __launch_bounds__(kThreads3, NB == 1 ? kMinBlocks3 : 2) k_solve_
     const int tid = threadIdx.x;
     const unsigned long long* gw = P.words + (size_t)b * P.n_words;
     if constexpr (TWIN) {
-        if (!states_agree(gw, P.words + (size_t)b2 * P.n_words, P.n_words)) return;
+        if (*P.n_active < P.twins || !states_agree(gw, P.words + (size_t)b2 * P.n_words, P.n_words)) return;
     } else if constexpr (NB == 1 && W == 8 && INFO && !COUNT) {
-        if (P.twins) {  // walked with its partner if their levels agree
+        if (P.twins && *P.n_active >= P.twins) {  // walked with its partner if their levels agree
             const int other = pair_partner(b, P.n_batch, P.pair_group);
             if (other != b && states_agree(gw, P.words + (size_t)other * P.n_words, P.n_words)) return;
         }
@@ -419,10 +419,12 @@ cudaError_t launch3(K kernel, dim3 grid, size_t smem, cudaStream_t s, const Hdda
 // lines, 16 directions, one walk per batch -> with pairs: 128 x 96 x 80, 32 wavelengths
 // 13.5 -> 11.0 ms, 24 (a lone batch) 9.08 -> 8.09; 48 x 40 x 40, 32 (600 CTAs) 0.882 ->
 // 0.830, 16 (300) 0.524 -> 0.537; 32^3, 32 (256) 0.488 -> 0.518.  Where the levels differ
-// the check costs under 1%.
-static bool twins_apply3(const Hdda3Params& P)
+// the check costs under 1%.  Returns the active blocks from which it does, counted on the
+// device (HddaParams::twins).
+static int twins_from3(const Hdda3Params& P)
 {
-    return (long long)P.cap_active * kParts3 * pair_count(P.n_batch, P.pair_group) >= 456;
+    const long long ctas = (long long)kParts3 * pair_count(P.n_batch, P.pair_group);
+    return (long long)P.cap_active * ctas >= 456 ? (int)((455 + ctas) / ctas) : 0;
 }
 
 bool solve_hdda3_paired_applies(const Hdda3Params& P)
@@ -484,8 +486,8 @@ cudaError_t launch_solve_hdda3(cudaStream_t s, const Hdda3Params& P0)
         return cudaSuccess;
     }
     const dim3 grid((unsigned)P.cap_active * kParts3, (unsigned)P.n_batch);
-    if (info && P.scanned && twins_apply3(P)) {
-        P.twins = 1;
+    if (info && P.scanned) P.twins = twins_from3(P);
+    if (P.twins) {
         const dim3 pairs((unsigned)P.cap_active * kParts3, (unsigned)pair_count(P.n_batch, P.pair_group));
         switch (P.storage) {
             case kStoreF32: e = launch3(k_solve_hdda3<8, false, kStoreF32, 2, true, true>, pairs, smem, s, P); break;

@@ -74,6 +74,7 @@ __global__ void __launch_bounds__(pair_threads<ST>(), pair_min_blocks<ST>()) k_s
     const unsigned long long* w1 = P.words + (size_t)b1 * P.n_words;
     const unsigned long long* w2 = P.words + (size_t)b2 * P.n_words;
     if constexpr (TWIN) {
+        if (*P.n_active < P.twins || (P.active_to && *P.n_active >= P.active_to)) return;
         if (!states_agree(w1, w2, P.n_words)) return;
     }
     const int n_blocks = P.nbx * P.nbz;
@@ -230,14 +231,15 @@ __global__ void __launch_bounds__(pair_threads<ST>(), pair_min_blocks<ST>()) k_s
 }
 
 template <int ST>
-cudaError_t launch_pair(cudaStream_t s, const HddaParams& P0, bool twin = false)
+cudaError_t launch_pair(cudaStream_t s, const HddaParams& P0, bool twin = false, bool twin_split = false)
 {
     HddaParams P = P0;
     const unsigned pairs = (unsigned)pair_count(P.n_batch, P.pair_group);
     P.split_at = (P.nbx * P.nbz + 3) & ~3;
-    const bool split = split_directions(P);
+    const bool split = twin ? twin_split : split_directions(P);
+    const int blocks = P.active_to ? min(P.active_to, P.cap_active) : P.cap_active;
     const size_t smem = sizeof(int) * (size_t)P.split_at + (split ? split_bytes<16>() : 0);
-    const dim3 grid((unsigned)P.cap_active * (split ? 8u : (unsigned)pair_parts<ST>()), pairs);
+    const dim3 grid((unsigned)blocks * (split ? 8u : (unsigned)pair_parts<ST>()), pairs);
     auto kernel = P.seg_count ? (P.exclude_own ? k_solve_hdda_pair<ST, true, true, false>
                                                : k_solve_hdda_pair<ST, true, false, false>)
                   : twin      ? (split ? k_solve_hdda_pair<ST, false, false, true, true>
@@ -263,12 +265,12 @@ bool solve_hdda_paired_applies(const HddaParams& P)
            (!P.exclude_own || P.storage == kStoreF32);
 }
 
-cudaError_t launch_solve_hdda_twins(cudaStream_t s, const HddaParams& P)
+cudaError_t launch_solve_hdda_twins(cudaStream_t s, const HddaParams& P, bool split)
 {
     switch (P.storage) {
-        case kStoreF32: return launch_pair<kStoreF32>(s, P, true);
-        case kStoreBF16: return launch_pair<kStoreBF16>(s, P, true);
-        case kStoreF16: return launch_pair<kStoreF16>(s, P, true);
+        case kStoreF32: return launch_pair<kStoreF32>(s, P, true, split);
+        case kStoreBF16: return launch_pair<kStoreBF16>(s, P, true, split);
+        case kStoreF16: return launch_pair<kStoreF16>(s, P, true, split);
         default: return cudaErrorInvalidValue;
     }
 }
