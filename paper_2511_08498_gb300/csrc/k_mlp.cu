@@ -540,9 +540,8 @@ __global__ void k_mlp_targets(long long n, const float* __restrict__ xau, float*
 {
     stage_dawson(C);
     __syncthreads();
-    const long long s = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (s >= n) return;
-    out[s] = logf(voigt_h(C, xau[3 * s + 1], xau[3 * s] - xau[3 * s + 2]));
+    for (long long s = blockIdx.x * (long long)blockDim.x + threadIdx.x; s < n; s += (long long)gridDim.x * blockDim.x)
+        out[s] = logf(voigt_h<false>(C, xau[3 * s + 1], xau[3 * s] - xau[3 * s + 2]));
 }
 
 }  // namespace
@@ -610,7 +609,8 @@ cudaError_t launch_mlp_adam(cudaStream_t s, float* p, const float* g, float* m, 
 cudaError_t launch_mlp_targets(cudaStream_t s, long long n, const float* xau, float* out)
 {
     if (n == 0) return cudaSuccess;
-    k_mlp_targets<<<(unsigned)((n + 255) / 256), 256, 0, s>>>(n, xau, out, voigt_coefficients());
+    const long long ctas = (n + 255) / 256;
+    k_mlp_targets<<<(unsigned)(ctas < 152 * 8 ? ctas : 152 * 8), 256, 0, s>>>(n, xau, out, voigt_coefficients());
     return cudaGetLastError();
 }
 
