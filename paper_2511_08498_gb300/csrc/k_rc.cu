@@ -338,7 +338,7 @@ __global__ void __launch_bounds__(kRcThreads, (NB == 1 ? 1024 : 512) / kRcThread
         }
     }
     if (capped) raise_status(P.status, DEX_ERR_TRAVERSAL_CAP);
-    if (COUNT && P.seg_count != nullptr) atomicAdd(P.seg_count, (unsigned long long)nseg);
+    if (COUNT && nseg && P.seg_count != nullptr) atomicAdd(P.seg_count, (unsigned long long)nseg);
 }
 
 // J at every cell of every non-empty block: the mean of the cascade-0 radiance
