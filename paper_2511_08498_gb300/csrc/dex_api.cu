@@ -1536,9 +1536,12 @@ int dex_rc_solve(dex_ctx* ctx, int nx, int nz, int n_lambda, int W, int max_mip,
     cudaError_t e = cudaMemsetAsync(J, 0, sizeof(float) * (size_t)n_lambda * n_cells, ctx->stream);
     // tables in the half of the workspace that cascade 0 does not use, beyond the quarter
     // of it that an upper cascade fills; counting solves run rays to exactly zero
-    // transmission, so they take no bounds
+    // transmission, so they take no bounds, and neither do few cascades, whose intervals
+    // are too short for rays to end in, or one or two wavelengths, whose bricks cost most
+    // to read (128^2, three cascades, W = 4: 144 us with bounds)
     if (e == cudaSuccess)
-        e = dex::launch_rc_tables(ctx->stream, P, workspace + (n_cascades % 2 == 1 ? half : 0) + half / 2, !seg_count);
+        e = dex::launch_rc_tables(ctx->stream, P, workspace + (n_cascades % 2 == 1 ? half : 0) + half / 2,
+                                  !seg_count && W >= 4 && n_cascades >= 4);
     // direction offsets: cascade i starts at n0 (4^i - 1) / 3
     const float* upper = nullptr;
     float* out = nullptr;
