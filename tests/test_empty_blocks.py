@@ -47,6 +47,21 @@ def test_bits(nx, nz, L, rows, storage):
     ctx.check()
 
 
+@pytest.mark.parametrize("W,L,storage", [(1, 2, 0), (2, 4, 0), (4, 8, 0), (4, 8, 1), (4, 7, 2)])
+@pytest.mark.parametrize("rows", [10, 14, 15])
+def test_bits_of_narrow_batches(W, L, storage, rows):
+    """Two batches of 1024 blocks, 640, 896 and 960 active pairs."""
+    from paper_2511_08498_gb300 import api
+    ctx = api.Context(0)
+    eta, chi = medium(512, 512, L, rows, 1050 + W, False)
+    grid = api.grid_build(ctx, 512, 512, eta, chi)
+    mips = api.mips_build(ctx, grid, eta, chi, W, 3, 1e-2, 1e-2, storage=storage)
+    dirs, w = synth.directions(5, offset=0.0)
+    full = api.formal_solve_hdda(ctx, grid, mips, dirs, w, band=BAND, i_bc=0.2, count_segments=True)
+    assert torch.equal(full[0], api.formal_solve_hdda(ctx, grid, mips, dirs, w, band=BAND, i_bc=0.2)[0])
+    ctx.check()
+
+
 def best_ms(f):
     best = float("inf")
     for _ in range(8):
