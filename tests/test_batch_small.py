@@ -1,4 +1,4 @@
-"""Batched solves of a few small atmospheres: the default launch is the one for small batches."""
+"""Batched solves of a few small atmospheres (packets of 128 probes) and of more: one by one the same bits."""
 
 import numpy as np
 import pytest
@@ -28,18 +28,6 @@ def batch(api, ctx, W, n_dir, sizes):
     return items, keep
 
 
-def best_ms(f):
-    best = float("inf")
-    for _ in range(8):
-        a, b = (torch.cuda.Event(enable_timing=True) for _ in range(2))
-        a.record()
-        f()
-        b.record()
-        b.synchronize()
-        best = min(best, a.elapsed_time(b))
-    return best
-
-
 # below and above two packets for each of the 456 default CTAs
 @pytest.mark.parametrize("walk", ["per_batch", "paired"])
 @pytest.mark.parametrize("W,sizes", [(8, ((128, 128, 32), (192, 128, 24), (128, 192, 17))), (8, ((384, 320, 32), (128, 64, 9))),
@@ -62,18 +50,3 @@ def test_same_as_one_by_one(walk, W, sizes):
             ref, _, _ = api.formal_solve_hdda(ctx, grid, mips, dirs, w, band=BAND, i_bc=0.2)
             assert torch.equal(J, ref)
     ctx.check()
-
-
-@pytest.mark.parametrize("walk", ["per_batch", "paired"])
-def test_small_packets_are_the_default(walk):
-    """Three uneven atmospheres of 128 to 192 cells a side: packets of 128 probes are a tenth faster."""
-    from paper_2511_08498_gb300 import api
-    from perf import cases
-    s = cases.prepare(dict(kind="batch", n_atm=3, low=128, high=192, walk=walk), 16)
-    ctx, items, queue = s["ctx"], s["items"], s["queue"]
-    sms = torch.cuda.get_device_properties(0).multi_processor_count
-    small = best_ms(lambda: api.batch_solve_config(ctx, items, 8, ctas=6 * sms, packet=128, staging=1, queue=queue))
-    large = best_ms(lambda: api.batch_solve_config(ctx, items, 8, ctas=3 * sms, packet=256, staging=1, queue=queue))
-    default = best_ms(lambda: api.batch_solve(ctx, items, 8, queue=queue))
-    ctx.check()
-    assert default < 1.03 * min(small, large), (default, small, large)

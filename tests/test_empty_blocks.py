@@ -64,7 +64,7 @@ def test_bits_of_narrow_batches(W, L, storage, rows):
 
 def best_ms(f):
     best = float("inf")
-    for _ in range(8):
+    for _ in range(30):
         a, b = (torch.cuda.Event(enable_timing=True) for _ in range(2))
         a.record()
         f()
